@@ -103,7 +103,8 @@ typedef struct {
                                  2: FP64; 3: every body in double-float; 0: never (FP32 only).
                                  Other values: PABD_ERR_ARG. */
     int sweep_mode;           /* 1: a bond launch + a solve launch per sweep; 2: one launch per
-                                 sweep (the solve evaluates its bonds); 3: one cooperative launch
+                                 sweep (the solve evaluates its bonds), or one for all sweeps
+                                 where every group fits a thread-block cluster; 3: one cooperative launch
                                  runs all n_iter sweeps; 0: the library's choice -- an autotuner
                                  times modes 1 and 2, each with the light bodies ordered by end
                                  count or not, on the state at creation (pabd_tune repeats it on
@@ -196,8 +197,9 @@ typedef struct {
     int64_t tuned;            /* 1 if sweep_mode and light_order were chosen by timing (sweep_mode
                                  0 in the descriptor, no resid_tol, no AL_DISTANCE bonds) */
     int64_t tune_sweep_ns[4]; /* the autotuner's time per sweep for each candidate (the fastest of
-                                 four timed passes over n_iter sweeps), nanoseconds: one
-                                 launch per sweep ordered / in body order, a bond and a solve
+                                 up to four timed passes over n_iter sweeps and of its
+                                 thread counts per body), nanoseconds: one launch per sweep
+                                 ordered (or one for all sweeps over clusters) / in body order, a bond and a solve
                                  launch per sweep ordered / in body order (0: not tuned) */
 } pabd_info;
 

@@ -56,7 +56,6 @@ __global__ void __launch_bounds__(HEAVY_T, 4) k_sweep_fused(Dev d) {
     const int lane = threadIdx.x & (L - 1);
     const int grp = tid / L;
     const int ngrp = (gridDim.x * blockDim.x) / L;
-    const unsigned mask = lane_mask<L>();
     const int nheavy = d.ctr[C_NHEAVY];
     const unsigned limit = *d.wait_limit;
     for (int it = 0; it < d.p.n_iter; ++it) {
@@ -66,17 +65,14 @@ __global__ void __launch_bounds__(HEAVY_T, 4) k_sweep_fused(Dev d) {
         // bodies with many ends first: the first HEAVY_BLOCKS blocks take the heavy role (the
         // launch uses HEAVY_T threads per block and at least HEAVY_BLOCKS blocks)
         if ((int)blockIdx.x < HEAVY_BLOCKS && nheavy > 0)
-            heavy_role<X>(d, blockIdx.x, qi, qo, last,
-                [&](int b, auto& s, const float* c, const float* A, const float* xs, int e0, int e1, int ln) {
-                    gather_ends<32>(d, qi, b, c, A, xs, e0, e1, ln, it, s);
-                },
-                [&](int b, auto& s, const float* c, const float* A, const float* xs, int e0, int e1, int t) {
-                    gather_ends<HEAVY_T>(d, qi, b, c, A, xs, e0, e1, t, it, s);
-                });
-        for (int b = grp; b < d.N; b += ngrp)
-            solve_body<L, X>(d, b, lane, mask, qi, qo, last, [&](auto& s, const float* c, const float* A, const float* xs, int e0, int e1) {
-                gather_ends<L>(d, qi, b, c, A, xs, e0, e1, lane, it, s);
-            });
+            heavy_role<X>(d, blockIdx.x, qi, qo, last, end_gather(d, GlobalQ{qi}, it));
+        for (int g0 = grp - (threadIdx.x & 31) / L; g0 < d.N; g0 += ngrp) {  // (the warp's first body)
+            const int b = g0 + (threadIdx.x & 31) / L;
+            const unsigned team = __ballot_sync(0xffffffffu, b < d.N);
+            if (b < d.N)
+                solve_body<L, L, X>(d, b, lane, team, qi, qo, last, end_gather(d, GlobalQ{qi}, it));
+            __syncwarp();
+        }
         if (it + 1 < d.p.n_iter && !grid_sync(d.gbar, &d.ctr[C_STATUS], limit)) return;
     }
 }
@@ -86,11 +82,8 @@ __global__ void k_end_records(Dev d) {
     pdl_enter();
     const int ne = d.end_off[d.N];
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < ne; p += gridDim.x * blockDim.x) {
-        const int bond = d.end_id[p] >> 1;
-        const int4 m = d.bmeta[bond];
-        d.rec_m[p] = make_int4(m.x, m.y, m.z, bond);
-        d.rec_a[p] = d.bxi[bond];
-        d.rec_b[p] = d.bxj[bond];
+        const int id = d.end_id[p], bond = id >> 1;
+        pack_end(d.rec + 3 * (size_t)p, bond, d.bmeta[bond], d.bxi[bond], d.bxj[bond], d.bn[bond], id & 1);
     }
 }
 

@@ -5,7 +5,8 @@
 //            ends' records (w, f'), w = h^2 phi+(d)/d and f' = f - w y_self, the right-hand
 //            side term of Eq. 19 minus H's own-body term (the "delta" form) -- equal and
 //            opposite f' on the two ends; each record is stored at the end's CSR slot.
-//   k_solve  L lanes per body (the warp-cooperative gather): each lane adds its share of
+//   k_solve  L lanes per body, a thread each or a thread per two (the warp-cooperative
+//            gather): each lane adds its share of
 //            the body's CSR slice and a fixed shuffle tree combines them; it forms, by the Kronecker
 //            structure of H (Eq. 20, 23-24: H = P (G (x) I3) P^T with G the 4x4
 //            diag(m, Pi) + sum w [1;x][1;x]^T), the 4x3 system G dX = M(s - q^k) + sum
@@ -17,7 +18,7 @@
 //            flagged, or a Cholesky pivot below 1e-3 of its diagonal): those sum the same
 //            single-precision records and factor in an extended type -- double-float on
 //            the FP32 pipes (precision policy 1), or FP64 (policy 2).
-#include "sweep_math.cuh"
+#include "sweep_shape.h"
 
 namespace pabd {
 
@@ -49,11 +50,16 @@ __device__ __forceinline__ void bond_one(const Dev& d, const float4* __restrict_
                                          const BondStatic& s) {
     float c[3], A[9];
     ld_q(q, s.m.x, c, A);
-    const int4 mm = make_int4(s.m.x, s.m.y, s.m.z, b);
+    float co[3], Ao[9];
+    ld_other(q, s.m.y, s.xj, co, Ao);
+    EndBond e;
+    e.xs = s.xi; e.xo = s.xj;
+    e.nm = (s.m.z == K_CONTACT || s.m.z == K_GROUND) ? d.bn[b] : make_float4(0.f, 0.f, 0.f, 0.f);
+    e.type = s.m.z; e.other = s.m.y; e.side_j = false; e.bond = b;
     // a bond between two fixed ends is advanced by the final update alone (as in the sweep kernels)
     const bool writer = !(s.fi & BF_PINNED) || !(s.fj & BF_PINNED);
     float f[3];
-    const float w = end_force(d, q, s.m.x, c, A, mm, s.xi, s.xj, it, writer, f);
+    const float w = end_force(d, e, co, Ao, c, A, it, writer, f);
     if (s.p0 >= 0) d.ends[s.p0] = make_float4(w, f[0], f[1], f[2]);
     if (s.p1 >= 0) d.ends[s.p1] = make_float4(w, -f[0], -f[1], -f[2]);
 }
@@ -75,51 +81,62 @@ __global__ void __launch_bounds__(BOND_T) k_bond(Dev d, const float4* __restrict
     for (int b = b0 + gridDim.x * blockDim.x; b < nb; b += gridDim.x * blockDim.x) bond_one(d, q, it, b, bond_static(d, b));
 }
 
-// add the records of ends p0, p0 + stride, ... < e1 in that order, each loaded one round
-// ahead of its sum (the loads of the next end overlap the arithmetic of this one)
-template <class T>
-__device__ __forceinline__ void add_records(const Dev& d, Sys<T>& s, int p0, int e1, int stride, const float* xs) {
-    if (p0 >= e1) return;
-    float4 e = d.ends[p0], x = d.end_x[p0];
-    for (int p = p0; p < e1; p += stride) {
-        const float4 ec = e, xc = x;
-        if (p + stride < e1) {
-            e = d.ends[p + stride];
-            x = d.end_x[p + stride];
-        }
-        sys_add(s, ec, xc, xs);
-    }
-}
+// Sums a body's ends from the bond kernel's records, each loaded one round ahead of its sum (the
+// loads of the next end overlap the arithmetic of this one).
+struct RecordGather {
+    const Dev& d;
 
-// One body per group of L lanes; lane l adds the bond kernel's records of the body's ends
-// l, l + L, ... -- in FP32, or in the extended type for a body on the extended path (the same
-// records and order as the one-launch sweep, so the two modes agree bit for bit).  The first
-// HEAVY_BLOCKS blocks take the heavy bodies (more than HEAVY_ENDS ends), a block each, and are
-// dispatched first; the blocks after them stay resident and take the light bodies.
-template <int L, class X>
+    template <class T>
+    __device__ __forceinline__ void one(Sys<T>& s, const float*, const float*, const float* xs, int p, int e1, int L) const {
+        if (p >= e1) return;
+        float4 e = d.ends[p], x = d.end_x[p];
+        for (; p < e1; p += L) {
+            const float4 ec = e, xc = x;
+            if (p + L < e1) {
+                e = d.ends[p + L];
+                x = d.end_x[p + L];
+            }
+            sys_add(s, ec, xc, xs);
+        }
+    }
+    template <class T>
+    __device__ __forceinline__ void two(Sys<T>& s, Sys<T>& t, const float* c, const float* A, const float* xs, int p,
+                                        int e1, int L) const {
+        if (sizeof(T) != 4) {  // (a lane after the other: the second sum starts once the first is complete)
+            one(s, c, A, xs, p, e1, L);
+            one(t, c, A, xs, p + 1, e1, L);
+            return;
+        }
+        for (; p + 1 < e1; p += L) {
+            const float4 e0 = d.ends[p], x0 = d.end_x[p], e1_ = d.ends[p + 1], x1 = d.end_x[p + 1];
+            sys_add(s, e0, x0, xs);
+            sys_add(t, e1_, x1, xs);
+        }
+        if (p < e1) sys_add(s, d.ends[p], d.end_x[p], xs);
+    }
+};
+
+// One body per P threads, which sum its L logical lanes (sys_sum_lanes); lane l adds the bond
+// kernel's records of the body's ends l, l + L, ... -- in FP32, or in the extended type for a
+// body on the extended path (the same records and order as the one-launch sweep, so the two
+// modes agree bit for bit).  The first HEAVY_BLOCKS blocks take the heavy bodies (more than
+// HEAVY_ENDS ends), and are dispatched first; the blocks after them stay resident and take the
+// light bodies.
+template <int L, int P, class X>
 __global__ void __launch_bounds__(SOLVE_T, 4) k_solve(Dev d, const float4* __restrict__ qi, float4* __restrict__ qo,
                                                    int it) {
     pdl_enter();
     const int last = it == d.p.n_iter - 1;
     if ((int)blockIdx.x < HEAVY_BLOCKS) {
-        heavy_role<X>(d, blockIdx.x, qi, qo, last,
-            [&](int b, auto& s, const float* c, const float* A, const float* xs, int e0, int e1, int ln) {
-                add_records(d, s, e0 + ln, e1, 32, xs);
-            },
-            [&](int b, auto& s, const float* c, const float* A, const float* xs, int e0, int e1, int t) {
-                add_records(d, s, e0 + t, e1, HEAVY_T, xs);
-            });
+        heavy_role<X>(d, blockIdx.x, qi, qo, last, RecordGather{d});
         return;
     }
     // the light bodies in this step's (class, end count) order, or in body order (a body on
     // the heavy list then returns at once); either way the same arithmetic per body
-    const int lane = threadIdx.x & (L - 1);
-    for_light_slots<L>(&d.ctr[C_SOLVE_NEXT], d.light_sorted ? d.ctr[C_NLIGHT] : d.N, HEAVY_BLOCKS, [&](int slot) {
+    const int plane = threadIdx.x & (P - 1);
+    for_light_slots<P>(&d.ctr[C_SOLVE_NEXT], d.light_sorted ? d.ctr[C_NLIGHT] : d.N, HEAVY_BLOCKS, [&](int slot, unsigned team) {
         const int b = d.light_sorted ? d.order[slot] : slot;
-        solve_body<L, X>(d, b, lane, lane_mask<L>(), qi, qo, last,
-                         [&](auto& s, const float* c, const float* A, const float* xs, int e0, int e1) {
-            add_records(d, s, e0 + lane, e1, L, xs);
-        });
+        solve_body<L, P, X>(d, b, plane, team, qi, qo, last, RecordGather{d});
     });
 }
 
@@ -128,35 +145,21 @@ void launch_bond(const Dev& d, const float4* q, int it, cudaStream_t st, long lo
     *launches += 1;
 }
 
-void launch_solve(const Dev& d, const float4* q_in, float4* q_out, int it, int lanes, cudaStream_t st,
+void launch_solve(const Dev& d, const float4* q_in, float4* q_out, int it, int lanes, int threads, cudaStream_t st,
                   long long* launches) {
     static_assert(SOLVE_T == HEAVY_T, "the solve launch's blocks are the heavy bodies' blocks");
     // resident light blocks: as many as fit beside each other (4 per SM by the launch bounds),
     // fewer when the bodies do not need them
     const int slots = resident_slots(4);
-    const long long n = (long long)(d.N > 0 ? d.N : 1) * lanes;
+    const long long n = (long long)(d.N > 0 ? d.N : 1) * threads;
     const long long need = (n + SOLVE_T - 1) / SOLVE_T;
     const int light = (int)(need < slots ? need : slots);
-    const int grid = HEAVY_BLOCKS + light;
-    const bool f64 = d.p.precision_policy == 2;
-    switch (lanes) {
-        case 1: f64 ? launch_pdl(k_solve<1, double>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it)
-                    : launch_pdl(k_solve<1, ca>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it); break;
-        case 2: f64 ? launch_pdl(k_solve<2, double>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it)
-                    : launch_pdl(k_solve<2, ca>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it); break;
-        case 4: f64 ? launch_pdl(k_solve<4, double>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it)
-                    : launch_pdl(k_solve<4, ca>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it); break;
-        case 8: f64 ? launch_pdl(k_solve<8, double>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it)
-                    : launch_pdl(k_solve<8, ca>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it); break;
-        default: f64 ? launch_pdl(k_solve<16, double>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it)
-                     : launch_pdl(k_solve<16, ca>, dim3(grid), dim3(SOLVE_T), 0, st, d, q_in, q_out, it); break;
-    }
+    with_sweep_shape(lanes, threads, d.p.precision_policy == 2, [&](auto l, auto p, auto x) {
+        launch_pdl(k_solve<decltype(l)::value, decltype(p)::value, typename decltype(x)::type>,
+                   dim3(HEAVY_BLOCKS + light), dim3(SOLVE_T), 0, st, d, q_in, q_out, it);
+    });
     *launches += 1;
 }
-
-}  // namespace pabd
-
-namespace pabd {
 
 // augmented Lagrangian warm start at the start of a step (Eq. 29), from the values the
 // previous step ended with (parity n_iter): kappa <- max(gamma kappa, kappa_start),
@@ -179,8 +182,8 @@ __global__ void k_al_final(Dev d, const float4* __restrict__ q) {
     const float4 xi = d.bxi[b], xj = d.bxj[b];
     float ci[3], Ai[9], cj[3], Aj[9], r[3];
     ld_q(q, m.x, ci, Ai);
-    ld_q_or_zero(q, m.y, cj, Aj);
-    bond_vec_dot2(ci, Ai, xi, cj, Aj, xj, m.y < 0, r);
+    ld_other(q, m.y, xj, cj, Aj);
+    bond_vec_dot2(ci, Ai, xi, cj, Aj, xj, false, r);
     const float cc = sqrtf(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) - xj.w;
     const int it = d.p.n_iter;
     const float beta = d.al_par[b].y;

@@ -164,6 +164,9 @@ struct pabd_scene {
     double prof_acc[PABD_PROFILE_SLOTS] = {0};
     // fused sweep launch shape
     int fused = 0, mode = 1, lanes = 8, sw_block = 128, sw_grid = 1;
+    int threads = 8;  // threads per body of the sweep launches (sweep_threads)
+    BinsShape bins;   // mode 2: all sweeps in one launch where in_bins (choose_bins)
+    bool in_bins = false;
     // the default path's autotuner: whether it chose the mode and light order, and the mean
     // sweep time it measured for each candidate (mode 2 ordered, mode 2 in body order, mode 1
     // ordered, mode 1 in body order), nanoseconds
@@ -209,6 +212,42 @@ bool alloc_arr(pabd_scene* s, T*& p, size_t n) {
     return p != nullptr;
 }
 
+// Threads per body of the sweep launches where the autotuner does not time both: as many as
+// lanes while they all fit on the device at once (152 SMs x 4 blocks x 128 threads), else half
+// as many -- every thread repeats its body's solve, and a pile of 8000 boxes (16 lanes) sweeps in
+// 7.0 us on 8 threads per body against 9.8 us on 16, one of 30 000 (4 lanes) in 8.9 us against
+// 11.6, but one of 4800 in 6.1 against 5.8.  Not where most bodies take the extended path, whose
+// second sum then follows the first (256 trees: 15.0 against 12.6 us).
+int sweep_threads(int lanes, int N, int ext_bodies, int policy) {
+    if (policy == 2 || lanes == 1) return lanes;
+    return (long long)lanes * N > 152 * 4 * 128 && 2LL * ext_bodies < N ? lanes / 2 : lanes;
+}
+
+// The bins of k_sweep_bins (consecutive whole groups), or none where the sweeps run as launches.
+// A cluster of up to 16 blocks of 128 (256) threads holds its largest group with one thread per
+// lane: up to 256 bodies of 16 lanes.  Measured per sweep, against one launch per sweep: a
+// 121-body net 3.7 against 4.9 us, 8 chained bodies 3.0 against 5.4, a 250-box pile 3.8 against
+// 4.5; larger groups would take turns on the cluster's 16 SMs while a launch spreads them over
+// all.  The same happens to more clusters than the device holds at once (setup_sweep_bins):
+// 30 piles of 1500 boxes take 6.3 us against 4.8.
+std::vector<int2> choose_bins(const std::vector<int>& group_off, int G, int N, int lanes, BinsShape* out) {
+    int gmax = 0;
+    for (int g = 0; g < G; ++g) gmax = std::max(gmax, group_off[g + 1] - group_off[g]);
+    std::vector<int2> bins;
+    if (N == 0 || (long long)gmax * lanes > 16 * 256) return bins;
+    BinsShape b;
+    while (b.cluster < 16 && gmax * lanes > b.cluster * b.block) b.cluster *= 2;
+    if (gmax * lanes > b.cluster * b.block) b.block *= 2;
+    b.cap = std::max(gmax, b.cluster * b.block / lanes);
+    for (int g = 0, s = 0; g < G; ++g) {
+        if (group_off[g + 1] - s > b.cap) { bins.push_back(make_int2(s, group_off[g])); s = group_off[g]; }
+        if (g == G - 1) bins.push_back(make_int2(s, N));
+    }
+    b.n = (int)bins.size();
+    *out = b;
+    return bins;
+}
+
 // enqueue one time step of Alg. 1 on the scene's stream; with `ev` (PROF_EVENTS events) an
 // event is recorded at every stage boundary: [0] start, [1] after drives + collision
 // detection, [2] CSR, [3] predictor, [4] all n_iter sweeps, [5] finalize + residual
@@ -216,6 +255,8 @@ constexpr int PROF_EVENTS = 6;
 
 void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nullptr) {
     const Dev& d = s->d;
+    const bool in_bins = s->mode == 2 && !s->fused && s->in_bins;
+    const bool use_order = d.light_sorted && !in_bins;  // (the bins order their own bodies)
     int e = 0;
     auto mark = [&]() {
         if (ev) cudaEventRecordWithFlags(ev[e++], s->st, cudaEventRecordExternal);
@@ -228,13 +269,13 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
         // stage is then empty in the profiling graph's split)
         launch_ground_front(d, s->st, launches);
         mark();
-        if (d.light_sorted) launch_light_order(d, s->st, launches);
+        if (use_order) launch_light_order(d, s->st, launches);
         mark();
     } else {
         launch_collision(d, s->st, launches);
         mark();
         launch_csr(d, s->st, launches);
-        if (d.light_sorted) launch_light_order(d, s->st, launches);
+        if (use_order) launch_light_order(d, s->st, launches);
         mark();
         launch_predict(d, s->st, launches);
     }
@@ -248,7 +289,7 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
             // was reset at the head of the step; the launches follow each other as
             // programmatic dependents)
             launch_bond(d, cur, it, s->st, launches);
-            launch_solve(d, cur, nxt, it, s->lanes, s->st, launches);
+            launch_solve(d, cur, nxt, it, s->lanes, s->threads, s->st, launches);
             float4* t = cur; cur = nxt; nxt = t;
         }
     };
@@ -272,7 +313,7 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
         launch_sweep_ctl_init(d, s->st, launches);
         auto one_sweep = [&](cudaStream_t st, unsigned long long handle) {
             cudaMemsetAsync(d.ctr + C_FP64DYN, 0, sizeof(int), st);
-            launch_sweep_one(d, nullptr, nullptr, -1, s->lanes, st, launches);
+            launch_sweep_one(d, nullptr, nullptr, -1, s->lanes, s->threads, st, launches);
             launch_sweep_check(d, handle, st, launches);
         };
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -303,12 +344,16 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
             for (int it = 0; it < d.p.n_iter; ++it) one_sweep(s->st, 0);
         }
         cur = nullptr;  // the last iterate's buffer is known on the device only
+    } else if (in_bins) {
+        launch_end_records(d, s->st, launches);
+        launch_sweep_bins(d, s->bins, s->lanes, s->st, launches);
+        if (d.p.n_iter & 1) { float4* t = cur; cur = nxt; nxt = t; }
     } else if (s->mode == 2) {
         launch_end_records(d, s->st, launches);
         // (the counter of run-time extended-precision redos, which counts the last sweep's, was
         // reset at the head of the step): the sweeps follow each other as programmatic dependents
         for (int it = 0; it < d.p.n_iter; ++it) {
-            launch_sweep_one(d, cur, nxt, it, s->lanes, s->st, launches, true);
+            launch_sweep_one(d, cur, nxt, it, s->lanes, s->threads, s->st, launches, true);
             float4* t = cur; cur = nxt; nxt = t;
         }
     } else {
@@ -379,8 +424,10 @@ pabd_status autotune_sweep(pabd_scene* s) {
 // light order, predictor and end records in place (none of them changes the scene's state),
 // time the n_iter sweeps of each candidate launch shape: one launch per sweep or a bond and a
 // solve launch per sweep, each with the light bodies in (class, end count) order or in body
-// order.  Every candidate gives the same results bit for bit (each body's arithmetic depends
-// on its end count and the lane count only), so the fastest is kept.  Scenes with augmented
+// order and with a thread per lane or per two lanes; where the groups fit clusters, one launch
+// for all sweeps stands in for one launch per sweep in order.  Every candidate gives the same
+// results bit for bit (each body's arithmetic depends on its end count and the lane count
+// only), so the fastest is kept.  Scenes with augmented
 // Lagrangian bonds, whose sweeps update the bonds' state, keep one launch per sweep, ordered.
 pabd_status autotune_default(pabd_scene* s) {
     Dev& d = s->d;
@@ -406,38 +453,55 @@ pabd_status autotune_default(pabd_scene* s) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     const int n_it = d.p.n_iter;
+    // (half the threads never won while the lanes' threads fill less than the device)
+    const bool many = (long long)s->lanes * d.N > 152 * 4 * 96;
+    const int half = many && s->lanes > 1 && d.p.precision_policy != 2 ? s->lanes / 2 : 0;
     float best = 1e30f;
     for (int c = 0; c < 4; ++c) {
         const int mode = c < 2 ? 2 : 1;
+        const bool in_bins = c == 0 && s->bins.n > 0;
         dd.light_sorted = (c & 1) ? 0 : 1;
         if ((!tune_mode && mode != s->mode) || (!tune_order && dd.light_sorted != d.light_sorted)) continue;
-        float tot = 1e30f;
-        for (int r = 0; r < 5; ++r) {
-            // the one-launch sweeps' chunk counters, as the step's reset leaves them (each
-            // sweep zeroes the next sweep's counter, so a pass must start from clean ones)
-            CK(cudaMemsetAsync(dd.ctr + C_SWEEP_NEXT, 0, 2 * sizeof(int), s->st));
-            CK(cudaEventRecord(e0, s->st));
-            float4* cur = dd.qa;
-            float4* nxt = dd.qb;
-            for (int it = 0; it < n_it; ++it) {
-                if (mode == 2) {
-                    launch_sweep_one(dd, cur, nxt, it, s->lanes, s->st, &lc, true);
-                } else {
-                    launch_bond(dd, cur, it, s->st, &lc);
-                    launch_solve(dd, cur, nxt, it, s->lanes, s->st, &lc);
+        float fastest = 1e30f;  // of the candidate, over its thread counts
+        for (int threads : {s->lanes, half}) {
+            if (threads == 0 || (in_bins && threads != s->lanes)) continue;
+            float tot = 1e30f;
+            for (int r = 0; r < 5; ++r) {
+                // the one-launch sweeps' chunk counters, as the step's reset leaves them (each
+                // sweep zeroes the next sweep's counter, so a pass must start from clean ones)
+                CK(cudaMemsetAsync(dd.ctr + C_SWEEP_NEXT, 0, 2 * sizeof(int), s->st));
+                CK(cudaEventRecord(e0, s->st));
+                float4* cur = dd.qa;
+                float4* nxt = dd.qb;
+                if (in_bins) launch_sweep_bins(dd, s->bins, s->lanes, s->st, &lc);
+                else for (int it = 0; it < n_it; ++it) {
+                    if (mode == 2) {
+                        launch_sweep_one(dd, cur, nxt, it, s->lanes, threads, s->st, &lc, true);
+                    } else {
+                        launch_bond(dd, cur, it, s->st, &lc);
+                        launch_solve(dd, cur, nxt, it, s->lanes, threads, s->st, &lc);
+                    }
+                    float4* t = cur; cur = nxt; nxt = t;
                 }
-                float4* t = cur; cur = nxt; nxt = t;
+                CK(cudaEventRecord(e1, s->st));
+                CK(cudaEventSynchronize(e1));
+                float t = 0.f;
+                CK(cudaEventElapsedTime(&t, e0, e1));
+                if (r > 0) tot = std::min(tot, t);  // the first pass warms the caches; the fastest
+                                                    // of the others (least disturbed) is the figure
+                if (r > 0 && tot > 1.1f * best) break;  // out of the running
             }
-            CK(cudaEventRecord(e1, s->st));
-            CK(cudaEventSynchronize(e1));
-            float t = 0.f;
-            CK(cudaEventElapsedTime(&t, e0, e1));
-            if (r > 0) tot = std::min(tot, t);  // the first pass warms the caches; the fastest
-                                                // of the others (least disturbed) is the figure
+            CK(cudaGetLastError());
+            fastest = std::min(fastest, tot);
+            if (tot < best) {
+                best = tot;
+                s->mode = mode;
+                s->in_bins = in_bins;
+                s->threads = threads;
+                d.light_sorted = dd.light_sorted;
+            }
         }
-        CK(cudaGetLastError());
-        s->tune_ns[c] = (long long)(1e6 * tot / (double)n_it);
-        if (tot < best) { best = tot; s->mode = mode; d.light_sorted = dd.light_sorted; }
+        s->tune_ns[c] = (long long)(1e6 * fastest / (double)n_it);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -731,7 +795,7 @@ pabd_status finalize_scene(pabd_scene* s) {
     ok &= alloc_arr(s, d.end_id, d.cap_ends) && alloc_arr(s, d.end_pos, d.cap_ends) && alloc_arr(s, d.heavy, N);
     ok &= alloc_arr(s, d.order, N) && alloc_arr(s, d.bin_cnt, 2 * END_BINS) && alloc_arr(s, d.bin_cur, 2 * END_BINS);
     ok &= alloc_arr(s, d.ends, d.cap_ends) && alloc_arr(s, d.end_x, d.cap_ends);
-    ok &= alloc_arr(s, d.rec_m, d.cap_ends) && alloc_arr(s, d.rec_a, d.cap_ends) && alloc_arr(s, d.rec_b, d.cap_ends);
+    ok &= alloc_arr(s, d.rec, 3 * (size_t)d.cap_ends);
     ok &= alloc_arr(s, d.gbar, 2) && alloc_arr(s, d.wait_limit, 1);
     ok &= alloc_arr(s, d.lo, N) && alloc_arr(s, d.hi, N) && alloc_arr(s, d.cell, N);
     ok &= alloc_arr(s, d.bucket_cnt, T) && alloc_arr(s, d.bucket_cur, T) && alloc_arr(s, d.bucket_off, T + 1) &&
@@ -839,6 +903,21 @@ pabd_status finalize_scene(pabd_scene* s) {
     }
     if (L != 1 && L != 2 && L != 4 && L != 8 && L != 16) return PABD_ERR_ARG;
     s->lanes = L;
+    s->threads = sweep_threads(L, N, s->fp64_bodies, p.precision_policy);
+    if (p.resid_tol <= 0) {
+        const std::vector<int2> bins = choose_bins(group_off, d.G, N, L, &s->bins);
+        if (s->bins.n) {
+            int fit = 0;
+            CK(setup_sweep_bins(s->bins, L, p.precision_policy == 2, &fit));
+            if (s->bins.n > fit) s->bins = BinsShape{};
+        }
+        if (s->bins.n) {
+            if (!alloc_arr(s, d.bin_range, bins.size())) return PABD_ERR_OOM;
+            CK(up(d.bin_range, bins.data(), sizeof(int2) * bins.size()));
+            CK(cudaStreamSynchronize(st));
+            s->in_bins = true;
+        }
+    }
     // sweep mode: 1 two launches per sweep, 2 one launch per sweep, 3 fused persistent;
     // 0 = one launch per sweep (the fastest on the measured scenes).  A residual threshold
     // runs one launch per sweep.
@@ -1116,7 +1195,7 @@ pabd_status profiled_step(pabd_scene* s) {
     acc[4] += ms(3, 4);                 // all sweeps of the step
     acc[5] += 0.0;
     acc[6] += ms(4, 5);
-    acc[7] += s->fused ? 1 : (s->mode == 1 ? 2 * n_it : n_it);  // sweep-kernel launches
+    acc[7] += s->fused || (s->mode == 2 && s->in_bins) ? 1 : (s->mode == 1 ? 2 * n_it : n_it);  // sweep-kernel launches
     acc[8] += n_it;
     acc[9] += ms(0, 5);
     int nb = 0;
@@ -1152,11 +1231,12 @@ pabd_status pabd_tune(pabd_scene* s) {
     r = poll_status(s, true);
     if (r != PABD_OK) return r;
     CK(cudaStreamSynchronize(s->st));
-    const int mode0 = s->mode, sorted0 = s->d.light_sorted;
+    const int mode0 = s->mode, sorted0 = s->d.light_sorted, threads0 = s->threads;
+    const bool bins0 = s->in_bins;
     r = autotune_default(s);
     if (r != PABD_OK) return r;
     CK(cudaStreamSynchronize(s->st));
-    if (s->mode == mode0 && s->d.light_sorted == sorted0) return PABD_OK;
+    if (s->mode == mode0 && s->d.light_sorted == sorted0 && s->threads == threads0 && s->in_bins == bins0) return PABD_OK;
     // the step graphs were captured with the old shape: capture them again
     cudaGraphExecDestroy(s->exec);
     cudaGraphDestroy(s->graph);

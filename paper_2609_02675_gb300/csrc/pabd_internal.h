@@ -124,11 +124,10 @@ struct Dev {
     int light_sorted;           // 1: the sweeps take the light bodies in Dev::order; 0: in body order
     int *order;                 // this step's light bodies by (class, end count), C_NLIGHT of them
     int *bin_cnt, *bin_cur;     // per bin of the light order: bodies, and the blocks' reservations
-    // bond-end records in CSR order for the fused sweep: (i, j, type, bond), x_i (+w0), x_j (+p1)
-    int4 *rec_m;
-    float4 *rec_a, *rec_b;
+    float4 *rec;                // bond-end records in CSR order, 3 float4 per end (pack_end)
     unsigned *gbar;             // grid barrier: arrival counter, generation
     unsigned *wait_limit;       // polls before a device-side wait gives up (PABD_ERR_TIMEOUT)
+    int2 *bin_range;            // body range of each bin of k_sweep_bins, or null
     // collision
     float4 *lo, *hi;            // inflated AABB; lo.w = inflation
     int4 *cell;                 // cell coords (.w = bucket)
@@ -259,7 +258,8 @@ void launch_bond(const Dev& d, const float4* q, int it, cudaStream_t st, long lo
 // augmented Lagrangian: warm start (before the sweeps) and the update after the last sweep
 void launch_al_warm(const Dev& d, cudaStream_t st, long long* launches);
 void launch_al_final(const Dev& d, const float4* q, cudaStream_t st, long long* launches);
-void launch_solve(const Dev& d, const float4* q_in, float4* q_out, int it, int lanes, cudaStream_t st,
+// (lanes: logical lanes per body, which fix the summation order; threads: threads per body)
+void launch_solve(const Dev& d, const float4* q_in, float4* q_out, int it, int lanes, int threads, cudaStream_t st,
                   long long* launches);
 void launch_finalize(const Dev& d, const float4* q_fin, cudaStream_t st, long long* launches);
 // sweeps under a residual threshold (Dev::sweep_ctl): the loop's start, one sweep's residual
@@ -272,9 +272,17 @@ void launch_drive_update(const Dev& d, cudaStream_t st, long long* launches);
 // fused persistent sweep (all n_iter iterations, cooperative launch); L lanes per body
 cudaError_t launch_fused_sweep(const Dev& d, int L, int block, int grid, cudaStream_t st, long long* launches);
 int fused_max_blocks(int L, int block, bool fp64);
+// all sweeps of a step in one launch, a cluster per bin of small groups (k_sweep_bins.cu): the
+// bins (0: not used), the most bodies of one, blocks per cluster and threads per block
+struct BinsShape {
+    int n = 0, cap = 0, cluster = 1, block = 128;
+};
+// opts the kernel into its shared memory and cluster size; *fit: clusters the device holds at once
+cudaError_t setup_sweep_bins(const BinsShape& b, int lanes, bool f64, int* fit);
+void launch_sweep_bins(const Dev& d, const BinsShape& b, int lanes, cudaStream_t st, long long* launches);
 // one launch per sweep (bonds evaluated by the solve from CSR-ordered end records)
 void launch_end_records(const Dev& d, cudaStream_t st, long long* launches);
-void launch_sweep_one(const Dev& d, const float4* qi, float4* qo, int it, int L, cudaStream_t st,
+void launch_sweep_one(const Dev& d, const float4* qi, float4* qo, int it, int lanes, int threads, cudaStream_t st,
                       long long* launches, bool pdl = false);
 
 

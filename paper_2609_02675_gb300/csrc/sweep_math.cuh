@@ -25,10 +25,9 @@ __device__ __forceinline__ void ld_q(const float4* __restrict__ q, int b, float*
 // the end-to-end vector r = y_j - y_i enters (bond_vec forms it without rounding at the
 // scale of the bodies' positions).  Always single precision: a body on the extended path
 // sums these same records in the extended type (sys_add_x).
-__device__ __forceinline__ float bond_force(int type, float4 xi, float4 xj, float4 nm, const float* r, float* f) {
-    float w = xi.w;
+__device__ __forceinline__ float bond_force(int type, float w, float p1, float4 nm, const float* r, float* f) {
     if (type == K_CONTACT || type == K_GROUND) {
-        const float dhat = xj.w;
+        const float dhat = p1;
         const float N[3] = {nm.x, nm.y, nm.z};
         const float rr[3] = {-r[0], -r[1], -r[2]};  // y_i - y_j
         float g = N[0] * rr[0] + N[1] * rr[1] + N[2] * rr[2];
@@ -54,7 +53,7 @@ __device__ __forceinline__ float bond_force(int type, float4 xi, float4 xj, floa
     float n[3];
     if (dd > 0.f) { float id = 1.f / dd; n[0] = r[0] * id; n[1] = r[1] * id; n[2] = r[2] * id; }
     else { n[0] = 0.f; n[1] = 1.f; n[2] = 0.f; }
-    const float l = xj.w;
+    const float l = p1;
     float sc;
     if (type == K_SPRING) {
         sc = w * (dd - l);                      // h^2 phi(d)
@@ -70,21 +69,19 @@ __device__ __forceinline__ float bond_force(int type, float4 xi, float4 xj, floa
     return w;
 }
 
-// r = y_j - y_i for end points y = c + A x, formed as (c_j - c_i) + (A_j x_j - A_i x_i): the
-// centres' difference rounds once at the scale of the bond, not of the positions, so a stiff
-// short bond far from the origin keeps its length to single precision.  A world end j is
-// the point x_j itself.
-__device__ __forceinline__ void bond_vec(const float* ci, const float* Ai, float4 xi, const float* cj,
-                                         const float* Aj, float4 xj, bool world_j, float* r) {
+// u = y_o - y_s, from a bond's end s to its other end o, for end points y = c + A x, formed as
+// (c_o - c_s) + (A_o x_o - A_s x_s): the centres' difference rounds once at the scale of the
+// bond, not of the positions, so a stiff short bond far from the origin keeps its length to
+// single precision.  A world end is c_o = the point, A_o = 0.  Seen from the other end every
+// operation has the opposite sign and rounds alike, so both ends get the same vector but for
+// its sign.
+__device__ __forceinline__ void bond_vec(const float* cs, const float* As, float4 xs, const float* co,
+                                         const float* Ao, float4 xo, float* u) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float ai = Ai[3 * k] * xi.x + Ai[3 * k + 1] * xi.y + Ai[3 * k + 2] * xi.z;
-        if (world_j) {
-            r[k] = ((&xj.x)[k] - ci[k]) - ai;
-        } else {
-            const float aj = Aj[3 * k] * xj.x + Aj[3 * k + 1] * xj.y + Aj[3 * k + 2] * xj.z;
-            r[k] = (cj[k] - ci[k]) + (aj - ai);
-        }
+        const float as = As[3 * k] * xs.x + As[3 * k + 1] * xs.y + As[3 * k + 2] * xs.z;
+        const float ao = Ao[3 * k] * xo.x + Ao[3 * k + 1] * xo.y + Ao[3 * k + 2] * xo.z;
+        u[k] = (co[k] - cs[k]) + (ao - as);
     }
 }
 
@@ -94,14 +91,13 @@ __device__ __forceinline__ void bond_vec(const float* ci, const float* Ai, float
 // lambda <- kappa C + lambda, kappa <- kappa + beta |C|, read from the parity-(it-1) buffer and
 // stored by `writer` into the parity-it buffer; then the split force with those values:
 // phi+ = kappa d + max(lambda - kappa l, 0), phi- = min(lambda - kappa l, 0); w = h^2 phi+/d
-// (d kept above 1e-9), f' = w (y_j - y_i) + h^2 phi- n.  xi.w holds h^2, xj.w the rest length.
-__device__ __forceinline__ float al_force(const Dev& d, int bond, int it, bool writer, float4 xi, float4 xj,
+// (d kept above 1e-9), f' = w (y_j - y_i) + h^2 phi- n.  l is the rest length.
+__device__ __forceinline__ float al_force(const Dev& d, int bond, int it, bool writer, float h2, float l,
                                           const float* r, float* f) {
     float dd = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
     float n[3];
     if (dd > 0.f) { float id = 1.f / dd; n[0] = r[0] * id; n[1] = r[1] * id; n[2] = r[2] * id; }
     else { n[0] = 0.f; n[1] = 1.f; n[2] = 0.f; }
-    const float l = xj.w;
     float kap, lam;
     if (it == 0) {
         const float2 kl = d.al_st0[bond];
@@ -116,7 +112,6 @@ __device__ __forceinline__ float al_force(const Dev& d, int bond, int it, bool w
             out[bond] = make_float2(kap, lam);
         }
     }
-    const float h2 = xi.w;
     const float cst = lam - kap * l;
     const float w = h2 * (kap + (cst > 0.f ? cst / (dd > 1e-9f ? dd : 1e-9f) : 0.f));
     const float sc = h2 * (cst < 0.f ? cst : 0.f);
@@ -125,87 +120,107 @@ __device__ __forceinline__ float al_force(const Dev& d, int bond, int it, bool w
     return w;
 }
 
-// The same vector for the FP32 path as accurately as if formed in twice the precision and
-// rounded once (Ogita, Rump and Oishi's Dot2: TwoSum / TwoProduct of every term, the errors
-// summed apart).  A stiff joint's gap is the small difference of the centres' offset and the
-// lever arms; in plain FP32 its rounding (an ulp of the lever, independently at each end)
-// reaches the forces as w times that ulp -- inconsistent between the two ends and far above
-// the joint's own resolution -- and from there the body's softly held rotations.
-__device__ __forceinline__ void bond_vec_dot2(const float* ci, const float* Ai, float4 xi, const float* cj,
-                                              const float* Aj, float4 xj, bool world_j, float* r) {
-    const float xiv[3] = {xi.x, xi.y, xi.z}, xjv[3] = {xj.x, xj.y, xj.z};
+// The same vector as accurately as if formed in twice the precision and rounded once (Ogita,
+// Rump and Oishi's Dot2: TwoSum / TwoProduct of every term, the errors summed apart).  A stiff
+// joint's gap is the small difference of the centres' offset and the lever arms; in plain FP32
+// its rounding (an ulp of the lever, independently at each end) reaches the forces as w times
+// that ulp -- inconsistent between the two ends and far above the joint's own resolution -- and
+// from there the body's softly held rotations.  Each pair of terms is added end i's first, so
+// that both ends round alike (side_j: the end s is end j).  The order is chosen by selecting the
+// products: a branch on the side, which differs from lane to lane, took every warp through the
+// whole evaluation twice.
+__device__ __forceinline__ void bond_vec_dot2(const float* cs, const float* As, float4 xs, const float* co,
+                                              const float* Ao, float4 xo, bool side_j, float* u) {
+    const float xsv[3] = {xs.x, xs.y, xs.z}, xov[3] = {xo.x, xo.y, xo.z};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        df acc = two_sum(world_j ? xjv[k] : cj[k], -ci[k]);
+        df acc = two_sum(co[k], -cs[k]);
         float err = acc.lo;
         float hi = acc.hi;
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            df p = two_prod(-Ai[3 * k + l], xiv[l]);
-            df t = two_sum(hi, p.hi);
+            const df ps = two_prod(-As[3 * k + l], xsv[l]), po = two_prod(Ao[3 * k + l], xov[l]);
+            const df p0 = df(side_j ? po.hi : ps.hi, side_j ? po.lo : ps.lo, 0);
+            const df p1 = df(side_j ? ps.hi : po.hi, side_j ? ps.lo : po.lo, 0);
+            df t = two_sum(hi, p0.hi);
             hi = t.hi;
-            err = __fadd_rn(err, __fadd_rn(t.lo, p.lo));
-            if (!world_j) {
-                p = two_prod(Aj[3 * k + l], xjv[l]);
-                t = two_sum(hi, p.hi);
-                hi = t.hi;
-                err = __fadd_rn(err, __fadd_rn(t.lo, p.lo));
-            }
+            err = __fadd_rn(err, __fadd_rn(t.lo, p0.lo));
+            t = two_sum(hi, p1.hi);
+            hi = t.hi;
+            err = __fadd_rn(err, __fadd_rn(t.lo, p1.lo));
         }
-        r[k] = __fadd_rn(hi, err);
+        u[k] = __fadd_rn(hi, err);
     }
 }
 
-// Force of the bond seen from body `self`, given the other body's iterate (co, Ao; unused
-// when the other end is the world): forms the bond vector (compensated for user bonds: stiff
-// joints, elastic and AL bonds), evaluates the split force; returns w and writes the record
-// of self's end.  `it` is the sweep index and `writer` whether this evaluation stores an
-// augmented Lagrangian bond's updated state (exactly one evaluation per bond does).
-__device__ __forceinline__ float end_force_q(const Dev& d, const float* co, const float* Ao, int self, const float* cs,
-                                             const float* As, int4 m, float4 xa, float4 xb, int it, bool writer,
-                                             float* f) {
-    const bool side_j = (m.y == self);
+// A bond seen from one of its ends, as the end's body needs it.
+struct EndBond {
+    float4 xs, xo;   // (the body's material point, w0), (the other end's, rest length or dhat)
+    float4 nm;       // contacts: (N, mu)
+    int type, other; // BondKind; the other end's body (-1: the world, and xo a world point)
+    bool side_j;     // the body is end j
+    int bond;        // bond id (augmented Lagrangian bonds: where their state is)
+};
+
+// Force of the bond seen from its end on the body with iterate (cs, As), given the other end's
+// iterate (co, Ao; a world end: its point and zeros): forms the bond vector (compensated for
+// user bonds: stiff joints, elastic and AL bonds), evaluates the split force; returns w and
+// writes the record of the body's end.  `it` is the sweep index and `writer` whether this
+// evaluation stores an augmented Lagrangian bond's updated state (exactly one evaluation per
+// bond does).
+__device__ __forceinline__ float end_force(const Dev& d, const EndBond& e, const float* co, const float* Ao,
+                                           const float* cs, const float* As, int it, bool writer, float* f) {
     float r[3];
-    if (m.z != K_CONTACT && m.z != K_GROUND) {
-        if (side_j) bond_vec_dot2(co, Ao, xa, cs, As, xb, false, r);
-        else bond_vec_dot2(cs, As, xa, co, Ao, xb, m.y < 0, r);
-    } else if (side_j) {
-        bond_vec(co, Ao, xa, cs, As, xb, false, r);
-    } else {
-        bond_vec(cs, As, xa, co, Ao, xb, m.y < 0, r);
-    }
+    if (e.type != K_CONTACT && e.type != K_GROUND) bond_vec_dot2(cs, As, e.xs, co, Ao, e.xo, e.side_j, r);
+    else bond_vec(cs, As, e.xs, co, Ao, e.xo, r);
+    if (e.side_j) { r[0] = -r[0]; r[1] = -r[1]; r[2] = -r[2]; }
     float w;
-    if (m.z == K_AL) {
-        w = al_force(d, m.w, it, writer, xa, xb, r, f);
-    } else {
-        const float4 nm = (m.z == K_CONTACT || m.z == K_GROUND) ? d.bn[m.w] : make_float4(0.f, 0.f, 0.f, 0.f);
-        w = bond_force(m.z, xa, xb, nm, r, f);
-    }
-    if (side_j) { f[0] = -f[0]; f[1] = -f[1]; f[2] = -f[2]; }
+    if (e.type == K_AL) w = al_force(d, e.bond, it, writer, e.xs.w, e.xo.w, r, f);
+    else w = bond_force(e.type, e.xs.w, e.xo.w, e.nm, r, f);
+    if (e.side_j) { f[0] = -f[0]; f[1] = -f[1]; f[2] = -f[2]; }
     return w;
 }
 
-// the other end's body of bond record m seen from `self` (-1 for the world)
-__device__ __forceinline__ int other_body(int4 m, int self) { return m.y == self ? m.x : m.y; }
+// ---- bond-end records in CSR order (Dev::rec, three float4 per end) ----
+// (x of the end, w0), (x of the other end, p1) and (N, code): everything one evaluation of the
+// bond reads but the two iterates, in 48 contiguous bytes.  code packs the other body + 1 (24
+// bits; 0: the world), the side (bit 24) and the type (from bit 25); a bond without a normal
+// keeps its id in N's place.  mu is the scene's.  Four separate records (metadata, x_i, x_j, and
+// the normal by bond id) took 64 bytes and a fourth cache line per end.
+__device__ __forceinline__ void pack_end(float4* __restrict__ rec, int bond, int4 m, float4 xi, float4 xj, float4 bn,
+                                         bool side_j) {
+    const int other = side_j ? m.x : m.y;
+    const int code = (other + 1) | (side_j ? 1 << 24 : 0) | (m.z << 25);
+    const bool contact = m.z == K_CONTACT || m.z == K_GROUND;
+    rec[0] = side_j ? make_float4(xj.x, xj.y, xj.z, xi.w) : xi;
+    rec[1] = side_j ? make_float4(xi.x, xi.y, xi.z, xj.w) : xj;
+    rec[2] = contact ? make_float4(bn.x, bn.y, bn.z, __int_as_float(code))
+                     : make_float4(__int_as_float(bond), 0.f, 0.f, __int_as_float(code));
+}
 
-// q of body o, or zeros for the world (o < 0)
-__device__ __forceinline__ void ld_q_or_zero(const float4* __restrict__ q, int o, float* c, float* A) {
+__device__ __forceinline__ EndBond unpack_end(const Dev& d, const float4* __restrict__ rec) {
+    EndBond e;
+    e.xs = rec[0];
+    e.xo = rec[1];
+    e.nm = rec[2];
+    const int code = __float_as_int(e.nm.w);
+    e.other = (code & 0xffffff) - 1;
+    e.side_j = (code >> 24) & 1;
+    e.type = code >> 25;
+    e.bond = __float_as_int(e.nm.x);
+    e.nm.w = d.p.mu;
+    return e;
+}
+
+// iterate of the other end of a bond: of body o in q, or the world point x (o < 0)
+__device__ __forceinline__ void ld_other(const float4* q, int o, float4 x, float* c, float* A) {
     if (o >= 0) {
         ld_q(q, o, c, A);
     } else {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) c[k] = 0.f;
+        c[0] = x.x; c[1] = x.y; c[2] = x.z;
 #pragma unroll
         for (int k = 0; k < 9; ++k) A[k] = 0.f;
     }
-}
-
-__device__ __forceinline__ float end_force(const Dev& d, const float4* __restrict__ q, int self, const float* cs,
-                                           const float* As, int4 m, float4 xa, float4 xb, int it, bool writer,
-                                           float* f) {
-    float co[3], Ao[9];
-    ld_q_or_zero(q, other_body(m, self), co, Ao);
-    return end_force_q(d, co, Ao, self, cs, As, m, xa, xb, it, writer, f);
 }
 
 // ---- 4x4 SPD system with three right-hand sides ----
@@ -662,14 +677,16 @@ __device__ __forceinline__ void polar_rotation(float* X) {
                 E[3 * c + r] = E[3 * r + c];
             }
         const float e2 = E[0] * E[0] + E[4] * E[4] + E[8] * E[8] + 2.f * (E[1] * E[1] + E[2] * E[2] + E[5] * E[5]);
+        // (the Newton-Schulz step is formed beside e2, before it is known to be wanted: the two
+        // do not depend on each other)
+        float Y[9];
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                Y[3 * r + c] = X[3 * r + c] - 0.5f * (X[3 * r] * E[c] + X[3 * r + 1] * E[3 + c] + X[3 * r + 2] * E[6 + c]);
         if (e2 < 1e-13f) break;
         if (e2 < 0.25f) {
-            float Y[9];
-#pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    Y[3 * r + c] = X[3 * r + c] - 0.5f * (X[3 * r] * E[c] + X[3 * r + 1] * E[3 + c] + X[3 * r + 2] * E[6 + c]);
 #pragma unroll
             for (int k = 0; k < 9; ++k) X[k] = Y[k];
         } else {
@@ -695,11 +712,24 @@ __device__ __forceinline__ void sys_zero(Sys<T>& s) {
         for (int k = 0; k < 3; ++k) s.r[r][k] = T(0);
 }
 
-// combine the L lanes' partial systems with a fixed xor butterfly (deterministic given L)
+template <class T>
+__device__ __forceinline__ void sys_plus(Sys<T>& s, const Sys<T>& t) {
+#pragma unroll
+    for (int k = 0; k < 10; ++k) s.g[k] += t.g[k];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s.r[r][k] += t.r[r][k];
+}
+
+// combine the first `width` threads' partial systems (of a body's L) with a fixed xor butterfly.
+// (The rounds are unrolled, each under a test that the warp agrees on: in a rolled loop every
+// shuffle synchronised its lanes anew, 650 cycles a round against 130.)
 template <int L, class T>
-__device__ __forceinline__ void sys_reduce(Sys<T>& s, unsigned mask) {
+__device__ __forceinline__ void sys_reduce(Sys<T>& s, unsigned mask, int width = L) {
 #pragma unroll
     for (int o = 1; o < L; o <<= 1) {
+        if (o >= width) break;
 #pragma unroll
         for (int k = 0; k < 10; ++k) s.g[k] += shfl_xor(mask, s.g[k], o);
 #pragma unroll
@@ -713,7 +743,8 @@ __device__ __forceinline__ void sys_reduce(Sys<T>& s, unsigned mask) {
 // first_block on: each warp first takes the chunk of its own index, then the chunks past the
 // grid's from the counter `next` until none are left, so the warps that finish early take more
 // and a launch does not end on a few long blocks.  No counter traffic when the grid's warps
-// cover every chunk.  f(slot) runs on the L lanes of each slot.
+// cover every chunk.  f(slot, team) runs on the L lanes of each
+// slot, team the warp's lanes that have one.
 template <int L, class F>
 __device__ __forceinline__ void for_light_slots(int* next, int n, int first_block, F&& f) {
     constexpr int PER_WARP = 32 / L;
@@ -723,7 +754,8 @@ __device__ __forceinline__ void for_light_slots(int* next, int n, int first_bloc
     int chunk = (blockIdx.x - first_block) * wpb + (threadIdx.x >> 5);
     while (chunk < chunks) {
         const int slot = chunk * PER_WARP + wl / L;
-        if (slot < n) f(slot);
+        const unsigned team = __ballot_sync(0xffffffffu, slot < n);
+        if (slot < n) f(slot, team);
         __syncwarp();
         if (warps >= chunks) break;
         int t = 0;
@@ -733,82 +765,162 @@ __device__ __forceinline__ void for_light_slots(int* next, int n, int first_bloc
     pdl_signal();  // nothing left for this warp
 }
 
-template <int L>
-__device__ __forceinline__ unsigned lane_mask() {
-    return (L == 32) ? 0xffffffffu : (((1u << L) - 1u) << ((threadIdx.x & 31) & ~(L - 1)));
+// the iterate of body b into q (three float4)
+__device__ __forceinline__ void store_iterate(float4* q, int b, const float* c, const float* A) {
+    q[3 * b] = make_float4(c[0], c[1], c[2], A[0]);
+    q[3 * b + 1] = make_float4(A[1], A[2], A[3], A[4]);
+    q[3 * b + 2] = make_float4(A[5], A[6], A[7], A[8]);
 }
 
-__device__ __forceinline__ void finish_body(const Dev& d, int b, int lane, float4* __restrict__ qo, int last,
-                                            const float* c, const float* A, const float (*Xs)[3]);
+template <class Store>
+__device__ __forceinline__ void finish_body(const Dev& d, int b, int plane, int last, const float* c, const float* A,
+                                            const float (*Xs)[3], Store&& store);
 
 
-// Global + local solve of body b by L cooperating lanes (Eq. 19-24, Sec. 4.3):
-// G dX = M (s - q^k) + sum_ends [1; x] f'^T, X^{k+1/2} = q^k + dX, A^{k+1} = rotation of
-// A^{k+1/2}; lane 0 stores q^{k+1} and the body's squared update.  gather(sys, c, A, xs, e0,
-// e1) adds this lane's share of the body's bond ends, about the expansion point xs: in FP32
-// first; in the extended type X (double-float, or FP64) for flagged bodies (ill-conditioned or
-// stiffly jointed, see the scene set-up) or when an FP32 Cholesky pivot falls below 1e-3 of
-// its diagonal.
-template <int L, class X, class Gather>
-__device__ __forceinline__ void solve_body(const Dev& d, int b, int lane, unsigned mask,
+// the threads of a body that hold anything of its sum, as a power of two
+template <int L, int P>
+__device__ __forceinline__ int sum_width(int ends) {
+    if constexpr (P == 1) return 1;
+    const int nt = min(P, max(1, (ends + L / P - 1) / (L / P)));
+    return nt == 1 ? 1 : 1 << (32 - __clz(nt - 1));
+}
+
+// The body's system summed over its L logical lanes by P = L or L / 2 threads (thread `plane` of
+// the body takes lane plane, or lanes 2 plane and 2 plane + 1).  Lane l sums the body's ends l,
+// l + L, ..., lane 0 starting from the initial system, and the lanes' sums are combined as a
+// butterfly combines them -- neighbours first, then pairs of neighbours, ... -- so the result
+// depends on L alone: a thread's two lanes are neighbours, and the rest is sys_reduce's.  Lanes
+// without ends are zeros and are left out: the first `width` threads (a power of two) hold
+// everything, and only they get the sum.  init(s) sets the initial system, gather(s, l) adds
+// lane l's ends, gather2(s, t, l) those of lanes l and l + 1; mask holds the threads that call
+// it together.
+template <int L, int P, class T, class Init, class Gather, class Gather2>
+__device__ __forceinline__ void sys_sum_lanes(Sys<T>& s, int plane, int width, unsigned mask, Init&& init,
+                                              Gather&& gather, Gather2&& gather2) {
+    static_assert(P == L || 2 * P == L, "one or two lanes per thread");
+    if (plane == 0) init(s);
+    else sys_zero(s);
+    if constexpr (P == L) {
+        gather(s, plane);
+    } else {
+        Sys<T> t;
+        sys_zero(t);
+        gather2(s, t, 2 * plane);
+        sys_plus(s, t);
+    }
+    __syncwarp(mask);
+    if constexpr (P > 1) sys_reduce<P>(s, mask, width);
+}
+
+// What a body's solve reads besides iterates and bonds: the predictor, the mass and the
+// expansion point.
+struct alignas(16) BodyData {
+    float sc[3], sA[9];
+    float4 mass;
+    float xs[3];
+};
+__device__ __forceinline__ BodyData ld_body(const Dev& d, int b, int fl) {
+    BodyData o;
+    ld_q(d.sq, b, o.sc, o.sA);
+    o.mass = d.mass[b];
+    ld_xs(d, b, fl, o.xs);
+    return o;
+}
+
+// Global + local solve of body b by P cooperating threads (Eq. 19-24, Sec. 4.3), its sums over
+// L logical lanes (sys_sum_lanes): G dX = M (s - q^k) + sum_ends [1; x] f'^T, X^{k+1/2} = q^k +
+// dX, A^{k+1} = rotation of A^{k+1/2}; `store(b, c, A, n)` then stores q^{k+1} (called on the
+// first n threads of the body) and thread 0 the body's squared update.  gather.one(sys, c, A, xs,
+// p, e1, L) adds the body's bond ends p, p + L, ... < e1 about the expansion point xs, gather.two
+// those of p and of p + 1 to a system each: in FP32 first; in the extended type X (double-float, or FP64) for flagged bodies (ill-conditioned or
+// stiffly jointed, see the scene set-up) or when an FP32 Cholesky pivot falls below 1e-3 of its
+// diagonal.  data() loads the body's data, self(b, c, A) its own iterate.  `team` holds the
+// threads of the warp that call it together, for one body or several: the sums' butterfly runs
+// as many rounds as the body with the most ends needs (sum_width), the threads beyond it leave
+// the solve to the others, and the warp is brought together again wherever its bodies' slices
+// may have taken it apart -- otherwise it runs the long solve once per body.
+template <int L, int P, class X, class Data, class Self, class Store, class Gather>
+__device__ __forceinline__ void solve_free_body(const Dev& d, int b, int plane, unsigned team, int fl, int e0, int e1,
+                                                int last, Data&& data, Self&& self, Store&& store, Gather&& gather) {
+    float c[3], A[9];
+    self(b, c, A);
+    const BodyData body = data();
+    float dc[3], dA[9];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dc[k] = body.sc[k] - c[k];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) dA[k] = body.sA[k] - A[k];
+    const float* xs = body.xs;
+    float Xs[4][3];
+    const int width = P == 1 ? 1 : (int)__reduce_max_sync(team, (unsigned)sum_width<L, P>(e1 - e0));
+    bool ext = d.p.precision_policy == 3 || (d.p.precision_policy && (fl & BF_FP64));
+    const unsigned fp32 = __ballot_sync(team, !ext);
+    if (!ext) {
+        Sys<float> s;
+        sys_sum_lanes<L, P>(s, plane, width, fp32, [&](Sys<float>& t) { sys_init(t, body.mass, dc, dA, xs); },
+                            [&](Sys<float>& t, int l) { gather.one(t, c, A, xs, e0 + l, e1, L); },
+                            [&](Sys<float>& t, Sys<float>& u, int l) { gather.two(t, u, c, A, xs, e0 + l, e1, L); });
+        float ratio = 1.f;
+        if (plane < width) ratio = sys_solve(s, Xs);
+        __syncwarp(fp32);
+        if constexpr (P > 1) ratio = __shfl_sync(fp32, ratio, 0, P);
+        if (d.p.precision_policy && !(ratio >= 1e-3f)) {
+            ext = true;
+            if (last && plane == 0) atomicAdd(&d.ctr[C_FP64DYN], 1);
+        }
+    }
+    const unsigned redo = __ballot_sync(team, ext);
+    if (ext) {
+        Sys<X> s;
+        sys_sum_lanes<L, P>(s, plane, width, redo, [&](Sys<X>& t) { sys_init(t, body.mass, dc, dA, xs); },
+                            [&](Sys<X>& t, int l) { gather.one(t, c, A, xs, e0 + l, e1, L); },
+                            [&](Sys<X>& t, Sys<X>& u, int l) { gather.two(t, u, c, A, xs, e0 + l, e1, L); });
+        if (plane < width) {
+            const auto se = ext_sys(s);
+            ext_solve(se, Xs);
+        }
+    }
+    __syncwarp(team);
+    if (plane >= width) return;
+    unshift(Xs, xs);
+    finish_body(d, b, plane, last, c, A, Xs, [&](int o, const float* cn, const float* An) { store(o, cn, An, width); });
+}
+
+// One sweep of body b from qi to qo in global memory (thread 0 of the body stores): pinned,
+// stopped and held bodies keep their iterate; a body with more than max_ends ends is left to the
+// heavy role.
+template <int L, int P, class X, class Gather>
+__device__ __forceinline__ void solve_body(const Dev& d, int b, int plane, unsigned team,
                                            const float4* __restrict__ qi, float4* __restrict__ qo, int last,
                                            Gather&& gather, int max_ends = HEAVY_ENDS) {
     const int fl = d.bflags[b];
-    if (fl & BF_PINNED) {
-        if (lane == 0) {
+    const int e0 = d.end_off[b], e1 = d.end_off[b + 1];
+    const bool pinned = fl & BF_PINNED, many = !pinned && e1 - e0 > max_ends;
+    const bool still = !pinned && !many && ((d.group_done && d.group_done[d.group[b]]) || held(d, b));
+    team = __ballot_sync(team, !pinned && !many && !still);
+    if (pinned) {
+        if (plane == 0) {
             qo[3 * b] = d.qn[3 * b]; qo[3 * b + 1] = d.qn[3 * b + 1]; qo[3 * b + 2] = d.qn[3 * b + 2];
             if (last) d.resid_body[b] = 0.0;
         }
         return;
     }
-    const int e0 = d.end_off[b], e1 = d.end_off[b + 1];
-    if (e1 - e0 > max_ends) return;  // solved by the heavy role (heavy_role)
-    if ((d.group_done && d.group_done[d.group[b]]) || held(d, b)) {  // stopped (residual threshold) or held
-        if (lane == 0) { qo[3 * b] = qi[3 * b]; qo[3 * b + 1] = qi[3 * b + 1]; qo[3 * b + 2] = qi[3 * b + 2]; }
+    if (many) return;  // solved by the heavy role (heavy_role)
+    if (still) {       // stopped (residual threshold) or held
+        if (plane == 0) { qo[3 * b] = qi[3 * b]; qo[3 * b + 1] = qi[3 * b + 1]; qo[3 * b + 2] = qi[3 * b + 2]; }
         return;
     }
-    float c[3], A[9], sc[3], sA[9];
-    ld_q(qi, b, c, A);
-    ld_q(d.sq, b, sc, sA);
-    float dc[3], dA[9];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) dc[k] = sc[k] - c[k];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) dA[k] = sA[k] - A[k];
-    const float4 mass = d.mass[b];
-    float xs[3];
-    ld_xs(d, b, fl, xs);
-    float Xs[4][3];
-    bool ext = d.p.precision_policy == 3 || (d.p.precision_policy && (fl & BF_FP64));
-    if (!ext) {
-        Sys<float> s;
-        if (lane == 0) sys_init(s, mass, dc, dA, xs);
-        else sys_zero(s);
-        gather(s, c, A, xs, e0, e1);
-        sys_reduce<L>(s, mask);
-        const float ratio = sys_solve(s, Xs);
-        if (d.p.precision_policy && !(ratio >= 1e-3f)) {
-            ext = true;
-            if (last && lane == 0) atomicAdd(&d.ctr[C_FP64DYN], 1);
-        }
-    }
-    if (ext) {
-        Sys<X> s;
-        if (lane == 0) sys_init(s, mass, dc, dA, xs);
-        else sys_zero(s);
-        gather(s, c, A, xs, e0, e1);
-        sys_reduce<L>(s, mask);
-        const auto se = ext_sys(s);
-        ext_solve(se, Xs);
-    }
-    unshift(Xs, xs);
-    finish_body(d, b, lane, qo, last, c, A, Xs);
+    solve_free_body<L, P, X>(d, b, plane, team, fl, e0, e1, last, [&] { return ld_body(d, b, fl); },
+                             [&](int o, float* c, float* A) { ld_q(qi, o, c, A); },
+                             [&](int o, const float* c, const float* A, int) { if (plane == 0) store_iterate(qo, o, c, A); },
+                             gather);
 }
 
-// q^{k+1} from q^k and the solved update X: c + dc, rotation of A + dA; lane 0 stores it and,
-// on the last sweep, the body's squared update and the finiteness check
-__device__ __forceinline__ void finish_body(const Dev& d, int b, int lane, float4* __restrict__ qo, int last,
-                                            const float* c, const float* A, const float (*Xs)[3]) {
+// q^{k+1} from q^k and the solved update X: c + dc, rotation of A + dA; store(b, c, A) takes it,
+// and thread 0 notes, on the last sweep, the body's squared update and the finiteness check
+template <class Store>
+__device__ __forceinline__ void finish_body(const Dev& d, int b, int plane, int last, const float* c, const float* A,
+                                            const float (*Xs)[3], Store&& store) {
     float cn[3], An[9];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -817,8 +929,7 @@ __device__ __forceinline__ void finish_body(const Dev& d, int b, int lane, float
         for (int l = 0; l < 3; ++l) An[3 * k + l] = A[3 * k + l] + Xs[1 + l][k];
     }
     if (d.p.project) polar_rotation(An);
-    if (lane != 0) return;
-    if (last) {  // residual and finiteness of the step's last sweep only
+    if (last && plane == 0) {  // residual and finiteness of the step's last sweep only
         double r2 = 0.0;
         bool finite = true;
 #pragma unroll
@@ -828,89 +939,124 @@ __device__ __forceinline__ void finish_body(const Dev& d, int b, int lane, float
         if (!finite) atomicOr(&d.ctr[C_STATUS], ST_DIVERGED);
         d.resid_body[b] = r2;
     }
-    qo[3 * b] = make_float4(cn[0], cn[1], cn[2], An[0]);
-    qo[3 * b + 1] = make_float4(An[1], An[2], An[3], An[4]);
-    qo[3 * b + 2] = make_float4(An[5], An[6], An[7], An[8]);
+    store(b, cn, An);
 }
 
 // an augmented Lagrangian bond's state is stored by end i, or by end j when i is pinned
-__device__ __forceinline__ bool al_writer(const Dev& d, int4 m, int b) {
-    return (m.z == K_AL) && (m.x == b || (d.bflags[m.x] & BF_PINNED));
+__device__ __forceinline__ bool al_writer(const Dev& d, const EndBond& e) {
+    return e.type == K_AL && (!e.side_j || (d.bflags[e.other] & BF_PINNED));
 }
 
-// accumulate the ends lane, lane + L, ... of body b's CSR slice, in that order: each bond's
-// force in single precision (end_force_q), summed into the system type T.  Two ends per round
-// in FP32: both records and both other bodies' iterates are loaded before either force is
-// evaluated, so a lane waits for two dependent loads per pair of ends.
-template <int L, class T>
-__device__ __forceinline__ void gather_ends(const Dev& d, const float4* __restrict__ q, int b, const float* cb,
-                                            const float* Ab, const float* xs, int e0, int e1, int lane, int it,
-                                            Sys<T>& s) {
-    int p = e0 + lane;
-    // (the extended type keeps one end per round: fewer live registers)
-    if (sizeof(T) == 4) for (; p + L < e1; p += 2 * L) {
-        const int4 m0 = d.rec_m[p], m1 = d.rec_m[p + L];
-        const float4 a0 = d.rec_a[p], b0 = d.rec_b[p], a1 = d.rec_a[p + L], b1 = d.rec_b[p + L];
+// Sums a body's ends from their records: each bond's force in single precision (end_force),
+// summed into the system type T.  `other(e, c, A)` loads the iterate of the other end of e.  In
+// FP32 two ends per round: both records and both other bodies' iterates are loaded before
+// either force is evaluated, so a lane waits for two dependent loads per pair of ends (the
+// extended type keeps one end per round: fewer live registers).
+template <class Other>
+struct EndGather {
+    const Dev& d;
+    const Other& other;
+    int it;
+
+    template <class T>
+    __device__ __forceinline__ void end(Sys<T>& s, const EndBond& e, const float* co, const float* Ao, const float* c,
+                                        const float* A, const float* xs) const {
+        float f[3];
+        const float w = end_force(d, e, co, Ao, c, A, it, al_writer(d, e), f);
+        sys_add_t(s, w, f, e.xs, xs);
+    }
+    // end p to s, and end r to t (s may be t)
+    template <class T>
+    __device__ __forceinline__ void pair(Sys<T>& s, Sys<T>& t, const float* c, const float* A, const float* xs, int p,
+                                         int r) const {
+        const EndBond a = unpack_end(d, d.rec + 3 * (size_t)p), b = unpack_end(d, d.rec + 3 * (size_t)r);
         float c0[3], A0[9], c1[3], A1[9];
-        ld_q_or_zero(q, other_body(m0, b), c0, A0);
-        ld_q_or_zero(q, other_body(m1, b), c1, A1);
-        float f[3];
-        float w = end_force_q(d, c0, A0, b, cb, Ab, m0, a0, b0, it, al_writer(d, m0, b), f);
-        sys_add_t(s, w, f, (m0.y == b) ? b0 : a0, xs);
-        w = end_force_q(d, c1, A1, b, cb, Ab, m1, a1, b1, it, al_writer(d, m1, b), f);
-        sys_add_t(s, w, f, (m1.y == b) ? b1 : a1, xs);
+        other(a, c0, A0);
+        other(b, c1, A1);
+        end(s, a, c0, A0, c, A, xs);
+        end(t, b, c1, A1, c, A, xs);
     }
-    for (; p < e1; p += L) {
-        const int4 m = d.rec_m[p];
-        const float4 xa = d.rec_a[p], xb = d.rec_b[p];
-        float f[3];
-        const float w = end_force(d, q, b, cb, Ab, m, xa, xb, it, al_writer(d, m, b), f);
-        sys_add_t(s, w, f, (m.y == b) ? xb : xa, xs);
+    template <class T>
+    __device__ __forceinline__ void single(Sys<T>& s, const float* c, const float* A, const float* xs, int p) const {
+        const EndBond a = unpack_end(d, d.rec + 3 * (size_t)p);
+        float c0[3], A0[9];
+        other(a, c0, A0);
+        end(s, a, c0, A0, c, A, xs);
     }
+    template <class T>
+    __device__ __forceinline__ void one(Sys<T>& s, const float* c, const float* A, const float* xs, int p, int e1,
+                                        int L) const {
+        if (sizeof(T) == 4) for (; p + L < e1; p += 2 * L) pair(s, s, c, A, xs, p, p + L);
+        for (; p < e1; p += L) single(s, c, A, xs, p);
+    }
+    template <class T>
+    __device__ __forceinline__ void two(Sys<T>& s, Sys<T>& t, const float* c, const float* A, const float* xs, int p,
+                                        int e1, int L) const {
+        if (sizeof(T) != 4) {  // (a lane after the other: the second sum starts once the first is complete)
+            one(s, c, A, xs, p, e1, L);
+            one(t, c, A, xs, p + 1, e1, L);
+            return;
+        }
+        for (; p + 1 < e1; p += L) pair(s, t, c, A, xs, p, p + 1);
+        if (p < e1) single(s, c, A, xs, p);
+    }
+};
+template <class Other>
+__device__ __forceinline__ EndGather<Other> end_gather(const Dev& d, const Other& other, int it) {
+    return EndGather<Other>{d, other, it};
 }
+
+// iterates in global memory, for EndGather
+struct GlobalQ {
+    const float4* __restrict__ q;
+    __device__ __forceinline__ void operator()(const EndBond& e, float* c, float* A) const {
+        ld_other(q, e.other, e.xo, c, A);
+    }
+};
 
 // ---- bodies with many bond ends: one block of HEAVY_T threads per body ----
 
-// Sum the block's partial systems: a xor butterfly inside each warp, then thread 0 adds the
-// warps' sums in warp order (fixed, so the result depends only on HEAVY_T).  `buf` holds one
-// system per warp (as doubles, wide enough for every T).  The total is valid in thread 0.
-template <class T>
-__device__ __forceinline__ void block_reduce(Sys<T>& s, Sys<T>* buf) {
-    sys_reduce<32>(s, 0xffffffffu);
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) buf[w] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < HEAVY_T / 32; ++k) {
-#pragma unroll
-            for (int i = 0; i < 10; ++i) s.g[i] += buf[k].g[i];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) s.r[r][i] += buf[k].r[r][i];
-        }
+// HEAVY_T consecutive threads of a block (whole warps), and how they wait for each other.
+struct HeavyTeam {
+    int t;    // the thread's index in the team
+    int bar;  // the team's barrier: 0 where the block is one team
+    __device__ __forceinline__ void sync() const {
+        asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(HEAVY_T) : "memory");
     }
-    __syncthreads();
+};
+// a team's shared memory: one system per warp (as doubles, wide enough for every type)
+struct HeavyShared {
+    Sys<double> buf[HEAVY_T / 32];
+    int ext;
+};
+
+// Sum the team's partial systems: a xor butterfly inside each warp, then thread 0 adds the
+// warps' sums in warp order (fixed, so the result depends only on HEAVY_T).  The total is
+// valid in thread 0.
+template <class T>
+__device__ __forceinline__ void team_reduce(Sys<T>& s, Sys<T>* buf, HeavyTeam team) {
+    sys_reduce<32>(s, 0xffffffffu);
+    const int w = team.t >> 5;
+    if ((team.t & 31) == 0) buf[w] = s;
+    team.sync();
+    if (team.t == 0) {
+        for (int k = 1; k < HEAVY_T / 32; ++k) sys_plus(s, buf[k]);
+    }
+    team.sync();
 }
 
-// Global + local solve of body b (more than HEAVY_ENDS ends) by the whole block: thread t
-// gathers ends t, t + HEAVY_T, ...; FP32 first, the extended type X where ill-conditioned
-// (same rule as solve_body); thread 0 solves, projects and stores.  Every thread of the block
-// must call it with the same b.
-template <class X, class Gather>
-__device__ __forceinline__ void solve_heavy(const Dev& d, int b, const float4* __restrict__ qi,
-                                            float4* __restrict__ qo, int last, Gather&& gather) {
-    __shared__ Sys<double> buf_raw[HEAVY_T / 32];
-    __shared__ int s_ext;
-    const int t = threadIdx.x;
+// Global + local solve of body b (more than WIDE_ENDS ends) by a whole team: thread t gathers
+// ends t, t + HEAVY_T, ...; FP32 first, the extended type X where ill-conditioned (same rule as
+// solve_free_body); thread 0 solves, projects and stores.  Every thread of the team must call it
+// with the same b.
+template <class X, class Self, class Store, class Gather>
+__device__ __forceinline__ void solve_heavy(const Dev& d, int b, HeavyTeam team, HeavyShared& sh, int last,
+                                            Self&& self, Store&& store, Gather&& gather) {
+    const int t = team.t;
     const int fl = d.bflags[b];
-    if ((d.group_done && d.group_done[d.group[b]]) || held(d, b)) {  // stopped (residual threshold) or held
-        if (t == 0) { qo[3 * b] = qi[3 * b]; qo[3 * b + 1] = qi[3 * b + 1]; qo[3 * b + 2] = qi[3 * b + 2]; }
-        return;
-    }
     const int e0 = d.end_off[b], e1 = d.end_off[b + 1];
     float c[3], A[9], sc[3], sA[9];
-    ld_q(qi, b, c, A);
+    self(b, c, A);
     ld_q(d.sq, b, sc, sA);
     float dc[3], dA[9];
 #pragma unroll
@@ -921,29 +1067,29 @@ __device__ __forceinline__ void solve_heavy(const Dev& d, int b, const float4* _
     float xs[3];
     ld_xs(d, b, fl, xs);
     float Xs[4][3];
-    if (t == 0) s_ext = d.p.precision_policy == 3 || (d.p.precision_policy && (fl & BF_FP64));
-    __syncthreads();
-    if (!s_ext) {
+    if (t == 0) sh.ext = d.p.precision_policy == 3 || (d.p.precision_policy && (fl & BF_FP64));
+    team.sync();
+    if (!sh.ext) {
         Sys<float> s;
         if (t == 0) sys_init(s, mass, dc, dA, xs);
         else sys_zero(s);
-        gather(s, c, A, xs, e0, e1);
-        block_reduce(s, reinterpret_cast<Sys<float>*>(buf_raw));
+        gather.one(s, c, A, xs, e0 + t, e1, HEAVY_T);
+        team_reduce(s, reinterpret_cast<Sys<float>*>(sh.buf), team);
         if (t == 0) {
             const float ratio = sys_solve(s, Xs);
             if (d.p.precision_policy && !(ratio >= 1e-3f)) {
-                s_ext = 1;
+                sh.ext = 1;
                 if (last) atomicAdd(&d.ctr[C_FP64DYN], 1);
             }
         }
-        __syncthreads();
+        team.sync();
     }
-    if (s_ext) {
+    if (sh.ext) {
         Sys<X> s;
         if (t == 0) sys_init(s, mass, dc, dA, xs);
         else sys_zero(s);
-        gather(s, c, A, xs, e0, e1);
-        block_reduce(s, reinterpret_cast<Sys<X>*>(buf_raw));
+        gather.one(s, c, A, xs, e0 + t, e1, HEAVY_T);
+        team_reduce(s, reinterpret_cast<Sys<X>*>(sh.buf), team);
         if (t == 0) {
             const auto se = ext_sys(s);
             ext_solve(se, Xs);
@@ -951,36 +1097,36 @@ __device__ __forceinline__ void solve_heavy(const Dev& d, int b, const float4* _
     }
     if (t == 0) {
         unshift(Xs, xs);
-        finish_body(d, b, 0, qo, last, c, A, Xs);
+        finish_body(d, b, 0, last, c, A, Xs, store);
     }
-    __syncthreads();  // the shared buffers are reused by the block's next body
+    team.sync();  // the shared memory is reused by the team's next body
 }
 
 // The heavy role of a sweep launch's extra blocks (HEAVY_T threads each, block index hb of
 // HEAVY_BLOCKS): the bodies on the heavy list with up to WIDE_ENDS ends, one warp each
-// (32-lane butterfly, gather_w), then those with more, one block each (gather_b).  The
-// summation order depends only on the body's end count, never on which block runs it.
-template <class X, class GatherW, class GatherB>
+// (32-lane butterfly), then those with more, one block each.  The summation order depends only
+// on the body's end count, never on which block runs it.
+template <class X, class Gather>
 __device__ __forceinline__ void heavy_role(const Dev& d, int hb, const float4* __restrict__ qi,
-                                           float4* __restrict__ qo, int last, GatherW&& gather_w,
-                                           GatherB&& gather_b) {
+                                           float4* __restrict__ qo, int last, Gather&& gather) {
+    __shared__ HeavyShared sh;
+    const HeavyTeam team{(int)threadIdx.x, 0};
     const int nheavy = d.ctr[C_NHEAVY];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int h = hb * (HEAVY_T / 32) + warp; h < nheavy; h += HEAVY_BLOCKS * (HEAVY_T / 32)) {
         const int b = d.heavy[h];
         if (d.end_off[b + 1] - d.end_off[b] > WIDE_ENDS) continue;
-        solve_body<32, X>(d, b, lane, 0xffffffffu, qi, qo, last,
-                          [&](auto& s, const float* c, const float* A, const float* xs, int e0, int e1) {
-                              gather_w(b, s, c, A, xs, e0, e1, lane);
-                          },
-                          WIDE_ENDS);
+        solve_body<32, 32, X>(d, b, lane, 0xffffffffu, qi, qo, last, gather, WIDE_ENDS);
     }
     for (int h = hb; h < nheavy; h += HEAVY_BLOCKS) {
         const int b = d.heavy[h];
         if (d.end_off[b + 1] - d.end_off[b] <= WIDE_ENDS) continue;
-        solve_heavy<X>(d, b, qi, qo, last, [&](auto& s, const float* c, const float* A, const float* xs, int e0, int e1) {
-            gather_b(b, s, c, A, xs, e0, e1, (int)threadIdx.x);
-        });
+        if ((d.group_done && d.group_done[d.group[b]]) || held(d, b)) {  // stopped (residual threshold) or held
+            if (team.t == 0) { qo[3 * b] = qi[3 * b]; qo[3 * b + 1] = qi[3 * b + 1]; qo[3 * b + 2] = qi[3 * b + 2]; }
+            continue;
+        }
+        solve_heavy<X>(d, b, team, sh, last, [&](int o, float* c, float* A) { ld_q(qi, o, c, A); },
+                       [&](int o, const float* c, const float* A) { store_iterate(qo, o, c, A); }, gather);
     }
 }
 
