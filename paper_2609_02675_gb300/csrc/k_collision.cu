@@ -106,6 +106,19 @@ __device__ __forceinline__ void aabb_body(const Dev& d, int b) {
         const int m = __reduce_max_sync(act, lv == l ? bits : 0);
         if (leader && m > 0) atomicMax(&d.ctr[l == 0 ? C_CELLBITS : C_CELLBITS1 + l - 1], m);
     }
+    if (d.bvh_bounds) {  // LBVH: the box of the finite centres, as order-preserving ints
+        const float x[3] = {0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2])};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int i = __float_as_int(x[k]), o = i >= 0 ? i : i ^ 0x7fffffff;
+            const bool fin = isfinite(x[k]);
+            const int mn = __reduce_min_sync(act, fin ? o : 0x7fffffff), mx = __reduce_max_sync(act, fin ? o : (int)0x80000000);
+            if (leader) {
+                atomicMin(&d.bvh_bounds[k], mn);
+                atomicMax(&d.bvh_bounds[3 + k], mx);
+            }
+        }
+    }
     d.cell[b] = make_int4(0, 0, 0, large ? -1 : 0);
     if (d.blevel) d.blevel[b] = large ? -1 : lv;
     if (large && d.large_ids) d.large_ids[atomicAdd(&d.ctr[C_NLARGE], 1)] = b;

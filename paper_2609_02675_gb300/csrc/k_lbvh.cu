@@ -4,57 +4,38 @@
 //   1. scene box of the bodies' box centres (min / max over order-preserving int bits: exact
 //      and order-independent);
 //   2. 30-bit Morton code of every centre (10 bits per axis over the scene box);
-//   3. stable LSD radix sort of (code, body) -- 8-bit digits, tiles of 1024 keys per warp,
-//      per-(digit, tile) counts, their prefix sums, and a stable scatter that ranks equal
-//      digits within a tile with warp match masks, so the order is deterministic;
+//   3. stable LSD radix sort of (code, body) -- 8-bit digits, tiles of 1024 keys, a block of
+//      1024 threads each: per-(digit, tile) counts (taken by the pass before), their prefix sums,
+//      and a stable scatter that ranks equal digits by warp match masks and the warps' counts, so
+//      the order is deterministic;
 //   4. the binary radix tree over the sorted codes by Karras' construction ("Maximizing
 //      parallelism in the construction of BVHs, octrees, and k-d trees", HPG 2012): each
 //      internal node finds its range and split from the longest common prefixes (equal codes
 //      broken by leaf index);
-//   5. bottom-up refit of the internal nodes' boxes (the second child to arrive merges);
+//   5. bottom-up refit (the second child to arrive merges): an internal node is one 64-byte
+//      record of both children's boxes, their ids and the largest body id below each;
 //   6. every body i walks the tree for the leaves j > i its box overlaps that the pair filter
-//      accepts: a counting walk, prefix sums, a writing walk, then each body's partner slice
-//      sorted (warp or block).  The list is the sorted set of overlapping pairs: the same
-//      pairs, bit for bit, as the grid hash's.
+//      accepts, the bodies in leaf order so that a warp's walks stay together: a counting walk
+//      that keeps the first partners it finds, prefix sums, a write that replays them (or walks
+//      again where a body has more), then each body's partner slice sorted (warp or block).
+//      The list is the sorted set of overlapping pairs: the same pairs, bit for bit, as the grid
+//      hash's.
+//
+// Bound by the latency of its dependent steps: 20 011 boxes leave four warps per SM.  One node
+// record per visit (one dependent load instead of three), leaf order, subtrees without a larger
+// id skipped, the replayed write and 1024-thread tiles (a tile of 1024 keys was one warp's, 32
+// steps in series) took its collision stage from 387 to 156 us.
 #include "pair_filter.cuh"
 #include "sort_slices.cuh"
 
 namespace pabd {
 
 constexpr int BT = 256;        // threads per block for per-body / per-node kernels
-constexpr int RX_TILE = 1024;  // keys per radix tile (one warp)
+constexpr int RX_TILE = 1024;  // keys per radix tile (a block, one thread each)
 
 static inline int bblk(long long n) { return (int)((n + BT - 1) / BT > 0 ? (n + BT - 1) / BT : 1); }
 
-__device__ __forceinline__ int f2o(float f) {
-    const int i = __float_as_int(f);
-    return i >= 0 ? i : i ^ 0x7fffffff;
-}
 __device__ __forceinline__ float o2f(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
-
-__global__ void k_bvh_init(Dev d) {
-    if (threadIdx.x < 3) {
-        d.bvh_bounds[threadIdx.x] = 0x7fffffff;
-        d.bvh_bounds[3 + threadIdx.x] = (int)0x80000000;
-    }
-    if (threadIdx.x == 0) {
-        d.bvh_parent[0] = -1;
-        d.ctr[C_NPHEAVY] = 0;
-    }
-}
-
-__global__ void k_bvh_bounds(Dev d) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= d.N) return;
-    const float4 lo = d.lo[b], hi = d.hi[b];
-    const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        if (!isfinite(c[k])) continue;
-        atomicMin(&d.bvh_bounds[k], f2o(c[k]));
-        atomicMax(&d.bvh_bounds[3 + k], f2o(c[k]));
-    }
-}
 
 // spread the low 10 bits of v to every third bit
 __device__ __forceinline__ unsigned spread3(unsigned v) {
@@ -66,63 +47,83 @@ __device__ __forceinline__ unsigned spread3(unsigned v) {
     return v;
 }
 
-__global__ void k_bvh_morton(Dev d) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= d.N) return;
-    const float4 lo = d.lo[b], hi = d.hi[b];
-    const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-    unsigned q[3];
-    bool finite = true;
+// per tile of 1024 bodies: their codes, the counts of the first digit, and the scratch of the
+// passes that follow zeroed (the second digit's counts, the refit's arrivals)
+__global__ void __launch_bounds__(RX_TILE) k_bvh_morton(Dev d, int ntile) {
+    pdl_enter();
+    __shared__ int c[256];
+    const int tile = blockIdx.x, t = threadIdx.x;
+    if (t < 256) c[t] = 0;
+    __syncthreads();
+    const int b = tile * RX_TILE + t;
+    if (b == 0) d.bvh_parent[0] = -1;
+    if (b < d.N - 1) d.bvh_visit[b] = 0;
+    if (b < d.N) {
+        const float4 lo = d.lo[b], hi = d.hi[b];
+        const float x[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
+        unsigned q[3];
+        bool finite = true;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float b0 = o2f(d.bvh_bounds[k]), b1 = o2f(d.bvh_bounds[3 + k]);
-        const float ext = b1 - b0;
-        float u = ext > 0.f ? (c[k] - b0) / ext : 0.f;
-        finite = finite && isfinite(u);
-        u = fminf(fmaxf(u, 0.f), 1.f);
-        q[k] = min((unsigned)(u * 1024.f), 1023u);
+        for (int k = 0; k < 3; ++k) {
+            const float b0 = o2f(d.bvh_bounds[k]), b1 = o2f(d.bvh_bounds[3 + k]);
+            const float ext = b1 - b0;
+            float u = ext > 0.f ? (x[k] - b0) / ext : 0.f;
+            finite = finite && isfinite(u);
+            u = fminf(fmaxf(u, 0.f), 1.f);
+            q[k] = min((unsigned)(u * 1024.f), 1023u);
+        }
+        const unsigned key = finite ? (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]) : 0xffffffffu;
+        d.bvh_key[b] = key;
+        d.bvh_id[b] = b;
+        atomicAdd(&c[key & 255u], 1);
     }
-    d.bvh_key[b] = finite ? (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]) : 0xffffffffu;
-    d.bvh_id[b] = b;
+    __syncthreads();
+    if (t < 256) {
+        d.rx_cnt[t * ntile + tile] = c[t];
+        d.rx_cnt2[t * ntile + tile] = 0;
+    }
 }
 
 // ---- stable radix sort of (key, id), 8 bits per pass ----
 
-__global__ void k_rx_count(const unsigned* __restrict__ key, int n, int shift, int ntile, int* __restrict__ cnt) {
-    __shared__ int c[256];
-    const int tile = blockIdx.x, lane = threadIdx.x;
-    for (int k = lane; k < 256; k += 32) c[k] = 0;
-    __syncwarp();
-    for (int step = 0; step < RX_TILE / 32; ++step) {
-        const int idx = tile * RX_TILE + step * 32 + lane;
-        if (idx < n) atomicAdd(&c[(key[idx] >> shift) & 255u], 1);
-    }
-    __syncwarp();
-    for (int k = lane; k < 256; k += 32) cnt[k * ntile + tile] = c[k];
-}
-
-__global__ void k_rx_scatter(const unsigned* __restrict__ key_in, const int* __restrict__ id_in,
-                             unsigned* __restrict__ key_out, int* __restrict__ id_out, int n, int shift,
-                             int ntile, const int* __restrict__ off) {
-    __shared__ int base[256];
-    const int tile = blockIdx.x, lane = threadIdx.x;
-    for (int k = lane; k < 256; k += 32) base[k] = off[k * ntile + tile];
-    __syncwarp();
-    const unsigned below = (1u << lane) - 1u;
-    for (int step = 0; step < RX_TILE / 32; ++step) {
-        const int idx = tile * RX_TILE + step * 32 + lane;
-        const bool valid = idx < n;
-        const unsigned k = valid ? key_in[idx] : 0u;
-        const int digit = valid ? (int)((k >> shift) & 255u) : 256 + lane;  // unmatched if invalid
-        const unsigned peers = __match_any_sync(0xffffffffu, digit);
-        if (valid) {
-            const int dst = base[digit] + __popc(peers & below);
-            key_out[dst] = k;
-            id_out[dst] = id_in[idx];
+// One pass over a tile: each key's rank among the tile's equal digits is its rank in its warp
+// plus the equal digits of the warps before; the tile's first place for a digit comes from the
+// scanned counts.  The next pass's digit is counted at the key's destination (cnt_next), and
+// this pass's counts, already scanned, are zeroed for the pass after.
+__global__ void __launch_bounds__(RX_TILE) k_rx_scatter(const unsigned* key_in, const int* id_in, unsigned* key_out,
+                                                        int* id_out, int n, int shift, int ntile, const int* off,
+                                                        int* cnt, int* cnt_next) {
+    pdl_enter();
+    constexpr int NW = RX_TILE / 32;
+    __shared__ unsigned short wc[NW][256];
+    const int tile = blockIdx.x, t = threadIdx.x, w = t >> 5, lane = t & 31;
+    for (int k = t; k < NW * 256 / 2; k += RX_TILE) reinterpret_cast<unsigned*>(wc)[k] = 0;
+    __syncthreads();
+    const int idx = tile * RX_TILE + t;
+    const bool valid = idx < n;
+    const unsigned k = valid ? key_in[idx] : 0u;
+    const int id = valid ? id_in[idx] : 0;
+    const int digit = valid ? (int)((k >> shift) & 255u) : 256 + lane;  // unmatched if invalid
+    const unsigned peers = __match_any_sync(0xffffffffu, digit);
+    const int rank = __popc(peers & ((1u << lane) - 1u));
+    if (valid && rank == 0) wc[w][digit] = (unsigned short)__popc(peers);
+    __syncthreads();
+    if (t < 256) {
+        int run = 0;
+#pragma unroll 8
+        for (int v = 0; v < NW; ++v) {
+            const int c = wc[v][t];
+            wc[v][t] = (unsigned short)run;
+            run += c;
         }
-        __syncwarp();
-        if (valid && (peers & below) == 0) base[digit] += __popc(peers);  // the group's first lane
-        __syncwarp();
+        cnt[t * ntile + tile] = 0;
+    }
+    __syncthreads();
+    if (valid) {
+        const int dst = off[digit * ntile + tile] + wc[w][digit] + rank;
+        key_out[dst] = k;
+        id_out[dst] = id;
+        if (cnt_next) atomicAdd(&cnt_next[((k >> (shift + 8)) & 255u) * ntile + dst / RX_TILE], 1);
     }
 }
 
@@ -135,6 +136,7 @@ __device__ __forceinline__ int prefix(const unsigned* __restrict__ key, int n, i
 }
 
 __global__ void k_bvh_build(Dev d) {
+    pdl_enter();
     const int n = d.N;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
@@ -162,20 +164,29 @@ __global__ void k_bvh_build(Dev d) {
     d.bvh_parent[right] = i;
 }
 
-// the box of node c (a leaf: its body's inflated box)
+// An internal node's record (Dev::bvh_node, four float4): (lo, id) and (hi, largest body id) of
+// the left child, then of the right.  A leaf's id is n - 1 + its place; its largest body id is
+// its body.
+
+// the box of node c and the largest body id below it
 __device__ __forceinline__ void node_box(const Dev& d, int c, float4& lo, float4& hi) {
     const int n = d.N;
     if (c >= n - 1) {
         const int b = d.bvh_id[c - (n - 1)];
         lo = d.lo[b];
         hi = d.hi[b];
+        hi.w = __int_as_float(b);
     } else {
-        lo = __ldcg(&d.bvh_lo[c]);
-        hi = __ldcg(&d.bvh_hi[c]);
+        const float4* r = d.bvh_node + 4 * (size_t)c;
+        const float4 al = __ldcg(r), ah = __ldcg(r + 1), bl = __ldcg(r + 2), bh = __ldcg(r + 3);
+        lo = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.f);
+        hi = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z),
+                         __int_as_float(max(__float_as_int(ah.w), __float_as_int(bh.w))));
     }
 }
 
 __global__ void k_bvh_refit(Dev d) {
+    pdl_enter();
     const int n = d.N;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n || n < 2) return;
@@ -188,8 +199,13 @@ __global__ void k_bvh_refit(Dev d) {
         float4 al, ah, bl, bh;
         node_box(d, ch.x, al, ah);
         node_box(d, ch.y, bl, bh);
-        __stcg(&d.bvh_lo[node], make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.f));
-        __stcg(&d.bvh_hi[node], make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z), 0.f));
+        al.w = __int_as_float(ch.x);
+        bl.w = __int_as_float(ch.y);
+        float4* r = d.bvh_node + 4 * (size_t)node;
+        __stcg(r, al);
+        __stcg(r + 1, ah);
+        __stcg(r + 2, bl);
+        __stcg(r + 3, bh);
         node = d.bvh_parent[node];
     }
 }
@@ -203,39 +219,62 @@ __device__ __forceinline__ int bvh_partners(const Dev& d, int i, F&& f) {
     const int gi = d.group[i], fi = d.bflags[i];
     int stack[64];
     int sp = 0, cnt = 0;
-    stack[sp++] = 0;
-    while (sp > 0) {
-        const int node = stack[--sp];
-        const int2 ch = d.bvh_kids[node];
-        const int kid[2] = {ch.x, ch.y};
+    int node = 0;
+    for (;;) {
+        const float4* r = d.bvh_node + 4 * (size_t)node;
+        const float4 box[4] = {r[0], r[1], r[2], r[3]};
+        int next = -1;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            if (kid[c] >= n - 1) {
-                const int j = d.bvh_id[kid[c] - (n - 1)];
-                if (j > i && pair_ok(d, i, j, gi, fi)) { f(j, cnt); ++cnt; }
-            } else if (overlap(li, hi, d.bvh_lo[kid[c]], d.bvh_hi[kid[c]])) {
-                if (sp < 64) stack[sp++] = kid[c];
-                else atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);  // deeper than any tree of 30-bit codes
+            const int kid = __float_as_int(box[2 * c].w), top = __float_as_int(box[2 * c + 1].w);
+            if (top <= i || !overlap(li, hi, box[2 * c], box[2 * c + 1])) continue;
+            if (kid >= n - 1) {  // the leaf of body `top`, whose box is the one just tested
+                if (d.group[top] != gi || ((fi & BF_PINNED) && (d.bflags[top] & BF_PINNED)) || adj_has(d, i, top)) continue;
+                f(top, cnt);
+                ++cnt;
+            } else if (next < 0) {
+                next = kid;
+            } else if (sp < 64) {
+                stack[sp++] = kid;
+            } else {
+                atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);  // deeper than any tree of 30-bit codes
             }
         }
+        if (next < 0) {
+            if (sp == 0) return cnt;
+            next = stack[--sp];
+        }
+        node = next;
     }
-    return cnt;
 }
 
+// counts the partners of the bodies in leaf order, keeping the first BVH_STASH of each (slot k of
+// body i at k N + i)
 __global__ void k_bvh_pair_count(Dev d) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d.N) return;
-    d.pair_cnt[i] = bvh_partners(d, i, [](int, int) {});
+    pdl_enter();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= d.N) return;
+    const int i = d.bvh_id[k];
+    d.pair_cnt[i] = bvh_partners(d, i, [&](int j, int c) {
+        if (c < BVH_STASH) d.bvh_stash[(size_t)c * d.N + i] = j;
+    });
 }
 
 __global__ void k_bvh_pair_write(Dev d) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d.N) return;
-    const int s = d.pair_off[i], cap = d.cap_pairs;
-    bvh_partners(d, i, [&](int j, int k) {
-        if (s + k < cap) d.pair_j[s + k] = j;
-    });
-    if (i == d.N - 1) {
+    pdl_enter();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= d.N) return;
+    const int i = d.bvh_id[k];
+    const int s = d.pair_off[i], n = d.pair_off[i + 1] - s, cap = d.cap_pairs;
+    if (n <= BVH_STASH) {
+        for (int c = 0; c < n; ++c)
+            if (s + c < cap) d.pair_j[s + c] = d.bvh_stash[(size_t)c * d.N + i];
+    } else {
+        bvh_partners(d, i, [&](int j, int c) {
+            if (s + c < cap) d.pair_j[s + c] = j;
+        });
+    }
+    if (k == d.N - 1) {
         const int tot = d.pair_off[d.N];
         if (tot > cap) atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);
         d.ctr[C_NPAIRS] = min(tot, cap);
@@ -283,33 +322,32 @@ void launch_pair_sort(const Dev& d, cudaStream_t st, long long* launches) {
     *launches += 2;
 }
 
+// (the bounds of the centres are zeroed by launch_step_reset and taken by k_aabb)
 void launch_lbvh_pairs(const Dev& d, cudaStream_t st, long long* launches) {
     const int n = d.N;
-    k_bvh_init<<<1, 32, 0, st>>>(d);
-    k_bvh_bounds<<<bblk(n), BT, 0, st>>>(d);
-    k_bvh_morton<<<bblk(n), BT, 0, st>>>(d);
-    *launches += 3;
     const int ntile = (n + RX_TILE - 1) / RX_TILE > 0 ? (n + RX_TILE - 1) / RX_TILE : 1;
+    launch_pdl(k_bvh_morton, dim3(ntile), dim3(RX_TILE), 0, st, d, ntile);
     unsigned* ka = d.bvh_key;
     unsigned* kb = d.bvh_key2;
     int* ia = d.bvh_id;
     int* ib = d.bvh_id2;
+    int* ca_ = d.rx_cnt;
+    int* cb = d.rx_cnt2;
     for (int shift = 0; shift < 32; shift += 8) {
-        k_rx_count<<<ntile, 32, 0, st>>>(ka, n, shift, ntile, d.rx_cnt);
-        scan_exclusive(d.rx_cnt, d.rx_off, nullptr, 256 * ntile, d.scan_scratch, st, launches);
-        k_rx_scatter<<<ntile, 32, 0, st>>>(ka, ia, kb, ib, n, shift, ntile, d.rx_off);
-        *launches += 2;
+        scan_exclusive(ca_, d.rx_off, nullptr, 256 * ntile, d.scan_scratch, st, launches);
+        launch_pdl(k_rx_scatter, dim3(ntile), dim3(RX_TILE), 0, st, ka, ia, kb, ib, n, shift, ntile, d.rx_off, ca_,
+                   shift < 24 ? cb : (int*)nullptr);
         unsigned* tk = ka; ka = kb; kb = tk;
         int* ti = ia; ia = ib; ib = ti;
+        int* tc = ca_; ca_ = cb; cb = tc;
     }
     // four passes: the sorted keys and ids are back in bvh_key / bvh_id
-    cudaMemsetAsync(d.bvh_visit, 0, sizeof(int) * (n > 1 ? n - 1 : 1), st);
-    k_bvh_build<<<bblk(n - 1), BT, 0, st>>>(d);
-    k_bvh_refit<<<bblk(n), BT, 0, st>>>(d);
-    k_bvh_pair_count<<<bblk(n), BT, 0, st>>>(d);
+    launch_pdl(k_bvh_build, dim3(bblk(n - 1)), dim3(BT), 0, st, d);
+    launch_pdl(k_bvh_refit, dim3(bblk(n)), dim3(BT), 0, st, d);
+    launch_pdl(k_bvh_pair_count, dim3((n + 63) / 64 > 0 ? (n + 63) / 64 : 1), dim3(64), 0, st, d);
     scan_exclusive(d.pair_cnt, d.pair_off, nullptr, n, d.scan_scratch, st, launches);
-    k_bvh_pair_write<<<bblk(n), BT, 0, st>>>(d);
-    *launches += 4;
+    launch_pdl(k_bvh_pair_write, dim3(bblk(n)), dim3(BT), 0, st, d);
+    *launches += 9;
     launch_pair_sort(d, st, launches);
 }
 

@@ -375,6 +375,7 @@ __global__ void k_step_reset(Dev d) {
         d.ctr[C_FP64DYN] = 0;
         for (int k = C_NPHEAVY; k < C_COUNT; ++k) d.ctr[k] = 0;
     }
+    if (d.bvh_bounds && t < 6) d.bvh_bounds[t] = t < 3 ? 0x7fffffff : (int)0x80000000;
     if (d.p.broadphase == 0 && t < (1 << d.table_bits)) {
         d.bucket_cnt[t] = 0;
         d.bucket_cur[t] = 0;

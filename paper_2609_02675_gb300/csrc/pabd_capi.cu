@@ -825,9 +825,9 @@ pabd_status finalize_scene(pabd_scene* s) {
     if (p.broadphase == 1) {
         const size_t ntile = ((size_t)N + 1023) / 1024 + 1;
         ok &= alloc_arr(s, d.bvh_key, N) && alloc_arr(s, d.bvh_key2, N) && alloc_arr(s, d.bvh_id, N) &&
-              alloc_arr(s, d.bvh_id2, N) && alloc_arr(s, d.rx_cnt, 256 * ntile) && alloc_arr(s, d.rx_off, 256 * ntile + 1);
-        ok &= alloc_arr(s, d.bvh_kids, N) && alloc_arr(s, d.bvh_parent, 2 * (size_t)N) && alloc_arr(s, d.bvh_lo, N) &&
-              alloc_arr(s, d.bvh_hi, N) && alloc_arr(s, d.bvh_visit, N) && alloc_arr(s, d.bvh_bounds, 6);
+              alloc_arr(s, d.bvh_id2, N) && alloc_arr(s, d.rx_cnt, 256 * ntile) && alloc_arr(s, d.rx_cnt2, 256 * ntile) && alloc_arr(s, d.rx_off, 256 * ntile + 1);
+        ok &= alloc_arr(s, d.bvh_kids, N) && alloc_arr(s, d.bvh_parent, 2 * (size_t)N) && alloc_arr(s, d.bvh_node, 4 * (size_t)N) &&
+              alloc_arr(s, d.bvh_stash, (size_t)BVH_STASH * N) && alloc_arr(s, d.bvh_visit, N) && alloc_arr(s, d.bvh_bounds, 6);
     }
     if (p.broadphase == 1 || d.multilevel) {
         ok &= alloc_arr(s, d.pair_j, d.cap_pairs) && alloc_arr(s, d.pair_tmp, d.cap_pairs) &&

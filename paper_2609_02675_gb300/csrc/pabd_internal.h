@@ -74,6 +74,7 @@ constexpr int END_BINS = HEAVY_ENDS + 1;
 constexpr int RES_CHUNK = 4096;
 constexpr int PAIR_STASH = 4;
 constexpr int STASH_DELIVER = 0x40000000;
+constexpr int BVH_STASH = 16;
 
 struct Dev {
     Params p;
@@ -146,10 +147,11 @@ struct Dev {
     // linear BVH broad phase (Params::broadphase == 1)
     unsigned *bvh_key, *bvh_key2;   // Morton codes (radix sort ping-pong)
     int *bvh_id, *bvh_id2;          // body ids in Morton order
-    int *rx_cnt, *rx_off;           // radix sort: counts per (digit, tile) and their prefix sums
+    int *rx_cnt, *rx_cnt2, *rx_off; // radix sort: counts per (digit, tile) of this pass and the next, prefix sums
     int2 *bvh_kids;                 // children of the internal nodes (leaf k is node N - 1 + k)
     int *bvh_parent;                // parent of every node (-1 at the root)
-    float4 *bvh_lo, *bvh_hi;        // boxes of the internal nodes
+    float4 *bvh_node;               // 4 float4 per internal node: its children's boxes and ids
+    int *bvh_stash;                 // the first BVH_STASH partners each body's counting walk found
     int *bvh_visit;                 // refit arrivals per internal node
     int *bvh_bounds;                // box of the centres (order-preserving int bits: min xyz, max xyz)
     int *pair_j, *pair_tmp;         // partner slices while they are sorted
