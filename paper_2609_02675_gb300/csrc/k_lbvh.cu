@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(LONG_T) k_pair_sort_long(Dev d) {
     for (int h = blockIdx.x; h < nh; h += gridDim.x) {
         const int i = d.pair_heavy[h];
         const int s = min(d.pair_off[i], cap), e = min(d.pair_off[i + 1], cap);
-        block_sort_slice(d.pair_j + s, e - s, d.pair_tmp + s, key);
+        block_sort_slice<LONG_T>(d.pair_j + s, e - s, d.pair_tmp + s, key);
         for (int p = s + threadIdx.x; p < e; p += LONG_T) d.pairs[p] = make_int2(i, d.pair_j[p]);
         __syncthreads();
     }

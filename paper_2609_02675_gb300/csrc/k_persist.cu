@@ -77,16 +77,6 @@ __global__ void __launch_bounds__(HEAVY_T, 4) k_sweep_fused(Dev d) {
     }
 }
 
-// copy of every bond end's record into CSR order (once per step, after the CSR sort)
-__global__ void k_end_records(Dev d) {
-    pdl_enter();
-    const int ne = d.end_off[d.N];
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < ne; p += gridDim.x * blockDim.x) {
-        const int id = d.end_id[p], bond = id >> 1;
-        pack_end(d.rec + 3 * (size_t)p, bond, d.bmeta[bond], d.bxi[bond], d.bxj[bond], d.bn[bond], id & 1);
-    }
-}
-
 using FusedFn = void (*)(Dev);
 
 static FusedFn fused_fn(int L, bool fp64) {
@@ -116,14 +106,7 @@ int fused_max_blocks(int L, int block, bool fp64) {
     return per_sm * sms;
 }
 
-void launch_end_records(const Dev& d, cudaStream_t st, long long* launches) {
-    const int nrec = d.cap_ends > 0 ? d.cap_ends : 1;
-    launch_pdl(k_end_records, dim3(stride_grid(nrec, 256)), dim3(256), 0, st, d);
-    *launches += 1;
-}
-
 cudaError_t launch_fused_sweep(const Dev& d, int L, int block, int grid, cudaStream_t st, long long* launches) {
-    launch_end_records(d, st, launches);
     // a barrier that gave up in an earlier launch leaves its arrivals counted: start clean
     cudaMemsetAsync(d.gbar, 0, 2 * sizeof(unsigned), st);
     Dev dd = d;

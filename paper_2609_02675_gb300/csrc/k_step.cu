@@ -1,8 +1,8 @@
 // Per-step kernels around the sweep: the predictor and the velocity recovery of Alg. 1,
 // the time-dependent drive anchors, the CSR of bond ends and the per-group residual.
+#include "csr.cuh"
 #include "pabd_internal.h"
 #include "predict.cuh"
-#include "sort_slices.cuh"
 
 namespace pabd {
 
@@ -85,76 +85,33 @@ __global__ void k_finalize(Dev d, const float4* __restrict__ qf, int dyn) {
     finalize_body(d, b, qf);
 }
 
-// Drive anchors at t = (step + 1) h: x_i = x_i0 + arm (cos th r + sin th (u x r)),
-// th = amp sin(2 pi t / period + phase).
 __global__ void k_drive_update(Dev d) {
     pdl_enter();
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= d.Ndrive) return;
-    const double t = (double)(*d.step_index + 1) * d.p.h_d;
-    float4 a = d.drv[3 * k], r = d.drv[3 * k + 1], ur = d.drv[3 * k + 2];
-    float2 pp = d.drv_t[k];
-    const float th = r.w * sinf((float)(6.283185307179586 * t / (double)pp.x) + pp.y);
-    float cs, sn;
-    sincosf(th, &sn, &cs);
-    const int bi = d.drv_bond[k];
-    float4 cur = d.bxi[bi];
-    d.bxi[bi] = make_float4(a.x + a.w * (cs * r.x + sn * ur.x), a.y + a.w * (cs * r.y + sn * ur.y),
-                            a.z + a.w * (cs * r.z + sn * ur.z), cur.w);
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < d.Ndrive) drive_update(d, k);
 }
 
-// ---- CSR of bond ends: ends of dynamic bodies, sorted by (body, 2 * bond + side) ----
-
-__device__ __forceinline__ bool end_live(const Dev& d, int body) {
-    return body >= 0 && !(d.bflags[body] & BF_PINNED);
-}
+// ---- CSR of bond ends (csr.cuh) ----
 
 // (both stride over this step's bonds, C_NBONDS of them)
 __global__ void k_csr_count(Dev d) {
     pdl_enter();
     const int nb = d.ctr[C_NBONDS];
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
-        int4 m = d.bmeta[b];
-        if (end_live(d, m.x)) atomicAdd(&d.end_cnt[m.x], 1);
-        if (end_live(d, m.y)) atomicAdd(&d.end_cnt[m.y], 1);
-    }
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) csr_count_bond(d, b);
 }
 
 __global__ void k_csr_fill(Dev d) {
     pdl_enter();
     const int nb = d.ctr[C_NBONDS];
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
-        int4 m = d.bmeta[b];
-        if (end_live(d, m.x)) d.end_id[d.end_off[m.x] + atomicAdd(&d.end_cur[m.x], 1)] = 2 * b;
-        else d.end_pos[2 * b] = -1;
-        if (end_live(d, m.y)) d.end_id[d.end_off[m.y] + atomicAdd(&d.end_cur[m.y], 1)] = 2 * b + 1;
-        else d.end_pos[2 * b + 1] = -1;
-    }
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) csr_fill_bond(d, b);
 }
 
-// Sort each body's slice of end ids (one warp per body), then record every end's slot and
-// material point.  Slices of up to HEAVY_ENDS (64) ends are sorted in registers by a bitonic
-// network (element k sits in lane k / 2, slot k % 2; padding is INT_MAX); a longer slice's
-// body goes on the heavy list, whose slices k_csr_sort_long sorts.  Either way the slice ends
-// up in ascending end id.
+// CSR_LANES lanes per body
+template <int WANT>
 __global__ void k_csr_sort(Dev d) {
     pdl_enter();
-    const int body = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (body >= d.N) return;
-    const int s = d.end_off[body], e = d.end_off[body + 1], n = e - s;
-    if (n > HEAVY_ENDS) {
-        if (lane == 0) d.heavy[atomicAdd(&d.ctr[C_NHEAVY], 1)] = body;
-        return;
-    }
-    warp_sort_slice64(d.end_id + s, n, lane);
-    __syncwarp();
-    for (int p = s + lane; p < e; p += 32) {
-        const int id = d.end_id[p];
-        const int bond = id >> 1;
-        d.end_pos[id] = p;
-        const float4 x = (id & 1) ? d.bxj[bond] : d.bxi[bond];
-        d.end_x[p] = make_float4(x.x, x.y, x.z, 0.f);
-    }
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, body = t / CSR_LANES;
+    if (body < d.N) csr_place_body<WANT>(d, body, t % CSR_LANES);
 }
 
 // CSR of a scene whose only contacts are with the ground.  Contact bonds follow the static
@@ -163,6 +120,7 @@ __global__ void k_csr_sort(Dev d) {
 // ground contacts, and starts at sta_off[b] + gnd_off[b] -- the sum of two prefix sums: no
 // count, atomics or sort.  Ground contacts past the contact capacity were not written (the
 // narrow phase latched PABD_ERR_CAPACITY); the slices skip them.
+template <int WANT>
 __global__ void k_csr_ground(Dev d) {
     pdl_enter();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -176,42 +134,21 @@ __global__ void k_csr_ground(Dev d) {
     const int gn = min(d.gnd_off[b + 1], cap) - g0;
     for (int k = 0; k < sn; ++k) {
         const int id = d.sta_id[s0 + k];
-        const int bond = id >> 1;
-        d.end_id[off + k] = id;
-        d.end_pos[id] = off + k;
-        const float4 x = (id & 1) ? d.bxj[bond] : d.bxi[bond];
-        d.end_x[off + k] = make_float4(x.x, x.y, x.z, 0.f);
+        place_end<WANT>(d, id, off + k);
     }
     for (int k = 0; k < gn; ++k) {
-        const int bond = d.Nc + g0 + k;
-        const int p = off + sn + k;
-        d.end_id[p] = 2 * bond;
-        d.end_pos[2 * bond] = p;
-        const float4 x = d.bxi[bond];
-        d.end_x[p] = make_float4(x.x, x.y, x.z, 0.f);
+        place_end<WANT>(d, 2 * (d.Nc + g0 + k), off + sn + k);
     }
     if (sn + gn > HEAVY_ENDS) d.heavy[atomicAdd(&d.ctr[C_NHEAVY], 1)] = b;
 }
 
-// The heavy bodies' slices, one block per body (block_sort_slice), the end-record buffer
-// (unused at this stage) as scratch.
+// the heavy bodies' slices, one block per body
+template <int WANT>
 __global__ void __launch_bounds__(LONG_T) k_csr_sort_long(Dev d) {
     pdl_enter();
     extern __shared__ int key[];
     const int nheavy = d.ctr[C_NHEAVY];
-    for (int h = blockIdx.x; h < nheavy; h += gridDim.x) {
-        const int body = d.heavy[h];
-        const int s = d.end_off[body], e = d.end_off[body + 1], n = e - s;
-        block_sort_slice(d.end_id + s, n, reinterpret_cast<int*>(d.ends) + s, key);
-        for (int p = s + threadIdx.x; p < e; p += LONG_T) {
-            const int id = d.end_id[p];
-            const int bond = id >> 1;
-            d.end_pos[id] = p;
-            const float4 x = (id & 1) ? d.bxj[bond] : d.bxi[bond];
-            d.end_x[p] = make_float4(x.x, x.y, x.z, 0.f);
-        }
-        __syncthreads();
-    }
+    for (int h = blockIdx.x; h < nheavy; h += gridDim.x) csr_sort_heavy<LONG_T, WANT>(d, d.heavy[h], key);
 }
 
 // ---- light bodies ordered by (class, end count) ----
@@ -294,11 +231,6 @@ void launch_light_order(const Dev& d, cudaStream_t st, long long* launches) {
     *launches += 2;
 }
 
-cudaError_t setup_csr_kernels() {
-    return cudaFuncSetAttribute(k_csr_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                LONG_SMEM * (int)sizeof(int));
-}
-
 // per-group residual sqrt(sum over the group's bodies of |q^{k+1} - q^k|^2): one block of
 // RES_T threads per group, fixed per-thread strides, warp shuffle tree, warps summed in
 // order by thread 0 (deterministic)
@@ -367,14 +299,7 @@ void launch_drive_update(const Dev& d, cudaStream_t st, long long* launches) {
 __global__ void k_step_reset(Dev d) {
     pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t == 0) {
-        d.ctr[C_NPAIRS] = 0;
-        d.ctr[C_CELLBITS] = 0;
-        d.ctr[C_NLARGE] = 0;
-        d.ctr[C_NHEAVY] = 0;
-        d.ctr[C_FP64DYN] = 0;
-        for (int k = C_NPHEAVY; k < C_COUNT; ++k) d.ctr[k] = 0;
-    }
+    if (t == 0) reset_counters(d);
     if (d.bvh_bounds && t < 6) d.bvh_bounds[t] = t < 3 ? 0x7fffffff : (int)0x80000000;
     if (d.p.broadphase == 0 && t < (1 << d.table_bits)) {
         d.bucket_cnt[t] = 0;
@@ -401,17 +326,20 @@ void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches) {
 }
 
 void launch_csr(const Dev& d, cudaStream_t st, long long* launches) {
-    if (d.sta_off) {
-        launch_pdl(k_csr_ground, dim3(nblk(d.N + 1)), dim3(ST_T), 0, st, d);
-        *launches += 1;
-        return;
-    }
-    launch_pdl(k_csr_count, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
-    scan_exclusive(d.end_cnt, d.end_off, nullptr, d.N, d.scan_scratch, st, launches);
-    launch_pdl(k_csr_fill, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
-    launch_pdl(k_csr_sort, dim3(nblk(d.N * 32)), dim3(ST_T), 0, st, d);
-    launch_pdl(k_csr_sort_long, dim3(152), dim3(LONG_T), LONG_SMEM * sizeof(int), st, d);
-    *launches += 4;
+    with_want(d.csr_want, [&](auto w) {
+        constexpr int WANT = decltype(w)::value;
+        if (d.sta_off) {
+            launch_pdl(k_csr_ground<WANT>, dim3(nblk(d.N + 1)), dim3(ST_T), 0, st, d);
+            *launches += 1;
+            return;
+        }
+        launch_pdl(k_csr_count, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
+        scan_exclusive(d.end_cnt, d.end_off, nullptr, d.N, d.scan_scratch, st, launches);
+        launch_pdl(k_csr_fill, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
+        launch_pdl(k_csr_sort<WANT>, dim3(nblk(d.N * CSR_LANES)), dim3(ST_T), 0, st, d);
+        launch_pdl(k_csr_sort_long<WANT>, dim3(152), dim3(LONG_T), LONG_SMEM * sizeof(int), st, d);
+        *launches += 4;
+    });
 }
 
 // Scenes whose groups have at most 128 bodies (a block per group would leave most of its threads

@@ -18,6 +18,7 @@
 //            flagged, or a Cholesky pivot below 1e-3 of its diagonal): those sum the same
 //            single-precision records and factor in an extended type -- double-float on
 //            the FP32 pipes (precision policy 1), or FP64 (policy 2).
+#include "predict.cuh"
 #include "sweep_shape.h"
 
 namespace pabd {
@@ -68,7 +69,7 @@ __device__ __forceinline__ void bond_one(const Dev& d, const float4* __restrict_
 // holds room for every possible contact, far more than a step has).  Each thread loads its
 // first bond's static part before it waits for the previous sweep (pdl_enter), so that the
 // loads overlap that sweep's last blocks; q^k and the augmented Lagrangian state are read after.
-__global__ void __launch_bounds__(BOND_T) k_bond(Dev d, const float4* __restrict__ q, int it) {
+__global__ void __launch_bounds__(BOND_T, 5) k_bond(Dev d, const float4* __restrict__ q, int it) {
     const int nb = d.ctr[C_NBONDS];  // (set by the step's front, before the sweeps)
     const int b0 = blockIdx.x * blockDim.x + threadIdx.x;
     BondStatic s0;
@@ -161,16 +162,10 @@ void launch_solve(const Dev& d, const float4* q_in, float4* q_out, int it, int l
     *launches += 1;
 }
 
-// augmented Lagrangian warm start at the start of a step (Eq. 29), from the values the
-// previous step ended with (parity n_iter): kappa <- max(gamma kappa, kappa_start),
-// lambda <- alpha gamma lambda, into the parity-0 buffer read by the first sweep
 __global__ void k_al_warm(Dev d) {
     pdl_enter();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= d.Nc || d.bmeta[b].z != K_AL) return;
-    const float2 kl = (d.p.n_iter & 1) ? d.al_st1[b] : d.al_st0[b];
-    const float4 pr = d.al_par[b];  // (kappa_start, beta, alpha, gamma)
-    d.al_st0[b] = make_float2(fmaxf(pr.w * kl.x, pr.x), pr.z * pr.w * kl.y);
+    if (b < d.Nc) al_warm(d, b);
 }
 
 // the dual update from the step's final iterate (after the last sweep), into parity n_iter

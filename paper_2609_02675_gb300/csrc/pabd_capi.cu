@@ -254,32 +254,43 @@ std::vector<int2> choose_bins(const std::vector<int>& group_off, int G, int N, i
 constexpr int PROF_EVENTS = 6;
 
 void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nullptr) {
-    const Dev& d = s->d;
     const bool in_bins = s->mode == 2 && !s->fused && s->in_bins;
-    const bool use_order = d.light_sorted && !in_bins;  // (the bins order their own bodies)
+    const bool use_order = s->d.light_sorted && !in_bins;  // (the bins order their own bodies)
+    Dev d = s->d;
+    // (a cooperative launch that is refused falls back to the bond and solve launches)
+    d.csr_want = s->fused ? WANT_SLOTS | WANT_RECORDS : (s->mode == 2 ? WANT_RECORDS : WANT_SLOTS);
     int e = 0;
     auto mark = [&]() {
         if (ev) cudaEventRecordWithFlags(ev[e++], s->st, cudaEventRecordExternal);
     };
     mark();
-    launch_step_reset(d, s->st, launches);
-    launch_drive_update(d, s->st, launches);
-    if (d.sta_off) {
-        // ground-only scene: collision, CSR and predictor in one fused front (the predictor's
-        // stage is then empty in the profiling graph's split)
-        launch_ground_front(d, s->st, launches);
+    if (front_fits(d.N, d.p.body_contacts)) {
+        // small scene: everything up to the sweeps in one launch (its stages are then all in the
+        // profiling graph's first)
+        launch_front(d, s->st, launches);
         mark();
         if (use_order) launch_light_order(d, s->st, launches);
         mark();
     } else {
-        launch_collision(d, s->st, launches);
-        mark();
-        launch_csr(d, s->st, launches);
-        if (use_order) launch_light_order(d, s->st, launches);
-        mark();
-        launch_predict(d, s->st, launches);
+        launch_step_reset(d, s->st, launches);
+        launch_drive_update(d, s->st, launches);
+        if (d.sta_off) {
+            // ground-only scene: collision, CSR and predictor in one fused front (the predictor's
+            // stage is then empty in the profiling graph's split)
+            launch_ground_front(d, s->st, launches);
+            mark();
+            if (use_order) launch_light_order(d, s->st, launches);
+            mark();
+        } else {
+            launch_collision(d, s->st, launches);
+            mark();
+            launch_csr(d, s->st, launches);
+            if (use_order) launch_light_order(d, s->st, launches);
+            mark();
+            launch_predict(d, s->st, launches);
+        }
+        launch_al_warm(d, s->st, launches);
     }
-    launch_al_warm(d, s->st, launches);
     mark();
     float4* cur = d.qa;
     float4* nxt = d.qb;
@@ -309,7 +320,6 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
         // is at most resid_tol (or n_iter sweeps).  In a graph the loop is a conditional WHILE
         // node whose body is one sweep; launched eagerly, n_iter sweeps are enqueued and those
         // after the loop has ended return at once.
-        launch_end_records(d, s->st, launches);
         launch_sweep_ctl_init(d, s->st, launches);
         auto one_sweep = [&](cudaStream_t st, unsigned long long handle) {
             cudaMemsetAsync(d.ctr + C_FP64DYN, 0, sizeof(int), st);
@@ -345,11 +355,9 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
         }
         cur = nullptr;  // the last iterate's buffer is known on the device only
     } else if (in_bins) {
-        launch_end_records(d, s->st, launches);
         launch_sweep_bins(d, s->bins, s->lanes, s->st, launches);
         if (d.p.n_iter & 1) { float4* t = cur; cur = nxt; nxt = t; }
     } else if (s->mode == 2) {
-        launch_end_records(d, s->st, launches);
         // (the counter of run-time extended-precision redos, which counts the last sweep's, was
         // reset at the head of the step): the sweeps follow each other as programmatic dependents
         for (int it = 0; it < d.p.n_iter; ++it) {
@@ -371,7 +379,8 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
 // HEAVY_T-thread blocks; keep the fastest.  The shape never changes the results (each body's
 // arithmetic does not depend on which block runs it).
 pabd_status autotune_sweep(pabd_scene* s) {
-    Dev& d = s->d;
+    Dev d = s->d;
+    d.csr_want = WANT_RECORDS;
     long long lc = 0;
     launch_step_reset(d, s->st, &lc);
     launch_drive_update(d, s->st, &lc);
@@ -437,6 +446,7 @@ pabd_status autotune_default(pabd_scene* s) {
     if (d.N == 0 || d.Nal > 0 || (!tune_mode && !tune_order)) return PABD_OK;
     long long lc = 0;
     Dev dd = d;
+    dd.csr_want = WANT_SLOTS | WANT_RECORDS;
     launch_step_reset(dd, s->st, &lc);
     launch_drive_update(dd, s->st, &lc);
     if (dd.sta_off) {
@@ -447,7 +457,6 @@ pabd_status autotune_default(pabd_scene* s) {
         launch_predict(dd, s->st, &lc);
     }
     launch_light_order(dd, s->st, &lc);
-    launch_end_records(dd, s->st, &lc);
     CK(cudaGetLastError());
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
@@ -887,7 +896,6 @@ pabd_status finalize_scene(pabd_scene* s) {
     CK(cudaStreamSynchronize(st));
 
     // lanes per body from the descriptor; fused sweep block / grid from a timing sweep
-    CK(setup_csr_kernels());
     if (p.broadphase == 1 || d.multilevel) CK(setup_pair_sort());
 
     // lanes per body: given, or from the body count -- the largest of 16, 8, 4, 2, 1 lanes

@@ -71,6 +71,9 @@ constexpr int HEAVY_BLOCKS = 152;
 // the longest warps start first (the launch does not end on them).  2 * END_BINS bins; which
 // lanes take a body never changes its arithmetic.
 constexpr int END_BINS = HEAVY_ENDS + 1;
+// what the step's sweeps read of a bond end: its slot and material point (the bond and solve
+// launches), its record (the others)
+constexpr int WANT_SLOTS = 1, WANT_RECORDS = 2;
 constexpr int RES_CHUNK = 4096;
 constexpr int PAIR_STASH = 4;
 constexpr int STASH_DELIVER = 0x40000000;
@@ -126,6 +129,7 @@ struct Dev {
     int *order;                 // this step's light bodies by (class, end count), C_NLIGHT of them
     int *bin_cnt, *bin_cur;     // per bin of the light order: bodies, and the blocks' reservations
     float4 *rec;                // bond-end records in CSR order, 3 float4 per end (pack_end)
+    int csr_want;               // what the CSR is built with (WANT_SLOTS, WANT_RECORDS)
     unsigned *gbar;             // grid barrier: arrival counter, generation
     unsigned *wait_limit;       // polls before a device-side wait gives up (PABD_ERR_TIMEOUT)
     int2 *bin_range;            // body range of each bin of k_sweep_bins, or null
@@ -244,6 +248,10 @@ void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches);
 void launch_collision(const Dev& d, cudaStream_t st, long long* launches);
 // the front of a step in a ground-only scene: collision, CSR and predictor (k_collision.cu)
 void launch_ground_front(const Dev& d, cudaStream_t st, long long* launches);
+// the whole front of a small scene's step (reset, drives, collision, CSR, predictor, augmented
+// Lagrangian warm start) in one launch (k_front.cu), for scenes of so many bodies
+bool front_fits(int n_bodies, bool contacts);
+void launch_front(const Dev& d, cudaStream_t st, long long* launches);
 // LBVH pairs from this step's boxes (after k_aabb): the same output as the grid's pair stage
 void launch_lbvh_pairs(const Dev& d, cudaStream_t st, long long* launches);
 cudaError_t setup_pair_sort();
@@ -253,8 +261,6 @@ void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches);
 void launch_csr(const Dev& d, cudaStream_t st, long long* launches);
 // the light bodies ordered by (class, end count) into Dev::order (after launch_csr)
 void launch_light_order(const Dev& d, cudaStream_t st, long long* launches);
-// opt the CSR block sort into its 128 KB of dynamic shared memory (once per process and device)
-cudaError_t setup_csr_kernels();
 void launch_predict(const Dev& d, cudaStream_t st, long long* launches);
 void launch_bond(const Dev& d, const float4* q, int it, cudaStream_t st, long long* launches);
 // augmented Lagrangian: warm start (before the sweeps) and the update after the last sweep
@@ -283,7 +289,6 @@ struct BinsShape {
 cudaError_t setup_sweep_bins(const BinsShape& b, int lanes, bool f64, int* fit);
 void launch_sweep_bins(const Dev& d, const BinsShape& b, int lanes, cudaStream_t st, long long* launches);
 // one launch per sweep (bonds evaluated by the solve from CSR-ordered end records)
-void launch_end_records(const Dev& d, cudaStream_t st, long long* launches);
 void launch_sweep_one(const Dev& d, const float4* qi, float4* qo, int it, int lanes, int threads, cudaStream_t st,
                       long long* launches, bool pdl = false);
 

@@ -1,5 +1,7 @@
-// The predictor of Alg. 1 for one body, shared by the predictor kernel (k_step.cu) and the
-// fused per-body prelude of ground-only scenes (k_collision.cu).
+// What starts a step -- the predictor of Alg. 1, the drive anchors, the counters, the augmented
+// Lagrangian warm start -- shared by their kernels (k_step.cu, k_sweep.cu), the fused per-body
+// prelude of ground-only scenes (k_collision.cu) and the one-launch front of small scenes
+// (k_front.cu).
 #pragma once
 #include "pabd_internal.h"
 
@@ -44,6 +46,41 @@ __device__ __forceinline__ void predict_body(const Dev& d, int b) {
     store_q(d.sq, b, cs, A);
     store_q(d.qa, b, cs, A);
     d.qstar[b] = Qn;
+}
+
+// Drive anchors at t = (step + 1) h: x_i = x_i0 + arm (cos th r + sin th (u x r)),
+// th = amp sin(2 pi t / period + phase).
+__device__ __forceinline__ void drive_update(const Dev& d, int k) {
+    const double t = (double)(*d.step_index + 1) * d.p.h_d;
+    float4 a = d.drv[3 * k], r = d.drv[3 * k + 1], ur = d.drv[3 * k + 2];
+    float2 pp = d.drv_t[k];
+    const float th = r.w * sinf((float)(6.283185307179586 * t / (double)pp.x) + pp.y);
+    float cs, sn;
+    sincosf(th, &sn, &cs);
+    const int bi = d.drv_bond[k];
+    float4 cur = d.bxi[bi];
+    d.bxi[bi] = make_float4(a.x + a.w * (cs * r.x + sn * ur.x), a.y + a.w * (cs * r.y + sn * ur.y),
+                            a.z + a.w * (cs * r.z + sn * ur.z), cur.w);
+}
+
+// the step's counters (C_NBONDS and the contact counts are set again later in the step)
+__device__ __forceinline__ void reset_counters(const Dev& d) {
+    d.ctr[C_NPAIRS] = 0;
+    d.ctr[C_CELLBITS] = 0;
+    d.ctr[C_NLARGE] = 0;
+    d.ctr[C_NHEAVY] = 0;
+    d.ctr[C_FP64DYN] = 0;
+    for (int k = C_NPHEAVY; k < C_COUNT; ++k) d.ctr[k] = 0;
+}
+
+// augmented Lagrangian warm start of bond b at the start of a step (Eq. 29), from the values the
+// previous step ended with (parity n_iter): kappa <- max(gamma kappa, kappa_start),
+// lambda <- alpha gamma lambda, into the parity-0 buffer read by the first sweep
+__device__ __forceinline__ void al_warm(const Dev& d, int b) {
+    if (d.bmeta[b].z != K_AL) return;
+    const float2 kl = (d.p.n_iter & 1) ? d.al_st1[b] : d.al_st0[b];
+    const float4 pr = d.al_par[b];  // (kappa_start, beta, alpha, gamma)
+    d.al_st0[b] = make_float2(fmaxf(pr.w * kl.x, pr.x), pr.z * pr.w * kl.y);
 }
 
 }  // namespace pabd

@@ -58,21 +58,22 @@ __device__ __forceinline__ void warp_sort_slice64(int* v, int n, int lane) {
     if (2 * lane + 1 < n) v[2 * lane + 1] = v1;
 }
 
-// slice v[0..n) by a whole block of LONG_T threads with `key` LONG_SMEM ints of shared memory
+// slice v[0..n) by a whole block of T threads with `key` LONG_SMEM ints of shared memory
 // and tmp[0..n) scratch: runs of up to LONG_SMEM keys by a bitonic network in shared memory,
 // then runs merged pairwise (run length doubling), each key placed at its index in its run
 // plus its rank in the partner run (a binary search), ping-ponging between v and tmp.  Every
 // thread of the block calls it with the same slice.
+template <int T>
 __device__ __forceinline__ void block_sort_slice(int* v, int n, int* tmp, int* key) {
     for (int r0 = 0; r0 < n; r0 += LONG_SMEM) {
         const int rn = min(LONG_SMEM, n - r0);
         int m = 2;
         while (m < rn) m <<= 1;
-        for (int k = threadIdx.x; k < m; k += LONG_T) key[k] = k < rn ? v[r0 + k] : 0x7fffffff;
+        for (int k = threadIdx.x; k < m; k += T) key[k] = k < rn ? v[r0 + k] : 0x7fffffff;
         __syncthreads();
         for (int size = 2; size <= m; size <<= 1) {
             for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int k = threadIdx.x; k < m; k += LONG_T) {
+                for (int k = threadIdx.x; k < m; k += T) {
                     const int l = k ^ stride;
                     if (l > k) {
                         const bool up = (k & size) == 0;
@@ -83,13 +84,13 @@ __device__ __forceinline__ void block_sort_slice(int* v, int n, int* tmp, int* k
                 __syncthreads();
             }
         }
-        for (int k = threadIdx.x; k < rn; k += LONG_T) v[r0 + k] = key[k];
+        for (int k = threadIdx.x; k < rn; k += T) v[r0 + k] = key[k];
         __syncthreads();
     }
     int* src = v;
     int* dst = tmp;
     for (int R = LONG_SMEM; R < n; R <<= 1) {
-        for (int k = threadIdx.x; k < n; k += LONG_T) {
+        for (int k = threadIdx.x; k < n; k += T) {
             const int run = k / R, start = run * R, pstart = (run ^ 1) * R;
             const int plen = max(0, min(R, n - pstart));
             const int x = src[k];
@@ -104,7 +105,7 @@ __device__ __forceinline__ void block_sort_slice(int* v, int n, int* tmp, int* k
         int* t = src; src = dst; dst = t;
     }
     if (src != v) {
-        for (int k = threadIdx.x; k < n; k += LONG_T) v[k] = src[k];
+        for (int k = threadIdx.x; k < n; k += T) v[k] = src[k];
         __syncthreads();
     }
 }
