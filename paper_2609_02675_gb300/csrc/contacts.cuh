@@ -320,7 +320,7 @@ __device__ __forceinline__ void narrow_write_item(const Dev& d, int tt, int np, 
 // the step's contact and bond counts, once both prefix sums are known (one thread)
 __device__ __forceinline__ void set_contact_counts(const Dev& d, int npc) {
     int nk = npc + d.gnd_off[d.N];
-    if (nk > d.cap_contacts) { atomicOr(&d.ctr[C_STATUS], ST_CAPACITY); nk = d.cap_contacts; }
+    if (nk > d.cap_contacts) { latch_status(d, ST_CAPACITY); nk = d.cap_contacts; }
     d.ctr[C_NPC] = min(npc, d.cap_contacts);
     d.ctr[C_NGC] = nk - min(npc, d.cap_contacts);
     d.ctr[C_NBONDS] = d.Nc + nk;

@@ -242,7 +242,7 @@ __global__ void k_pair_write(Dev d) {
     }
     if (i == d.N - 1 && lane == 0) {
         int tot = d.pair_off[d.N];
-        if (tot > cap) atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);
+        if (tot > cap) latch_status(d, ST_CAPACITY);
         d.ctr[C_NPAIRS] = min(tot, cap);
     }
 }
@@ -360,7 +360,7 @@ __global__ void k_ml_pair_write(Dev d) {
     }
     if (i == d.N - 1 && lane == 0) {
         const int tot = d.pair_off[d.N];
-        if (tot > cap) atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);
+        if (tot > cap) latch_status(d, ST_CAPACITY);
         d.ctr[C_NPAIRS] = min(tot, cap);
     }
 }
@@ -528,7 +528,7 @@ __global__ void k_ground_bonds_csr(Dev d) {
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         int nk = gnd_prefix(d, nb);
-        if (nk > cap) { atomicOr(&d.ctr[C_STATUS], ST_CAPACITY); nk = cap; }
+        if (nk > cap) { latch_status(d, ST_CAPACITY); nk = cap; }
         d.ctr[C_NPC] = 0;
         d.ctr[C_NGC] = nk;
         d.ctr[C_NBONDS] = d.Nc + nk;

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(FT, 1) k_front(Dev d0) {
             __syncthreads();
         }
         if (t == 0) {
-            if (tot > cap) atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);
+            if (tot > cap) latch_status(d, ST_CAPACITY);
             d.ctr[C_NPAIRS] = np;
         }
         if (np <= FRONT_PAIRS) {

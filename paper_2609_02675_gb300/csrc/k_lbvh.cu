@@ -237,7 +237,7 @@ __device__ __forceinline__ int bvh_partners(const Dev& d, int i, F&& f) {
             } else if (sp < 64) {
                 stack[sp++] = kid;
             } else {
-                atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);  // deeper than any tree of 30-bit codes
+                latch_status(d, ST_CAPACITY);  // deeper than any tree of 30-bit codes
             }
         }
         if (next < 0) {
@@ -276,7 +276,7 @@ __global__ void k_bvh_pair_write(Dev d) {
     }
     if (k == d.N - 1) {
         const int tot = d.pair_off[d.N];
-        if (tot > cap) atomicOr(&d.ctr[C_STATUS], ST_CAPACITY);
+        if (tot > cap) latch_status(d, ST_CAPACITY);
         d.ctr[C_NPAIRS] = min(tot, cap);
     }
 }

@@ -19,7 +19,8 @@
 
 namespace pabd {
 
-__device__ __forceinline__ bool grid_sync(unsigned* bar, int* status, unsigned limit) {
+__device__ __forceinline__ bool grid_sync(const Dev& d, unsigned limit) {
+    unsigned* const bar = d.gbar;
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -36,7 +37,7 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, int* status, unsigned l
             unsigned spins = 0;
             while (*vgen == gen) {  // poll without sleeping first, then back off
                 if (++spins > limit) {
-                    atomicOr(status, ST_TIMEOUT);
+                    latch_status(d, ST_TIMEOUT);
                     ok = 0;
                     break;
                 }
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(HEAVY_T, 4) k_sweep_fused(Dev d) {
                 solve_body<L, L, X>(d, b, lane, team, qi, qo, last, end_gather(d, GlobalQ{qi}, it));
             __syncwarp();
         }
-        if (it + 1 < d.p.n_iter && !grid_sync(d.gbar, &d.ctr[C_STATUS], limit)) return;
+        if (it + 1 < d.p.n_iter && !grid_sync(d, limit)) return;
     }
 }
 

@@ -60,7 +60,7 @@ __device__ __forceinline__ void finalize_body(const Dev& d, int b, const float4*
             W[3 * r + c] = s * ih;
         }
     for (int k = 0; k < 9; ++k) finite &= isfinite(A1[k]);
-    if (!finite) atomicOr(&d.ctr[C_STATUS], ST_DIVERGED);
+    if (!finite) latch_status(d, ST_DIVERGED);
     d.vel[b] = make_float4(v[0], v[1], v[2], 0.f);
     d.omg[b] = make_float4(0.5f * (W[7] - W[5]), 0.5f * (W[2] - W[6]), 0.5f * (W[3] - W[1]), 0.f);
     float4 Q;

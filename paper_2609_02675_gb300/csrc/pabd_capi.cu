@@ -151,9 +151,7 @@ struct pabd_scene {
     size_t graph_nodes = 0;
     long long launches = 0;
     long long launches_per_step = 0;
-    int* h_status = nullptr;  // pinned
-    cudaEvent_t ev_status = nullptr;
-    bool status_pending = false;
+    int* h_status = nullptr;  // pinned: one word per status bit (Dev::host_status)
     int fp64_bodies = 0;
     int latched = 0;
     // stage timing: events recorded between the stages of a step, captured in a second graph
@@ -787,8 +785,14 @@ pabd_status finalize_scene(pabd_scene* s) {
 
     // device allocations
     bool ok = true;
-    ok &= alloc_arr(s, d.qn, 3 * N) && alloc_arr(s, d.qa, 3 * N) && alloc_arr(s, d.qb, 3 * N) && alloc_arr(s, d.sq, 3 * N);
-    ok &= alloc_arr(s, d.vel, N) && alloc_arr(s, d.omg, N) && alloc_arr(s, d.quat, N) && alloc_arr(s, d.qstar, N);
+    // the state in one piece, in the order of pabd_read_state_f32: q, Q, v, omega
+    ok &= alloc_arr(s, d.qn, 6 * (size_t)N) && alloc_arr(s, d.qa, 3 * N) && alloc_arr(s, d.qb, 3 * N) && alloc_arr(s, d.sq, 3 * N);
+    if (ok) {
+        d.quat = d.qn + 3 * (size_t)N;
+        d.vel = d.quat + N;
+        d.omg = d.vel + N;
+    }
+    ok &= alloc_arr(s, d.qstar, N);
     ok &= alloc_arr(s, d.mass, N) && alloc_arr(s, d.he, N) && alloc_arr(s, d.xs, N);
     ok &= alloc_arr(s, d.bflags, N) && alloc_arr(s, d.group, N) && alloc_arr(s, d.group_off, d.G + 1);
     ok &= alloc_arr(s, d.group_hold, d.G);
@@ -846,6 +850,9 @@ pabd_status finalize_scene(pabd_scene* s) {
         ok &= alloc_arr(s, d.blevel, N) && alloc_arr(s, d.pair_own, N) && alloc_arr(s, d.pair_cur, N);
     }
     if (!ok) return PABD_ERR_OOM;
+    if (!s->h_status) CK(cudaMallocHost(&s->h_status, sizeof(int) * STATUS_WORDS));
+    for (int k = 0; k < STATUS_WORDS; ++k) s->h_status[k] = 0;
+    CK(cudaHostGetDevicePointer((void**)&d.host_status, s->h_status, 0));
 
     cudaStream_t st = s->st;
     auto up = [&](void* dst, const void* src, size_t n) { return n ? cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st) : cudaSuccess; };
@@ -965,28 +972,19 @@ pabd_status finalize_scene(pabd_scene* s) {
 
     pabd_status cr = capture_step(s);
     if (cr != PABD_OK) return cr;
-    CK(cudaMallocHost(&s->h_status, sizeof(int)));
-    *s->h_status = 0;
-    CK(cudaEventCreateWithFlags(&s->ev_status, cudaEventDisableTiming));
+    // (the trial sweeps' status does not count)
+    for (int k = 0; k < STATUS_WORDS; ++k) s->h_status[k] = 0;
     s->ready = true;
     return PABD_OK;
 }
 
-pabd_status poll_status(pabd_scene* s, bool wait) {
-    if (!s->status_pending) return status_from_bits(s->latched);
-    cudaError_t q = wait ? cudaEventSynchronize(s->ev_status) : cudaEventQuery(s->ev_status);
-    if (q == cudaErrorNotReady) return PABD_OK;
-    CK(q);
-    s->status_pending = false;
-    s->latched |= *s->h_status;
+// the errors that the scene's work has latched so far (written by the device into page-locked
+// memory as they occur: no copy or event per step)
+pabd_status poll_status(pabd_scene* s) {
+    const volatile int* w = s->h_status;
+    for (int k = 0; w && k < STATUS_WORDS; ++k)
+        if (w[k]) s->latched |= 1 << k;
     return status_from_bits(s->latched);
-}
-
-pabd_status enqueue_status(pabd_scene* s) {
-    CK(cudaMemcpyAsync(s->h_status, s->d.ctr + C_STATUS, sizeof(int), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaEventRecord(s->ev_status, s->st));
-    s->status_pending = true;
-    return PABD_OK;
 }
 
 }  // namespace
@@ -1217,7 +1215,7 @@ pabd_status pabd_step(pabd_scene* s, int nsteps) {
     if (!s || nsteps < 0) return PABD_ERR_ARG;
     pabd_status r = finalize_scene(s);
     if (r != PABD_OK) return r;
-    r = poll_status(s, false);
+    r = poll_status(s);
     if (r != PABD_OK) return r;
     for (int k = 0; k < nsteps; ++k) {
         if (s->profiling) {
@@ -1228,7 +1226,7 @@ pabd_status pabd_step(pabd_scene* s, int nsteps) {
         CK(cudaGraphLaunch(s->exec, s->st));
         s->launches += s->launches_per_step;
     }
-    return enqueue_status(s);
+    return PABD_OK;
 }
 
 pabd_status pabd_tune(pabd_scene* s) {
@@ -1236,9 +1234,9 @@ pabd_status pabd_tune(pabd_scene* s) {
     pabd_status r = finalize_scene(s);
     if (r != PABD_OK) return r;
     if ((s->desc.sweep_mode != 0 && s->desc.light_order != 0) || s->d.p.resid_tol > 0 || s->fused) return PABD_OK;
-    r = poll_status(s, true);
-    if (r != PABD_OK) return r;
     CK(cudaStreamSynchronize(s->st));
+    r = poll_status(s);
+    if (r != PABD_OK) return r;
     const int mode0 = s->mode, sorted0 = s->d.light_sorted, threads0 = s->threads;
     const bool bins0 = s->in_bins;
     r = autotune_default(s);
@@ -1319,11 +1317,11 @@ pabd_status pabd_step_eager(pabd_scene* s, int nsteps) {
     if (!s || nsteps < 0) return PABD_ERR_ARG;
     pabd_status r = finalize_scene(s);
     if (r != PABD_OK) return r;
-    r = poll_status(s, false);
+    r = poll_status(s);
     if (r != PABD_OK) return r;
     for (int k = 0; k < nsteps; ++k) enqueue_step(s, &s->launches);
     CK(cudaGetLastError());
-    return enqueue_status(s);
+    return PABD_OK;
 }
 
 pabd_status pabd_detect(pabd_scene* s) {
@@ -1334,15 +1332,13 @@ pabd_status pabd_detect(pabd_scene* s) {
     launch_drive_update(s->d, s->st, &s->launches);
     launch_collision(s->d, s->st, &s->launches);
     CK(cudaGetLastError());
-    return enqueue_status(s);
+    return PABD_OK;
 }
 
 pabd_status pabd_sync(pabd_scene* s) {
     if (!s) return PABD_ERR_ARG;
     CK(cudaStreamSynchronize(s->st));
     if (!s->ready) return PABD_OK;
-    pabd_status r = poll_status(s, true);
-    if (r != PABD_OK) return r;
     int bits = 0;
     CK(cudaMemcpy(&bits, s->d.ctr + C_STATUS, sizeof(int), cudaMemcpyDeviceToHost));
     s->latched |= bits;
@@ -1403,11 +1399,8 @@ pabd_status pabd_read_state_f32(pabd_scene* s, float* host, size_t n) {
     if (r != PABD_OK) return r;
     const int N = s->d.N;
     if (n != (size_t)N) return PABD_ERR_ARG;
-    float* o = host;
-    CK(cudaMemcpyAsync(o, s->d.qn, sizeof(float4) * 3 * N, cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(o + 12 * (size_t)N, s->d.quat, sizeof(float4) * N, cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(o + 16 * (size_t)N, s->d.vel, sizeof(float4) * N, cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(o + 20 * (size_t)N, s->d.omg, sizeof(float4) * N, cudaMemcpyDeviceToHost, s->st));
+    // (the state is one piece on the device)
+    if (N) CK(cudaMemcpyAsync(host, s->d.qn, sizeof(float4) * 6 * (size_t)N, cudaMemcpyDeviceToHost, s->st));
     return PABD_OK;
 }
 
@@ -1417,11 +1410,7 @@ pabd_status pabd_write_state_f32(pabd_scene* s, const float* host, size_t n) {
     if (r != PABD_OK) return r;
     const int N = s->d.N;
     if (n != (size_t)N) return PABD_ERR_ARG;
-    const float* o = host;
-    CK(cudaMemcpyAsync(s->d.qn, o, sizeof(float4) * 3 * N, cudaMemcpyHostToDevice, s->st));
-    CK(cudaMemcpyAsync(s->d.quat, o + 12 * (size_t)N, sizeof(float4) * N, cudaMemcpyHostToDevice, s->st));
-    CK(cudaMemcpyAsync(s->d.vel, o + 16 * (size_t)N, sizeof(float4) * N, cudaMemcpyHostToDevice, s->st));
-    CK(cudaMemcpyAsync(s->d.omg, o + 20 * (size_t)N, sizeof(float4) * N, cudaMemcpyHostToDevice, s->st));
+    if (N) CK(cudaMemcpyAsync(s->d.qn, host, sizeof(float4) * 6 * (size_t)N, cudaMemcpyHostToDevice, s->st));
     return PABD_OK;
 }
 
@@ -1581,7 +1570,6 @@ pabd_status pabd_destroy_scene(pabd_scene* s) {
     if (s->prof_graph) cudaGraphDestroy(s->prof_graph);
     for (cudaEvent_t e : s->prof_ev) cudaEventDestroy(e);
     if (s->graph) cudaGraphDestroy(s->graph);
-    if (s->ev_status) cudaEventDestroy(s->ev_status);
     if (s->h_status) cudaFreeHost(s->h_status);
     for (void* p : s->allocs) {
         if (s->desc.free) s->desc.free(p, s->desc.alloc_ctx);

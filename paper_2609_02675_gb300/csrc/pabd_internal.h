@@ -17,6 +17,7 @@ namespace pabd {
 enum BondKind { K_SPHERICAL = 0, K_SPRING = 1, K_ELASTIC_NL = 2, K_DRIVE = 4, K_CONTACT = 5, K_GROUND = 6, K_AL = 7 };
 
 enum StatusBits { ST_CAPACITY = 1, ST_DIVERGED = 2, ST_TIMEOUT = 4 };
+constexpr int STATUS_WORDS = 3;  // host words, one per bit
 
 // BF_SHIFT: the body's system is assembled about a nonzero expansion point Dev::xs.
 // BF_STIFF: its static bonds' weights sum to more than 10 times its mass (stiff joints).
@@ -165,6 +166,7 @@ struct Dev {
     int *pair_own, *pair_cur;       // partners a body finds itself; cursor of those delivered to it
     // misc
     int *ctr;                   // Counter array
+    volatile int *host_status;  // page-locked host words, one per status bit (null: none)
     // sweeps under a residual threshold: (sweeps done, scenes still active, loop on, -) and
     // the scenes that have stopped
     int *sweep_ctl;
@@ -178,6 +180,13 @@ struct Dev {
 
 // body b's group is held still this step (pabd_set_group_hold)
 __device__ __forceinline__ bool held(const Dev& d, int b) { return d.group_hold[d.group[b]] != 0; }
+
+// latches a status bit in the scene's counters, and in the host's word for it (a store, not an
+// atomic: every bit has a word of its own)
+__device__ __forceinline__ void latch_status(const Dev& d, int bit) {
+    atomicOr(&d.ctr[C_STATUS], bit);
+    if (d.host_status) d.host_status[__ffs(bit) - 1] = 1;
+}
 
 // ---- programmatic dependent launch ----
 // A kernel launched by launch_pdl may be launched while its predecessor on the stream is still

@@ -921,7 +921,7 @@ __device__ __forceinline__ void finish_body(const Dev& d, int b, int plane, int 
         for (int k = 0; k < 3; ++k) { double t = (double)cn[k] - (double)c[k]; r2 += t * t; finite &= isfinite(cn[k]); }
 #pragma unroll
         for (int k = 0; k < 9; ++k) { double t = (double)An[k] - (double)A[k]; r2 += t * t; finite &= isfinite(An[k]); }
-        if (!finite) atomicOr(&d.ctr[C_STATUS], ST_DIVERGED);
+        if (!finite) latch_status(d, ST_DIVERGED);
         d.resid_body[b] = r2;
     }
     store(b, cn, An);
