@@ -74,12 +74,20 @@ __device__ __forceinline__ void csr_place_body(const Dev& d, int body, int lane)
     }
 }
 
-// A heavy body's slice, by a block of T threads (block_sort_slice), the end-record buffer of the
-// bond launch (unused at this stage) as scratch.
+// A heavy body's ends, by a block of T threads: ranked by a bitmap over the step's ends, or sorted
+// first with the bond launch's end-record buffer (unused at this stage) as scratch (the slab
+// under 48 x 48 boxes: CSR stage 73 us with the sort, 29 with the ranking).  key: 2 LONG_SMEM
+// ints.
 template <int T, int WANT>
 __device__ __forceinline__ void csr_sort_heavy(const Dev& d, int body, int* key) {
-    const int s = d.end_off[body], e = d.end_off[body + 1];
-    block_sort_slice<T>(d.end_id + s, e - s, reinterpret_cast<int*>(d.ends) + s, key);
+    const int s = d.end_off[body], e = d.end_off[body + 1], n = e - s;
+    const long long universe = 2ll * d.ctr[C_NBONDS];
+    if (rank_pays(n, universe)) {
+        block_rank_ids<T>(d.end_id + s, n, (int)universe, reinterpret_cast<unsigned*>(key), key + LONG_SMEM,
+                          [&](int id, int r) { place_end<WANT>(d, id, s + r); });
+        return;
+    }
+    block_sort_slice<T>(d.end_id + s, n, reinterpret_cast<int*>(d.ends) + s, key);
     for (int p = s + threadIdx.x; p < e; p += T) place_end<WANT>(d, d.end_id[p], p);
     __syncthreads();
 }

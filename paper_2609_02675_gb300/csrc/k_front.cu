@@ -73,9 +73,15 @@ template <int WANT>
 __global__ void __launch_bounds__(FT, 1) k_front(Dev d0) {
     __shared__ float4 lo[FRONT_N], hi[FRONT_N];
     __shared__ int cnt[FRONT_N], off[FRONT_N + 1], gcnt[FRONT_N], goff[FRONT_N + 1], ends[FRONT_N], cur[FRONT_N];
-    __shared__ int2 pairs[FRONT_PAIRS];
-    __shared__ int npc[FRONT_PAIRS], npc_off[FRONT_PAIRS + 1], ids[FRONT_ENDS], scan[FT / 32];
-    __shared__ int key[LONG_SMEM];
+    __shared__ int scan[FT / 32];
+    // the lists, and once they are done with, the heavy bodies' ranking
+    constexpr int LISTS = 4 * FRONT_PAIRS + 4 + FRONT_ENDS;
+    __shared__ int2 list[(LISTS > 2 * LONG_SMEM ? LISTS : 2 * LONG_SMEM) / 2];
+    int2* const pairs = list;
+    int* const npc = reinterpret_cast<int*>(pairs + FRONT_PAIRS);
+    int* const npc_off = npc + FRONT_PAIRS;
+    int* const ids = npc_off + FRONT_PAIRS + 4;
+    int* const key = reinterpret_cast<int*>(list);
     const int t = threadIdx.x, w = t >> 5, lane = t & 31, W = FT / 32;
     const int N = d0.N, cap = d0.cap_pairs;
     // the stages' view of the scene: what they hand on in shared memory

@@ -298,6 +298,8 @@ __global__ void k_pair_sort(Dev d) {
     for (int p = s + lane; p < e; p += 32) d.pairs[p] = make_int2(i, d.pair_j[p]);
 }
 
+// (an off-grid body's partners come in order: nothing to sort; the others are ranked by a bitmap
+// over the bodies, or sorted)
 __global__ void __launch_bounds__(LONG_T) k_pair_sort_long(Dev d) {
     pdl_enter();
     extern __shared__ int key[];
@@ -305,20 +307,24 @@ __global__ void __launch_bounds__(LONG_T) k_pair_sort_long(Dev d) {
     for (int h = blockIdx.x; h < nh; h += gridDim.x) {
         const int i = d.pair_heavy[h];
         const int s = min(d.pair_off[i], cap), e = min(d.pair_off[i + 1], cap);
-        block_sort_slice<LONG_T>(d.pair_j + s, e - s, d.pair_tmp + s, key);
+        bool unsorted = false;
+        for (int p = s + threadIdx.x; p + 1 < e; p += LONG_T) unsorted |= d.pair_j[p] > d.pair_j[p + 1];
+        if (__syncthreads_or(unsorted)) {
+            if (rank_pays(e - s, d.N)) {
+                block_rank_ids<LONG_T>(d.pair_j + s, e - s, d.N, reinterpret_cast<unsigned*>(key), key + LONG_SMEM,
+                                       [&](int j, int r) { d.pairs[s + r] = make_int2(i, j); });
+                continue;
+            }
+            block_sort_slice<LONG_T>(d.pair_j + s, e - s, d.pair_tmp + s, key);
+        }
         for (int p = s + threadIdx.x; p < e; p += LONG_T) d.pairs[p] = make_int2(i, d.pair_j[p]);
         __syncthreads();
     }
 }
 
-cudaError_t setup_pair_sort() {
-    return cudaFuncSetAttribute(k_pair_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                LONG_SMEM * (int)sizeof(int));
-}
-
 void launch_pair_sort(const Dev& d, cudaStream_t st, long long* launches) {
     launch_pdl(k_pair_sort, dim3(bblk((long long)d.N * 32)), dim3(BT), 0, st, d);
-    launch_pdl(k_pair_sort_long, dim3(152), dim3(LONG_T), LONG_SMEM * sizeof(int), st, d);
+    launch_pdl(k_pair_sort_long, dim3(152), dim3(LONG_T), 2 * LONG_SMEM * sizeof(int), st, d);
     *launches += 2;
 }
 

@@ -337,7 +337,7 @@ void launch_csr(const Dev& d, cudaStream_t st, long long* launches) {
         scan_exclusive(d.end_cnt, d.end_off, nullptr, d.N, d.scan_scratch, st, launches);
         launch_pdl(k_csr_fill, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
         launch_pdl(k_csr_sort<WANT>, dim3(nblk(d.N * CSR_LANES)), dim3(ST_T), 0, st, d);
-        launch_pdl(k_csr_sort_long<WANT>, dim3(152), dim3(LONG_T), LONG_SMEM * sizeof(int), st, d);
+        launch_pdl(k_csr_sort_long<WANT>, dim3(152), dim3(LONG_T), 2 * LONG_SMEM * sizeof(int), st, d);
         *launches += 4;
     });
 }

@@ -903,7 +903,6 @@ pabd_status finalize_scene(pabd_scene* s) {
     CK(cudaStreamSynchronize(st));
 
     // lanes per body from the descriptor; fused sweep block / grid from a timing sweep
-    if (p.broadphase == 1 || d.multilevel) CK(setup_pair_sort());
 
     // lanes per body: given, or from the body count -- the largest of 16, 8, 4, 2, 1 lanes
     // with lanes * N <= 2^17, but two rather than one for up to 2^18 bodies whose solves are

@@ -263,7 +263,6 @@ bool front_fits(int n_bodies, bool contacts);
 void launch_front(const Dev& d, cudaStream_t st, long long* launches);
 // LBVH pairs from this step's boxes (after k_aabb): the same output as the grid's pair stage
 void launch_lbvh_pairs(const Dev& d, cudaStream_t st, long long* launches);
-cudaError_t setup_pair_sort();
 // each body's partner slice of Dev::pair_j sorted ascending into Dev::pairs
 void launch_pair_sort(const Dev& d, cudaStream_t st, long long* launches);
 void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches);

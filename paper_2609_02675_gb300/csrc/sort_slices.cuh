@@ -110,4 +110,65 @@ __device__ __forceinline__ void block_sort_slice(int* v, int n, int* tmp, int* k
     }
 }
 
+// Ranks of unique ids in [0, universe) by a whole block of T threads: place(id, r) for every
+// id of v[0..n), r its place among them.  A bitmap of the ids in shared memory (LONG_SMEM words,
+// a window of the universe at a time) and the running count of its words: O(n + universe / 32)
+// instead of a sort's O(n log^2 n).  v is not changed.
+template <int T, class Place>
+__device__ __forceinline__ void block_rank_ids(const int* v, int n, int universe, unsigned* bits, int* before,
+                                               Place&& place) {
+    constexpr int PER = LONG_SMEM / T;
+    static_assert(PER * T == LONG_SMEM, "whole words per thread");
+    __shared__ int wsum[T / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int base = 0;  // ids below the window
+    for (long long w0 = 0; w0 < universe; w0 += 32ll * LONG_SMEM) {
+        for (int k = t; k < LONG_SMEM; k += T) bits[k] = 0u;
+        __syncthreads();
+        for (int k = t; k < n; k += T) {
+            const long long i = v[k] - w0;
+            if (i >= 0 && i < 32ll * LONG_SMEM) atomicOr(&bits[i >> 5], 1u << (i & 31));
+        }
+        __syncthreads();
+        int c[PER], s = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            c[k] = __popc(bits[t * PER + k]);
+            s += c[k];
+        }
+        int inc = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        int run = base + inc - s, all = 0;
+        for (int k = 0; k < T / 32; ++k) {
+            if (k < warp) run += wsum[k];
+            all += wsum[k];
+        }
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            before[t * PER + k] = run;
+            run += c[k];
+        }
+        __syncthreads();
+        for (int k = t; k < n; k += T) {
+            const int id = v[k];
+            const long long i = id - w0;
+            if (i >= 0 && i < 32ll * LONG_SMEM)
+                place(id, before[i >> 5] + __popc(bits[i >> 5] & ((1u << (i & 31)) - 1u)));
+        }
+        base += all;
+        __syncthreads();  // the bitmap is cleared for the next window
+    }
+}
+
+// ranking pays against sorting in place unless a short slice's ids spread over many windows
+__device__ __forceinline__ bool rank_pays(int n, long long universe) {
+    return universe <= 4ll * 32 * LONG_SMEM || n > LONG_SMEM;
+}
+
 }  // namespace pabd

@@ -975,6 +975,11 @@ struct EndGather {
         for (; p < e1; p += L) single(s, c, A, xs, p);
     }
     template <class T>
+    __device__ __forceinline__ void many(Sys<T>& s, const float* c, const float* A, const float* xs, int p, int e1,
+                                         int L) const {
+        one(s, c, A, xs, p, e1, L);
+    }
+    template <class T>
     __device__ __forceinline__ void two(Sys<T>& s, Sys<T>& t, const float* c, const float* A, const float* xs, int p,
                                         int e1, int L) const {
         if (sizeof(T) != 4) {  // (a lane after the other: the second sum starts once the first is complete)
@@ -1058,7 +1063,7 @@ __device__ __forceinline__ void solve_heavy(const Dev& d, int b, HeavyTeam team,
         Sys<float> s;
         if (t == 0) sys_init(s, mass, dc, dA, xs);
         else sys_zero(s);
-        gather.one(s, c, A, xs, e0 + t, e1, HEAVY_T);
+        gather.many(s, c, A, xs, e0 + t, e1, HEAVY_T);
         team_reduce(s, reinterpret_cast<Sys<float>*>(sh.buf), team);
         if (t == 0) {
             const float ratio = sys_solve(s, Xs);
@@ -1073,7 +1078,7 @@ __device__ __forceinline__ void solve_heavy(const Dev& d, int b, HeavyTeam team,
         Sys<X> s;
         if (t == 0) sys_init(s, mass, dc, dA, xs);
         else sys_zero(s);
-        gather.one(s, c, A, xs, e0 + t, e1, HEAVY_T);
+        gather.many(s, c, A, xs, e0 + t, e1, HEAVY_T);
         team_reduce(s, reinterpret_cast<Sys<X>*>(sh.buf), team);
         if (t == 0) {
             const auto se = ext_sys(s);

@@ -77,3 +77,41 @@ def test_cluster_sweeps_match_the_oracle(P, make, lanes):
         a, b = teacher_forced_step(g, ref)
         assert rel_err(a, b, np.asarray(sc.bodies["he"])) < REL_TOL
     g.close()
+
+
+@pytest.mark.parametrize("extra", [0, 20000, 70000])
+def test_heavy_slices_rank_alike_among_many_bonds(P, extra):
+    """Two slabs (about 400 and thousands of bond ends) step bit for bit alike alone and beside
+    `extra` boxes on the ground in a group of their own, whose contacts spread the slabs' end ids
+    over one, several and more than four windows of the ranking bitmap (and so over its sort)."""
+    parts = [S.slab_pile(10), S.slab_pile(40)]
+    n_slabs = sum(p.n_bodies for p in parts)
+    b = S._bodies(extra)
+    k = np.arange(extra)
+    b["he"], b["mass"] = 0.5, 1.0
+    b["c"] = np.stack([3.0 * (k % 300), np.full(extra, 0.5005), 3.0 * (k // 300)], 1)
+    par = dict(parts[0].params, n_iter=3)
+    outs = []
+    for order in ("slabs first", "boxes first"):
+        bodies = [parts[0].bodies.copy(), parts[1].bodies.copy()]
+        if extra:
+            bodies.insert(0 if order == "boxes first" else 2, b.copy())
+        for g, x in enumerate(bodies):
+            x["group"] = g
+        at = extra if order == "boxes first" else 0
+        for mode in (1, 2):
+            g = P.Scene(S.Scene("slabs", par, np.concatenate(bodies), S._bonds(0), 1), sweep_mode=mode, sweep_lanes=1)
+            g.step(8)
+            outs.append(g.state()[at:at + n_slabs])
+            if extra and order == "boxes first":
+                assert g.info()["n_bonds"] > 4 * extra
+            g.close()
+    alone = [x.copy() for x in (parts[0].bodies, parts[1].bodies)]
+    alone[1]["group"] = 1
+    g = P.Scene(S.Scene("slabs", par, np.concatenate(alone), S._bonds(0), 1), sweep_mode=2, sweep_lanes=1)
+    g.step(8)
+    ref = g.state()
+    assert g.info()["heavy_bodies"] == 2
+    g.close()
+    for o in outs:
+        assert np.array_equal(o, ref)
