@@ -103,17 +103,61 @@ __device__ __forceinline__ void aabb_body(const Dev& d, int b) {
     if (large && d.large_ids) d.large_ids[atomicAdd(&d.ctr[C_NLARGE], 1)] = b;
 }
 
-struct CPt {
-    float u[3], x[3];
+// A corner of the clipped incident face: u, its place in the reference box's frame, and (xa, xb),
+// its two coordinates along the incident face in the incident box's frame (the third is the
+// face's).  A polygon under clipping is read from one buffer of eight corners and written to
+// another; Poly::at(buffer, corner, component) says where they are.
+struct Corner {
+    float u[3], xa, xb;
 };
+struct LocalPoly {
+    float c[2][8][5];
+    __device__ __forceinline__ float& at(int b, int v, int k) { return c[b][v][k]; }
+};
+// in shared memory, element e of thread t at e T + t: no bank conflicts whatever the corner.
+// (Indexed by run-time corners, the buffers cannot be registers; in local memory the 384 bytes
+// of 800 threads per SM did not fit the L1 cache beside the shared memory.)
+template <int T>
+struct SharedPoly {
+    float* base;  // the thread's element 0
+    __device__ __forceinline__ float& at(int b, int v, int k) const { return base[((b * 8 + v) * 5 + k) * T]; }
+};
+template <class Poly>
+__device__ __forceinline__ Corner ld_corner(Poly& poly, int b, int v) {
+    return Corner{{poly.at(b, v, 0), poly.at(b, v, 1), poly.at(b, v, 2)}, poly.at(b, v, 3), poly.at(b, v, 4)};
+}
+template <class Poly>
+__device__ __forceinline__ void st_corner(Poly& poly, int b, int v, const Corner& c) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) poly.at(b, v, k) = c.u[k];
+    poly.at(b, v, 3) = c.xa;
+    poly.at(b, v, 4) = c.xb;
+}
+__device__ __forceinline__ float pick3(const float* v, int k) { return k == 0 ? v[0] : (k == 1 ? v[1] : v[2]); }
 
 __device__ __forceinline__ float dot_col(const float* A, int l, const float* r) {
     return FA(FA(FM(A[l], r[0]), FM(A[3 + l], r[1])), FM(A[6 + l], r[2]));
 }
 
-// Manifold of the pair (a, b); calls emit(i, j, x_i, x_j, N) for each contact, returns count.
-template <class Emit>
-__device__ int box_box(const FBox& fa, const FBox& fb, int a, int b, Emit&& emit) {
+// What a pair's contacts share: the incident and the reference body, the normal, and the incident
+// face (its axis ki and the coordinate xk along it).
+struct Manifold {
+    int ii, ir, ki;
+    float xk, N[3];
+};
+// the contact point in the incident body's frame
+__device__ __forceinline__ void corner_point(int ki, float xk, float xa, float xb, float* x) {
+    x[0] = ki == 0 ? xk : (ki == 2 ? xa : xb);
+    x[1] = ki == 1 ? xk : (ki == 0 ? xa : xb);
+    x[2] = ki == 2 ? xk : (ki == 1 ? xa : xb);
+}
+
+// Manifold of the pair (a, b); calls emit(corner, k) for contact k, whose corner's u is the point
+// in the reference body's frame, returns the count.  emit may write to buffer `out` of the
+// polygon up to corner k.
+template <class Poly, class Emit>
+__device__ __forceinline__ int box_box(const FBox& fa, const FBox& fb, int a, int b, Poly& poly, Manifold& mf, int& out,
+                                       Emit&& emit) {
     const float delta = FA(fa.infl, fb.infl);
     float dv[3], dab[3], dba[3], R[9];
 #pragma unroll
@@ -143,13 +187,28 @@ __device__ int box_box(const FBox& fa, const FBox& fb, int a, int b, Emit&& emit
         if (sep > best) { best = sep; ref_b = 0; l = ax; }
     }
     if (!(best <= delta)) return 0;
-    const FBox& fr = ref_b ? fb : fa;
-    const FBox& fi = ref_b ? fa : fb;
-    const int ir = ref_b ? b : a, ii = ref_b ? a : b;
-    const float sg = ref_b ? (dab[l] >= 0.f ? 1.f : -1.f) : (dba[l] >= 0.f ? 1.f : -1.f);
+    // the reference and the incident box (selected value by value: an index into the two boxes
+    // would put them in memory)
+    FBox fr, fi;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        fr.c[k] = ref_b ? fb.c[k] : fa.c[k];
+        fi.c[k] = ref_b ? fa.c[k] : fb.c[k];
+        fr.he[k] = ref_b ? fb.he[k] : fa.he[k];
+        fi.he[k] = ref_b ? fa.he[k] : fb.he[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        fr.A[k] = ref_b ? fb.A[k] : fa.A[k];
+        fi.A[k] = ref_b ? fa.A[k] : fb.A[k];
+    }
+    mf.ir = ref_b ? b : a;
+    mf.ii = ref_b ? a : b;
+    const float dl = ref_b ? pick3(dab, l) : pick3(dba, l);
+    const float sg = dl >= 0.f ? 1.f : -1.f, hl = pick3(fr.he, l);
     float N[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) N[k] = FM(sg, fr.A[3 * k + l]);
+    for (int k = 0; k < 3; ++k) mf.N[k] = N[k] = FM(sg, pick3(fr.A + 3 * k, l));
     int ki = 0;
     float bestd = 0.f, dsel = 0.f;
 #pragma unroll
@@ -158,61 +217,78 @@ __device__ int box_box(const FBox& fa, const FBox& fb, int a, int b, Emit&& emit
         if (k == 0 || fabsf(dk) > bestd) { bestd = fabsf(dk); ki = k; dsel = dk; }
     }
     const float si = dsel > 0.f ? -1.f : 1.f;
-    const int k1 = (ki + 1) % 3, k2 = (ki + 2) % 3;
-    const float sgn1[4] = {1.f, -1.f, -1.f, 1.f}, sgn2[4] = {1.f, 1.f, -1.f, -1.f};
-    CPt poly[8], tmp[8];
-    int np = 4;
+    const int k1 = ki == 2 ? 0 : ki + 1, k2 = ki == 0 ? 2 : ki - 1;
+    mf.ki = ki;
+    mf.xk = FM(si, pick3(fi.he, ki));
+    const float h1 = pick3(fi.he, k1), h2 = pick3(fi.he, k2);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-        float x[3], y[3], r[3];
-        x[ki] = FM(si, fi.he[ki]);
-        x[k1] = FM(sgn1[v], fi.he[k1]);
-        x[k2] = FM(sgn2[v], fi.he[k2]);
+        const float sgn1 = v == 0 || v == 3 ? 1.f : -1.f, sgn2 = v < 2 ? 1.f : -1.f;
+        Corner c;
+        c.xa = FM(sgn1, h1);
+        c.xb = FM(sgn2, h2);
+        float x[3], r[3];
+        corner_point(ki, mf.xk, c.xa, c.xb, x);
 #pragma unroll
         for (int dd = 0; dd < 3; ++dd) {
-            y[dd] = FA(FA(FA(fi.c[dd], FM(fi.A[3 * dd], x[0])), FM(fi.A[3 * dd + 1], x[1])), FM(fi.A[3 * dd + 2], x[2]));
-            r[dd] = FS(y[dd], fr.c[dd]);
+            const float y = FA(FA(FA(fi.c[dd], FM(fi.A[3 * dd], x[0])), FM(fi.A[3 * dd + 1], x[1])), FM(fi.A[3 * dd + 2], x[2]));
+            r[dd] = FS(y, fr.c[dd]);
         }
 #pragma unroll
-        for (int m = 0; m < 3; ++m) { poly[v].u[m] = dot_col(fr.A, m, r); poly[v].x[m] = x[m]; }
+        for (int m = 0; m < 3; ++m) c.u[m] = dot_col(fr.A, m, r);
+        st_corner(poly, 0, v, c);
     }
-    const int m1 = (l + 1) % 3, m2 = (l + 2) % 3;
+    const int m1 = l == 2 ? 0 : l + 1, m2 = l == 0 ? 2 : l - 1;
+    int np = 4, src = 0;
     for (int pl = 0; pl < 4 && np > 0; ++pl) {
         const int m = pl < 2 ? m1 : m2;
-        const float ps = (pl & 1) ? -1.f : 1.f, lim = fr.he[m];
+        const float ps = (pl & 1) ? -1.f : 1.f, lim = pick3(fr.he, m);
+        const Corner first = ld_corner(poly, src, 0);
+        const float dfirst = FS(FM(ps, pick3(first.u, m)), lim);
+        Corner P = first;
+        float dp = dfirst;
         int nt = 0;
         for (int v = 0; v < np; ++v) {
-            const CPt& P = poly[v];
-            const CPt& Q = poly[(v + 1) % np];
-            float dp = FS(FM(ps, P.u[m]), lim), dq = FS(FM(ps, Q.u[m]), lim);
-            bool pin = dp <= 0.f, qin = dq <= 0.f;
-            if (pin) tmp[nt++] = P;
-            if (pin != qin) {
-                float t = __fdiv_rn(dp, FS(dp, dq));
-                CPt X;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    X.u[c] = FA(P.u[c], FM(t, FS(Q.u[c], P.u[c])));
-                    X.x[c] = FA(P.x[c], FM(t, FS(Q.x[c], P.x[c])));
-                }
-                tmp[nt++] = X;
+            Corner Q = first;
+            float dq = dfirst;
+            if (v + 1 < np) {
+                Q = ld_corner(poly, src, v + 1);
+                dq = FS(FM(ps, pick3(Q.u, m)), lim);
             }
+            const bool pin = dp <= 0.f, qin = dq <= 0.f;
+            if (pin && nt < 8) st_corner(poly, src ^ 1, nt++, P);
+            if (pin != qin && nt < 8) {
+                const float t = __fdiv_rn(dp, FS(dp, dq));
+                Corner X;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) X.u[c] = FA(P.u[c], FM(t, FS(Q.u[c], P.u[c])));
+                X.xa = FA(P.xa, FM(t, FS(Q.xa, P.xa)));
+                X.xb = FA(P.xb, FM(t, FS(Q.xb, P.xb)));
+                st_corner(poly, src ^ 1, nt++, X);
+            }
+            P = Q;
+            dp = dq;
         }
         np = nt;
-        for (int v = 0; v < nt; ++v) poly[v] = tmp[v];
+        src ^= 1;
     }
+    out = src ^ 1;
     int cnt = 0;
+    const float top = FM(sg, hl);
     for (int v = 0; v < np; ++v) {
-        float hgt = FS(FM(sg, poly[v].u[l]), fr.he[l]);
+        Corner c = ld_corner(poly, src, v);
+        const float hgt = FS(FM(sg, pick3(c.u, l)), hl);
         if (!(hgt < delta)) continue;
-        float xj[3] = {poly[v].u[0], poly[v].u[1], poly[v].u[2]};
-        xj[l] = FM(sg, fr.he[l]);
-        emit(ii, ir, poly[v].x, xj, N, cnt);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k == l) c.u[k] = top;
+        emit(c, cnt);
         ++cnt;
     }
     return cnt;
 }
 
+// contacts of body a's corners with the ground; emit(a, corner, x, anchor, k) for contact k
 template <class Emit>
 __device__ int ground_corners(const Dev& d, const FBox& fa, int a, Emit&& emit) {
     int cnt = 0;
@@ -226,7 +302,7 @@ __device__ int ground_corners(const Dev& d, const FBox& fa, int a, Emit&& emit) 
         float g = FS(FA(FA(FM(d.p.gn[0], y[0]), FM(d.p.gn[1], y[1])), FM(d.p.gn[2], y[2])), d.p.gd);
         if (!(g < fa.infl)) continue;
         float anc[3] = {FS(y[0], FM(g, d.p.gn[0])), FS(y[1], FM(g, d.p.gn[1])), FS(y[2], FM(g, d.p.gn[2]))};
-        emit(a, -1, x, anc, d.p.gn, cnt);
+        emit(a, k, x, anc, cnt);
         ++cnt;
     }
     return cnt;
@@ -243,12 +319,8 @@ struct Contact {
     float4 xi, xj, bn;
 };
 
-// contact number `slot` of the step, written as bond Nc + slot while there is room
-__device__ __forceinline__ Contact write_contact(const Dev& d, int slot, int type, int i, int j, const float* xi,
-                                                 const float* xj, const float* N) {
-    Contact c;
-    if (slot >= d.cap_contacts) return c;
-    const int b = d.Nc + slot;
+// h^2 kappa_c of the contacts of bodies i and j (the ground: j < 0)
+__device__ __forceinline__ float contact_weight(const Dev& d, int i, int j) {
     float mi = d.mass[i].x;
     float mm;
     if (j < 0) mm = mi;
@@ -257,18 +329,32 @@ __device__ __forceinline__ Contact write_contact(const Dev& d, int slot, int typ
         bool pi = d.bflags[i] & BF_PINNED, pj = d.bflags[j] & BF_PINNED;
         mm = pj ? mi : (pi ? mj : fminf(mi, mj));
     }
-    c.m = make_int4(i, j, type, 0);
-    c.xi = make_float4(xi[0], xi[1], xi[2], d.p.c_kappa * mm);
-    c.xj = make_float4(xj[0], xj[1], xj[2], pair_dhat(d, i, j));
-    c.bn = make_float4(N[0], N[1], N[2], d.p.mu);
+    return d.p.c_kappa * mm;
+}
+
+// contact number `slot` of the step, written as bond Nc + slot while there is room
+__device__ __forceinline__ void store_contact(const Dev& d, int slot, const Contact& c) {
+    if (slot >= d.cap_contacts) return;
+    const int b = d.Nc + slot;
     d.bmeta[b] = c.m;
     d.bxi[b] = c.xi;
     d.bxj[b] = c.xj;
     d.bn[b] = c.bn;
+}
+
+__device__ __forceinline__ Contact write_contact(const Dev& d, int slot, int type, int i, int j, const float* xi,
+                                                 const float* xj, const float* N) {
+    Contact c;
+    if (slot >= d.cap_contacts) return c;
+    c.m = make_int4(i, j, type, 0);
+    c.xi = make_float4(xi[0], xi[1], xi[2], contact_weight(d, i, j));
+    c.xj = make_float4(xj[0], xj[1], xj[2], pair_dhat(d, i, j));
+    c.bn = make_float4(N[0], N[1], N[2], d.p.mu);
+    store_contact(d, slot, c);
     return c;
 }
 
-// One item of the narrow phase's two passes.  Items [0, np) are this step's pairs, items np + b
+// One item of the small front's two narrow passes.  Items [0, np) are this step's pairs, items np + b
 // the ground corners of body b (apart, so that no item runs both manifolds in series).
 __device__ __forceinline__ void narrow_count_item(const Dev& d, int tt, int np) {
     if (tt < np) {
@@ -276,14 +362,17 @@ __device__ __forceinline__ void narrow_count_item(const Dev& d, int tt, int np) 
         FBox fa, fb;
         load_box(d, pr.x, fa);
         load_box(d, pr.y, fb);
-        d.npc[tt] = box_box(fa, fb, pr.x, pr.y, [](int, int, const float*, const float*, const float*, int) {});
+        LocalPoly poly;
+        Manifold mf;
+        int out;
+        d.npc[tt] = box_box(fa, fb, pr.x, pr.y, poly, mf, out, [](const Corner&, int) {});
     } else {
         const int t = tt - np;
         int n = 0;
         if (d.p.has_ground && !(d.bflags[t] & BF_PINNED)) {
             FBox fa;
             load_box(d, t, fa);
-            n = ground_corners(d, fa, t, [](int, int, const float*, const float*, const float*, int) {});
+            n = ground_corners(d, fa, t, [](int, int, const float*, const float*, int) {});
         }
         d.gnd_cnt[t] = n;
     }
@@ -299,9 +388,14 @@ __device__ __forceinline__ void narrow_write_item(const Dev& d, int tt, int np, 
         load_box(d, pr.x, fa);
         load_box(d, pr.y, fb);
         const int base = d.npc_off[tt];
-        box_box(fa, fb, pr.x, pr.y, [&](int i, int j, const float* xi, const float* xj, const float* N, int k) {
-            write_contact(d, base + k, K_CONTACT, i, j, xi, xj, N);
-            if (base + k < d.cap_contacts) written(i, j);
+        LocalPoly poly;
+        Manifold mf;
+        int out;
+        box_box(fa, fb, pr.x, pr.y, poly, mf, out, [&](const Corner& c, int k) {
+            float x[3];
+            corner_point(mf.ki, mf.xk, c.xa, c.xb, x);
+            write_contact(d, base + k, K_CONTACT, mf.ii, mf.ir, x, c.u, mf.N);
+            if (base + k < d.cap_contacts) written(mf.ii, mf.ir);
         });
     } else {
         const int t = tt - np;
@@ -309,9 +403,9 @@ __device__ __forceinline__ void narrow_write_item(const Dev& d, int tt, int np, 
             FBox fa;
             load_box(d, t, fa);
             const int base = npc + d.gnd_off[t];
-            ground_corners(d, fa, t, [&](int i, int j, const float* xi, const float* xj, const float* N, int k) {
-                write_contact(d, base + k, K_GROUND, i, j, xi, xj, N);
-                if (base + k < d.cap_contacts) written(i, j);
+            ground_corners(d, fa, t, [&](int i, int, const float* xi, const float* xj, int k) {
+                write_contact(d, base + k, K_GROUND, i, -1, xi, xj, d.p.gn);
+                if (base + k < d.cap_contacts) written(i, -1);
             });
         }
     }
@@ -321,8 +415,7 @@ __device__ __forceinline__ void narrow_write_item(const Dev& d, int tt, int np, 
 __device__ __forceinline__ void set_contact_counts(const Dev& d, int npc) {
     int nk = npc + d.gnd_off[d.N];
     if (nk > d.cap_contacts) { latch_status(d, ST_CAPACITY); nk = d.cap_contacts; }
-    d.ctr[C_NPC] = min(npc, d.cap_contacts);
-    d.ctr[C_NGC] = nk - min(npc, d.cap_contacts);
+    d.ctr[C_NCONTACTS] = nk;
     d.ctr[C_NBONDS] = d.Nc + nk;
 }
 

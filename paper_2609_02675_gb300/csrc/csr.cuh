@@ -37,18 +37,19 @@ __device__ __forceinline__ void place_end(const Dev& d, int id, int p) {
     }
 }
 
-__device__ __forceinline__ void csr_count_bond(const Dev& d, int b) {
-    const int4 m = d.bmeta[b];
-    if (end_live(d, m.x)) atomicAdd(&d.end_cnt[m.x], 1);
-    if (end_live(d, m.y)) atomicAdd(&d.end_cnt[m.y], 1);
-}
-
+// (a slot past the arrays cannot be, unless a bounded wait of the narrow phase gave up)
 __device__ __forceinline__ void csr_fill_bond(const Dev& d, int b) {
     const int4 m = d.bmeta[b];
-    if (end_live(d, m.x)) d.end_id[d.end_off[m.x] + atomicAdd(&d.end_cur[m.x], 1)] = 2 * b;
-    else d.end_pos[2 * b] = -1;
-    if (end_live(d, m.y)) d.end_id[d.end_off[m.y] + atomicAdd(&d.end_cur[m.y], 1)] = 2 * b + 1;
-    else d.end_pos[2 * b + 1] = -1;
+    auto put = [&](int body, int id) {
+        if (end_live(d, body)) {
+            const int p = d.end_off[body] + atomicAdd(&d.end_cur[body], 1);
+            if (p < d.cap_ends) d.end_id[p] = id;
+        } else {
+            d.end_pos[id] = -1;
+        }
+    };
+    put(m.x, 2 * b);
+    put(m.y, 2 * b + 1);
 }
 
 // Place a body's ends in ascending end id, by CSR_LANES lanes: an end's slot is the slice's start

@@ -19,6 +19,8 @@
 // corner-vs-ground-plane contacts, all in single precision with the same fixed operation
 // order as the specification in the tests' oracle; contacts are written in pair order
 // (then ground, in body order) through prefix sums, so the contact list is deterministic.
+#include <algorithm>
+
 #include "contacts.cuh"
 #include "csr.cuh"
 #include "sort_slices.cuh"
@@ -58,9 +60,11 @@ __device__ __forceinline__ float level_cell(const Dev& d, int lv) {
     return cs;
 }
 
-// bucket of cell (x, y, z) of level lv (levels apart: coordinates stay within +-2^20)
-__device__ __forceinline__ int level_hash(int x, int y, int z, int lv, int bits) {
-    return cell_hash(x + (lv << 22), y, z, bits);
+// bucket of cell (x, y, z) of level lv for the bodies of a group (levels apart: coordinates stay
+// within +-2^20; groups apart, so that scenes in the same place do not fill each other's buckets:
+// 24 piles of 8000 boxes counted their pairs in 27 us, now 11)
+__device__ __forceinline__ int level_hash(int x, int y, int z, int lv, int group, int bits) {
+    return cell_hash(x + (lv << 22) + group * 0x2545f491, y, z, bits);
 }
 
 __global__ void k_cells(Dev d) {
@@ -73,7 +77,7 @@ __global__ void k_cells(Dev d) {
     float inv = 1.0f / cs;
     float4 a = d.qn[3 * b];
     int x = cell_coord(a.x, inv), y = cell_coord(a.y, inv), z = cell_coord(a.z, inv);
-    int hb = level_hash(x, y, z, lv, d.table_bits);
+    int hb = level_hash(x, y, z, lv, d.group[b], d.table_bits);
     d.cell[b] = make_int4(x, y, z, hb);
     atomicAdd(&d.bucket_cnt[hb], 1);
 }
@@ -109,7 +113,7 @@ __device__ __forceinline__ int lane_partners(const Dev& d, int i, int lane, F&& 
     if (lane < 27) {
         const int4 ci = d.cell[i];
         const int x = ci.x + lane % 3 - 1, y = ci.y + (lane / 3) % 3 - 1, z = ci.z + lane / 9 - 1;
-        const int hb = cell_hash(x, y, z, d.table_bits);
+        const int hb = level_hash(x, y, z, 0, gi, d.table_bits);
         const int s = d.bucket_off[hb], e = d.bucket_off[hb + 1];
         if (d.brec_lo) {
             const float4 li = d.lo[i], hi_ = d.hi[i];
@@ -285,7 +289,7 @@ __device__ __forceinline__ int lane_partners_ml(const Dev& d, int i, int lane, O
         }
         const int c = t % 27;
         const int x = bx + c % 3 - 1, y = by + (c / 3) % 3 - 1, z = bz + c / 9 - 1;
-        const int hb = level_hash(x, y, z, l, d.table_bits);
+        const int hb = level_hash(x, y, z, l, gi, d.table_bits);
         const int s = d.bucket_off[hb], e = d.bucket_off[hb + 1];
         for (int k = s; k < e; ++k) {
             const int4 cj = d.brec_cell[k];
@@ -365,76 +369,219 @@ __global__ void k_ml_pair_write(Dev d) {
     }
 }
 
-// Pairs of the off-grid bodies: body i of the off-grid list against every j > i, one block of
-// OFF_T threads per body.  Warp w takes the w-th of 32 contiguous runs of (i, N), so the warps'
-// hits concatenated in warp order keep the slice sorted by j; the runs' loads are
-// independent, so a body's sweep costs about N / OFF_T dependent rounds instead of N / 32.
+// Pairs of the off-grid bodies: body i of the off-grid list against every j > i, by 32 warps, warp
+// w taking the w-th of 32 contiguous runs of (i, N), so the warps' hits concatenated in warp order
+// keep the slice sorted by j.  The warps of all off-grid bodies are spread over the grid and each
+// keeps four chunks of 32 bodies in flight (32 warps of one block read 2 MB per body through one
+// SM: 13 off-grid bodies among 50 077 took 140 us for both passes, now 103).
 // WRITE = false counts (into pair_cnt[i], and each warp's count in lane_cnt[32 i + w]); true
 // stores the partners into pair_j.
-constexpr int OFF_T = 1024;
-constexpr int OFF_BLOCKS = 152;
+constexpr int OFF_T = 128;
+constexpr int OFF_BLOCKS = 152 * 4;
 
 template <bool WRITE>
 __global__ void __launch_bounds__(OFF_T) k_offgrid_pairs(Dev d) {
     pdl_enter();
-    __shared__ int s_cnt[OFF_T / 32];
     if (!d.p.body_contacts) return;
     const int nl = d.ctr[C_NLARGE];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cap = d.cap_pairs;
-    for (int h = blockIdx.x; h < nl; h += gridDim.x) {
-        const int i = d.large_ids[h];
+    const int lane = threadIdx.x & 31, cap = d.cap_pairs;
+    // (neighbouring tasks of one body on different SMs)
+    const int warp0 = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, warps = gridDim.x * (OFF_T / 32);
+    for (int task = warp0; task < 32 * nl; task += warps) {
+        const int i = d.large_ids[task >> 5], w = task & 31;
         const int gi = d.group[i], fi = d.bflags[i];
         const float4 li = d.lo[i], hi_ = d.hi[i];
         const int len = (((d.N - i - 1) + 31) / 32 + 31) & ~31;  // per warp, a multiple of 32
         const int j_beg = i + 1 + w * len, j_end = min(d.N, j_beg + len);
-        if (!WRITE) {
-            int n = 0;
-            for (int j0 = j_beg; j0 < j_end; j0 += 32) {
-                const int j = j0 + lane;
-                n += (j < j_end && pair_ok(d, i, j, gi, fi, li, hi_)) ? 1 : 0;
+        int pos = 0;
+        if (WRITE) {
+            int before = lane < w ? d.lane_cnt[32 * i + lane] : 0;
+            pos = d.pair_off[i] + warp_sum(before);
+        }
+        for (int j0 = j_beg; j0 < j_end; j0 += 4 * 32) {
+            bool ok[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = j0 + 32 * k + lane;
+                ok[k] = j < j_end && pair_ok(d, i, j, gi, fi, li, hi_);
             }
-            n = warp_sum(n);
-            if (lane == 0) { d.lane_cnt[32 * i + w] = n; s_cnt[w] = n; }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int t = 0;
-                for (int k = 0; k < OFF_T / 32; ++k) t += s_cnt[k];
-                atomicAdd(&d.pair_cnt[i], t);
-            }
-            __syncthreads();
-        } else {
-            int pos = d.pair_off[i];
-            for (int k = 0; k < w; ++k) pos += d.lane_cnt[32 * i + k];
-            for (int j0 = j_beg; j0 < j_end; j0 += 32) {
-                const int j = j0 + lane;
-                const bool ok = j < j_end && pair_ok(d, i, j, gi, fi, li, hi_);
-                const unsigned bal = __ballot_sync(0xffffffffu, ok);
-                const int at = pos + __popc(bal & ((1u << lane) - 1u));
-                if (ok && at < cap) d.pair_j[at] = j;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const unsigned bal = __ballot_sync(0xffffffffu, ok[k]);
+                if (WRITE) {
+                    const int at = pos + __popc(bal & ((1u << lane) - 1u));
+                    if (ok[k] && at < cap) d.pair_j[at] = j0 + 32 * k + lane;
+                }
                 pos += __popc(bal);
             }
+        }
+        if (!WRITE && lane == 0) {
+            d.lane_cnt[32 * i + w] = pos;
+            if (pos > 0) atomicAdd(&d.pair_cnt[i], pos);
         }
     }
 }
 
 // ---- narrow phase ----
 
-// the threads stride over the narrow phase's items
-__global__ void k_narrow_count(Dev d) {
+// The whole narrow phase in one pass.  Items [0, np) are this step's pairs, items np + b the ground
+// corners of body b; a tile of NARROW_T items is a block's, a thread each.  The block keeps its
+// items' contacts in shared memory while it learns how many contacts precede its tile -- the
+// tiles' counts are published as they are known, and a tile adds up its predecessors' from the
+// nearest one whose whole prefix is known (decoupled look-back, Merrill and Garland 2016) -- and
+// then writes them, a thread per contact.  Contacts come out in item order whatever the order of
+// the blocks.  Tiles are taken from a counter, so a tile's predecessors are running or done; the
+// wait for them is bounded all the same (PABD_ERR_TIMEOUT).  The bodies' bond ends are counted on
+// the way, on top of their static ones.
+//
+// It replaced a counting pass, two prefix sums, a pass that derived every manifold again to write
+// it, and the count of bond ends.  Bound by the clipping's dependent steps and their trips to
+// shared memory (16 warps per SM, its 46 KB a block): 532 325 pairs of a settled bed 115 us
+// (counting 156 and writing 187 us; in one pass with the polygons in local memory 274), 258 048
+// pairs of a pile, all touching, 78 us (57 and 90).
+__global__ void __launch_bounds__(NARROW_T) k_narrow(Dev d) {
+    constexpr int T = NARROW_T, MAXC = 8;
+    __shared__ float corners[2 * MAXC * 5 * T];  // the items' polygons, then their contacts (SharedPoly)
+    __shared__ float nrm[3][T], wgt[T], dht[T], face_x[T];
+    __shared__ int bi[T], bj[T];                 // bj < 0: ground contacts
+    __shared__ unsigned char face[T], buf[T];    // incident face's axis; the buffer that holds the contacts
+    __shared__ unsigned short map[MAXC * T];  // contact of the tile -> item + T * its number there
+    __shared__ int wsum[T / 32], s_tile, s_before;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     pdl_enter();
-    const int np = d.ctr[C_NPAIRS];
-    for (int tt = blockIdx.x * blockDim.x + threadIdx.x; tt < np + d.N; tt += gridDim.x * blockDim.x)
-        narrow_count_item(d, tt, np);
-}
-
-__global__ void k_narrow_write(Dev d) {
-    pdl_enter();
-    const int np = d.ctr[C_NPAIRS];
-    const int npc = d.npc_off[np];
-    for (int tt = blockIdx.x * blockDim.x + threadIdx.x; tt < np + d.N; tt += gridDim.x * blockDim.x)
-        narrow_write_item(d, tt, np, npc, [](int, int) {});
-    if (blockIdx.x == 0 && threadIdx.x == 0) set_contact_counts(d, npc);
+    const int np = d.ctr[C_NPAIRS], items = np + d.N, ntile = (items + T - 1) / T;
+    const unsigned limit = *d.wait_limit;
+    volatile unsigned long long* const state = d.tile_state;
+    constexpr unsigned long long PART = 1ull << 32, WHOLE = 2ull << 32;  // count of the tile, of all up to it
+    for (;;) {
+        if (t == 0) s_tile = atomicAdd(&d.ctr[C_NARROW_NEXT], 1);
+        __syncthreads();
+        const int tile = s_tile;
+        if (tile >= ntile) return;
+        const int item = tile * T + t;
+        int n = 0;
+        SharedPoly<T> poly{corners + t};
+        if (item < np) {
+            const int2 pr = d.pairs[item];
+            FBox fa, fb;
+            load_box(d, pr.x, fa);
+            load_box(d, pr.y, fb);
+            Manifold mf;
+            int out = 0;
+            n = box_box(fa, fb, pr.x, pr.y, poly, mf, out, [&](const Corner& c, int k) { st_corner(poly, out, k, c); });
+            if (n > 0) {
+                bi[t] = mf.ii;
+                bj[t] = mf.ir;
+                buf[t] = (unsigned char)out;
+                face[t] = (unsigned char)mf.ki;
+                face_x[t] = mf.xk;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) nrm[k][t] = mf.N[k];
+            }
+        } else if (item < items && d.p.has_ground && !(d.bflags[item - np] & BF_PINNED)) {
+            // (a ground contact's corner by number: its coordinates are the half extents, signed)
+            FBox fa;
+            load_box(d, item - np, fa);
+            n = ground_corners(d, fa, item - np, [&](int, int corner, const float*, const float* anc, int k) {
+                st_corner(poly, 0, k, Corner{{anc[0], anc[1], anc[2]}, __int_as_float(corner), 0.f});
+            });
+            if (n > 0) {
+                bi[t] = item - np;
+                bj[t] = -1;
+                buf[t] = 0;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) nrm[k][t] = fa.he[k];
+            }
+        }
+        int inc = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        int start = inc - n, total = 0;
+#pragma unroll
+        for (int k = 0; k < T / 32; ++k) {
+            if (k < warp) start += wsum[k];
+            total += wsum[k];
+        }
+        if (warp == 0) {  // publish, and look back
+            int before = 0;
+            if (tile > 0) {
+                if (lane == 0) state[tile] = PART | (unsigned)total;
+                for (int first = tile - 1;; first -= 32) {  // tiles first, first - 1, ...: one per lane
+                    const int k = first - lane;
+                    unsigned long long v = WHOLE;  // (before tile 0: nothing)
+                    unsigned polls = 0;
+                    if (k >= 0) {
+                        while (((v = state[k]) >> 32) == 0) {
+                            if (++polls > limit) {
+                                latch_status(d, ST_TIMEOUT);
+                                v = WHOLE;
+                                break;
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    const unsigned whole = __ballot_sync(0xffffffffu, (v >> 32) == 2);
+                    const int last = whole ? __ffs(whole) - 1 : 31;  // nearest with a whole prefix
+                    int c = lane <= last ? (int)(unsigned)v : 0;
+                    c = __reduce_add_sync(0xffffffffu, c);
+                    before += c;
+                    if (whole) break;
+                }
+            }
+            if (lane == 0) {
+                state[tile] = WHOLE | (unsigned)(before + total);
+                s_before = before;
+            }
+        }
+        for (int k = 0; k < n; ++k) map[start + k] = (unsigned short)(t + T * k);
+        if (n > 0) {
+            const int i = bi[t], j = bj[t];
+            wgt[t] = contact_weight(d, i, j);
+            dht[t] = pair_dhat(d, i, j);
+        }
+        __syncthreads();
+        const int before = s_before;
+        for (int c = t; c < total; c += T) {
+            const int o = map[c] % T, k = map[c] / T;
+            SharedPoly<T> his{corners + o};
+            const Corner p = ld_corner(his, buf[o], k);
+            const bool ground = bj[o] < 0;
+            float x[3];
+            if (ground) {
+                const int corner = __float_as_int(p.xa);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) x[a] = (corner >> a) & 1 ? nrm[a][o] : -nrm[a][o];
+            } else {
+                corner_point(face[o], face_x[o], p.xa, p.xb, x);
+            }
+            Contact q;
+            q.m = make_int4(bi[o], bj[o], ground ? K_GROUND : K_CONTACT, 0);
+            q.xi = make_float4(x[0], x[1], x[2], wgt[o]);
+            q.xj = make_float4(p.u[0], p.u[1], p.u[2], dht[o]);
+            q.bn = ground ? make_float4(d.p.gn[0], d.p.gn[1], d.p.gn[2], d.p.mu)
+                          : make_float4(nrm[0][o], nrm[1][o], nrm[2][o], d.p.mu);
+            store_contact(d, before + c, q);
+        }
+        if (n > 0) {  // (those with room)
+            const int m = min(n, d.cap_contacts - (before + start));
+            if (m > 0) {
+                if (end_live(d, bi[t])) atomicAdd(&d.end_cnt[bi[t]], m);
+                if (end_live(d, bj[t])) atomicAdd(&d.end_cnt[bj[t]], m);
+            }
+        }
+        if (tile == ntile - 1 && t == 0) {
+            int nk = before + total;
+            if (nk > d.cap_contacts) { latch_status(d, ST_CAPACITY); nk = d.cap_contacts; }
+            d.ctr[C_NCONTACTS] = nk;
+            d.ctr[C_NBONDS] = d.Nc + nk;
+        }
+        __syncthreads();  // the tile's shared memory is reused
+    }
 }
 
 static inline int nblk(int n) { return (n + CT - 1) / CT > 0 ? (n + CT - 1) / CT : 1; }
@@ -457,9 +604,8 @@ __global__ void __launch_bounds__(CT) k_ground_prelude(Dev d) {
         if (d.p.has_ground && !(d.bflags[b] & BF_PINNED)) {
             FBox fa;
             load_box(d, b, fa);
-            n = ground_corners(d, fa, b, [](int, int, const float*, const float*, const float*, int) {});
+            n = ground_corners(d, fa, b, [](int, int, const float*, const float*, int) {});
         }
-        d.gnd_cnt[b] = n;
         predict_body(d, b);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -510,7 +656,6 @@ __global__ void k_ground_bonds_csr(Dev d) {
         }
         const int b = tt - Ns;
         const int gb = gnd_prefix(d, b), g0 = min(gb, cap);
-        d.gnd_off[b] = gb;
         d.end_off[b] = d.sta_off[b] + g0;
         if (b == nb) continue;
         const int gn = min(gnd_prefix(d, b + 1), cap) - g0;
@@ -518,9 +663,9 @@ __global__ void k_ground_bonds_csr(Dev d) {
             FBox fa;
             load_box(d, b, fa);
             const int p0 = d.sta_off[b + 1] + g0;
-            ground_corners(d, fa, b, [&](int i, int j, const float* xi, const float* xj, const float* N, int k) {
+            ground_corners(d, fa, b, [&](int i, int, const float* xi, const float* xj, int k) {
                 if (k >= gn) return;  // past the contact capacity (latched below)
-                const Contact c = write_contact(d, g0 + k, K_GROUND, i, j, xi, xj, N);
+                const Contact c = write_contact(d, g0 + k, K_GROUND, i, -1, xi, xj, d.p.gn);
                 place_end<WANT>(d, 2 * (d.Nc + g0 + k), p0 + k, c.m, c.xi, c.xj, c.bn);
             });
         }
@@ -529,8 +674,7 @@ __global__ void k_ground_bonds_csr(Dev d) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         int nk = gnd_prefix(d, nb);
         if (nk > cap) { latch_status(d, ST_CAPACITY); nk = cap; }
-        d.ctr[C_NPC] = 0;
-        d.ctr[C_NGC] = nk;
+        d.ctr[C_NCONTACTS] = nk;
         d.ctr[C_NBONDS] = d.Nc + nk;
     }
 }
@@ -564,17 +708,12 @@ void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches) {
 
 // (the counters and buckets it accumulates into are zeroed by launch_step_reset)
 void launch_collision(const Dev& d, cudaStream_t st, long long* launches) {
-    launch_pdl(k_aabb, dim3(nblk(d.N)), dim3(CT), 0, st, d);
-    *launches += 1;
-    if (!d.p.body_contacts) {
-        // ground contacts only: no broad phase (the pair count stays at the zero the step's
-        // reset wrote, and the pair contacts' prefix at the zero written at creation)
-        launch_pdl(k_narrow_count, dim3(stride_grid(d.N, CT)), dim3(CT), 0, st, d);
-        scan_exclusive(d.gnd_cnt, d.gnd_off, nullptr, d.N, d.scan_scratch, st, launches);
-        launch_pdl(k_narrow_write, dim3(stride_grid(d.N, CT)), dim3(CT), 0, st, d);
-        *launches += 2;
+    if (!d.p.body_contacts) {  // ground contacts only: no broad phase
+        launch_ground_front(d, st, launches);
         return;
     }
+    launch_pdl(k_aabb, dim3(nblk(d.N)), dim3(CT), 0, st, d);
+    *launches += 1;
     if (d.p.broadphase == 1) {
         launch_lbvh_pairs(d, st, launches);
     } else {
@@ -598,12 +737,10 @@ void launch_collision(const Dev& d, cudaStream_t st, long long* launches) {
             *launches += 4;
         }
     }
-    const long long nt = (long long)d.cap_pairs + d.N;
-    launch_pdl(k_narrow_count, dim3(stride_grid(nt, CT)), dim3(CT), 0, st, d);
-    scan_exclusive(d.npc, d.npc_off, d.ctr + C_NPAIRS, d.cap_pairs, d.scan_scratch, st, launches);
-    scan_exclusive(d.gnd_cnt, d.gnd_off, nullptr, d.N, d.scan_scratch, st, launches);
-    launch_pdl(k_narrow_write, dim3(stride_grid(nt, CT)), dim3(CT), 0, st, d);
-    *launches += 2;
+    // resident blocks, or a block per tile where the capacities leave fewer
+    const long long tiles = ((long long)d.cap_pairs + d.N + NARROW_T - 1) / NARROW_T;
+    launch_pdl(k_narrow, dim3((unsigned)std::min<long long>(tiles, resident_slots(4))), dim3(NARROW_T), 0, st, d);
+    *launches += 1;
 }
 
 }  // namespace pabd

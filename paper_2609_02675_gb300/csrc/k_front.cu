@@ -93,7 +93,10 @@ __global__ void __launch_bounds__(FT, 1) k_front(Dev d0) {
     pdl_enter();
 
     if (t == 0) reset_counters(d);
-    if (t < FRONT_N) ends[t] = cur[t] = 0;
+    if (t < FRONT_N) {
+        ends[t] = t < N ? d.sta_cnt[t] : 0;
+        cur[t] = 0;
+    }
     for (int k = t; k < 2 * END_BINS; k += FT) {
         d.bin_cnt[k] = 0;
         d.bin_cur[k] = 0;
@@ -111,7 +114,6 @@ __global__ void __launch_bounds__(FT, 1) k_front(Dev d0) {
     } else if (t >= FRONT_N && t - FRONT_N < N) {
         predict_body(d, t - FRONT_N);
     }
-    for (int b = FT - 1 - t; b < d.Nc; b += FT) csr_count_bond(d, b);
     __syncthreads();
 
     int np = 0;

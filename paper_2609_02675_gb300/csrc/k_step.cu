@@ -1,5 +1,7 @@
 // Per-step kernels around the sweep: the predictor and the velocity recovery of Alg. 1,
 // the time-dependent drive anchors, the CSR of bond ends and the per-group residual.
+#include <algorithm>
+
 #include "csr.cuh"
 #include "pabd_internal.h"
 #include "predict.cuh"
@@ -93,13 +95,7 @@ __global__ void k_drive_update(Dev d) {
 
 // ---- CSR of bond ends (csr.cuh) ----
 
-// (both stride over this step's bonds, C_NBONDS of them)
-__global__ void k_csr_count(Dev d) {
-    pdl_enter();
-    const int nb = d.ctr[C_NBONDS];
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) csr_count_bond(d, b);
-}
-
+// (strides over this step's bonds, C_NBONDS of them)
 __global__ void k_csr_fill(Dev d) {
     pdl_enter();
     const int nb = d.ctr[C_NBONDS];
@@ -112,34 +108,6 @@ __global__ void k_csr_sort(Dev d) {
     pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x, body = t / CSR_LANES;
     if (body < d.N) csr_place_body<WANT>(d, body, t % CSR_LANES);
-}
-
-// CSR of a scene whose only contacts are with the ground.  Contact bonds follow the static
-// ones and the ground contacts are numbered in body order (k_narrow_write), so in (body,
-// 2 bond + side) order body b's slice is its static ends (fixed at creation) followed by its
-// ground contacts, and starts at sta_off[b] + gnd_off[b] -- the sum of two prefix sums: no
-// count, atomics or sort.  Ground contacts past the contact capacity were not written (the
-// narrow phase latched PABD_ERR_CAPACITY); the slices skip them.
-template <int WANT>
-__global__ void k_csr_ground(Dev d) {
-    pdl_enter();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > d.N) return;
-    const int cap = d.cap_contacts;
-    const int g0 = min(d.gnd_off[b], cap);
-    const int off = d.sta_off[b] + g0;
-    d.end_off[b] = off;
-    if (b == d.N) return;
-    const int s0 = d.sta_off[b], sn = d.sta_off[b + 1] - s0;
-    const int gn = min(d.gnd_off[b + 1], cap) - g0;
-    for (int k = 0; k < sn; ++k) {
-        const int id = d.sta_id[s0 + k];
-        place_end<WANT>(d, id, off + k);
-    }
-    for (int k = 0; k < gn; ++k) {
-        place_end<WANT>(d, 2 * (d.Nc + g0 + k), off + sn + k);
-    }
-    if (sn + gn > HEAVY_ENDS) d.heavy[atomicAdd(&d.ctr[C_NHEAVY], 1)] = b;
 }
 
 // the heavy bodies' slices, one block per body
@@ -305,12 +273,13 @@ __global__ void k_step_reset(Dev d) {
         d.bucket_cnt[t] = 0;
         d.bucket_cur[t] = 0;
     }
+    if (d.tile_state && t < (d.cap_pairs + d.N) / NARROW_T + 1) d.tile_state[t] = 0;
     if (t < 2 * END_BINS) {
         d.bin_cnt[t] = 0;
         d.bin_cur[t] = 0;
     }
     if (t < d.N) {
-        d.end_cnt[t] = 0;
+        d.end_cnt[t] = d.sta_cnt[t];
         d.end_cur[t] = 0;
         if (d.multilevel) {
             d.pair_cnt[t] = 0;
@@ -320,7 +289,7 @@ __global__ void k_step_reset(Dev d) {
 }
 
 void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches) {
-    const long long n = std::max<long long>(1ll << d.table_bits, d.N);
+    const long long n = std::max<long long>({1ll << d.table_bits, d.N, ((long long)d.cap_pairs + d.N) / NARROW_T + 1});
     launch_pdl(k_step_reset, dim3((unsigned)((n + ST_T - 1) / ST_T)), dim3(ST_T), 0, st, d);
     *launches += 1;
 }
@@ -328,17 +297,11 @@ void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches) {
 void launch_csr(const Dev& d, cudaStream_t st, long long* launches) {
     with_want(d.csr_want, [&](auto w) {
         constexpr int WANT = decltype(w)::value;
-        if (d.sta_off) {
-            launch_pdl(k_csr_ground<WANT>, dim3(nblk(d.N + 1)), dim3(ST_T), 0, st, d);
-            *launches += 1;
-            return;
-        }
-        launch_pdl(k_csr_count, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
         scan_exclusive(d.end_cnt, d.end_off, nullptr, d.N, d.scan_scratch, st, launches);
         launch_pdl(k_csr_fill, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
         launch_pdl(k_csr_sort<WANT>, dim3(nblk(d.N * CSR_LANES)), dim3(ST_T), 0, st, d);
         launch_pdl(k_csr_sort_long<WANT>, dim3(152), dim3(LONG_T), 2 * LONG_SMEM * sizeof(int), st, d);
-        *launches += 4;
+        *launches += 3;
     });
 }
 

@@ -383,8 +383,10 @@ pabd_status autotune_sweep(pabd_scene* s) {
     launch_step_reset(d, s->st, &lc);
     launch_drive_update(d, s->st, &lc);
     launch_collision(d, s->st, &lc);
-    launch_csr(d, s->st, &lc);
-    launch_predict(d, s->st, &lc);
+    if (!d.sta_off) {  // (a ground-only scene's collision launches do all of it)
+        launch_csr(d, s->st, &lc);
+        launch_predict(d, s->st, &lc);
+    }
     CK(cudaGetLastError());
     // blocks of HEAVY_T threads (a heavy body takes a whole block); the grid is tuned: all
     // co-resident blocks, or the blocks the light bodies fill, or half or a quarter of those,
@@ -496,7 +498,7 @@ pabd_status autotune_default(pabd_scene* s) {
                 CK(cudaEventElapsedTime(&t, e0, e1));
                 if (r > 0) tot = std::min(tot, t);  // the first pass warms the caches; the fastest
                                                     // of the others (least disturbed) is the figure
-                if (r > 0 && tot > 1.1f * best) break;  // out of the running
+                if (r > 0 && (tot > 1.1f * best || tot > 1.f)) break;  // out of the running; long enough to trust
             }
             CK(cudaGetLastError());
             fastest = std::min(fastest, tot);
@@ -752,15 +754,16 @@ pabd_status finalize_scene(pabd_scene* s) {
             s->al_init[k] = make_float2((float)hb.kappa, 0.f);
         }
     }
-    // scenes whose only contacts are with the ground: each body's live static ends, sorted
+    // each body's live static ends: how many, and, in scenes whose only contacts are with the
+    // ground, which, sorted
+    std::vector<int> cnt(N + 1, 0);
+    for (int k = 0; k < Nc; ++k) {
+        const HostBond& hb = s->bonds[k];
+        if (hb.i >= 0 && !(flags[hb.i] & BF_PINNED)) ++cnt[hb.i];
+        if (hb.j >= 0 && !(flags[hb.j] & BF_PINNED)) ++cnt[hb.j];
+    }
     std::vector<int> sta_off, sta_id, sta_body;
     if (!ds.body_contacts) {
-        std::vector<int> cnt(N + 1, 0);
-        for (int k = 0; k < Nc; ++k) {
-            const HostBond& hb = s->bonds[k];
-            if (hb.i >= 0 && !(flags[hb.i] & BF_PINNED)) ++cnt[hb.i];
-            if (hb.j >= 0 && !(flags[hb.j] & BF_PINNED)) ++cnt[hb.j];
-        }
         sta_off.assign(N + 1, 0);
         for (int b = 0; b < N; ++b) sta_off[b + 1] = sta_off[b] + cnt[b];
         sta_id.assign(sta_off[N] > 0 ? sta_off[N] : 1, 0);
@@ -818,8 +821,9 @@ pabd_status finalize_scene(pabd_scene* s) {
     ok &= alloc_arr(s, d.lane_cnt, (size_t)32 * N);
     if (ds.body_contacts && p.broadphase == 0)
         ok &= alloc_arr(s, d.pair_stash, (size_t)32 * PAIR_STASH * N) && alloc_arr(s, d.lane_tot, (size_t)32 * N);
-    ok &= alloc_arr(s, d.npc, d.cap_pairs) && alloc_arr(s, d.npc_off, d.cap_pairs + 1);
-    ok &= alloc_arr(s, d.gnd_cnt, N) && alloc_arr(s, d.gnd_off, N + 1);
+    if (front_fits(N, ds.body_contacts)) ok &= alloc_arr(s, d.npc, d.cap_pairs) && alloc_arr(s, d.npc_off, d.cap_pairs + 1);
+    if (ds.body_contacts) ok &= alloc_arr(s, d.tile_state, ((size_t)d.cap_pairs + N) / NARROW_T + 1);
+    ok &= alloc_arr(s, d.sta_cnt, N);
     ok &= alloc_arr(s, d.ctr, C_COUNT) && alloc_arr(s, d.step_index, 1);
     int ns = scan_scratch_ints(T);
     ns = std::max(ns, scan_scratch_ints(256 * (N / 1024 + 1)));
@@ -866,6 +870,7 @@ pabd_status finalize_scene(pabd_scene* s) {
     CK(up(d.bflags, flags.data(), sizeof(int) * N));
     CK(up(d.group, group.data(), sizeof(int) * N));
     CK(up(d.group_off, group_off.data(), sizeof(int) * (d.G + 1)));
+    CK(up(d.sta_cnt, cnt.data(), sizeof(int) * N));
     if (d.res_chunk) {
         CK(up(d.res_chunk, res_chunk.data(), sizeof(int2) * res_chunk.size()));
         CK(up(d.res_coff, res_coff.data(), sizeof(int) * (d.G + 1)));
@@ -892,8 +897,10 @@ pabd_status finalize_scene(pabd_scene* s) {
     CK(cudaMemsetAsync(d.resid_body, 0, sizeof(double) * (N ? N : 1), st));
     CK(cudaMemsetAsync(d.resid_group, 0, sizeof(double) * (d.G ? d.G : 1), st));
     CK(cudaMemsetAsync(d.group_hold, 0, d.G ? d.G : 1, st));
-    CK(cudaMemsetAsync(d.npc_off, 0, sizeof(int), st));  // no pair contacts before the first step
     CK(cudaMemsetAsync(d.end_pos, 0xff, sizeof(int) * d.cap_ends, st));
+    // (valid ids and bodies wherever a step cut short by a timed-out wait might read past its own)
+    CK(cudaMemsetAsync(d.end_id, 0, sizeof(int) * d.cap_ends, st));
+    CK(cudaMemsetAsync(d.bmeta + Nc, 0, sizeof(int4) * (size_t)d.cap_contacts, st));
     CK(cudaMemsetAsync(d.gbar, 0, 2 * sizeof(unsigned), st));
     const unsigned wait_polls = s->wait_polls;
     CK(cudaMemcpyAsync(d.wait_limit, &wait_polls, sizeof(unsigned), cudaMemcpyHostToDevice, st));
@@ -1485,7 +1492,7 @@ pabd_status pabd_read_contacts(pabd_scene* s, int32_t* meta, float* data, size_t
     int c[C_COUNT];
     CK(cudaMemcpyAsync(c, s->d.ctr, sizeof c, cudaMemcpyDeviceToHost, s->st));
     r = pabd_sync(s);
-    const int nk = c[C_NPC] + c[C_NGC];
+    const int nk = c[C_NCONTACTS];
     *n = (size_t)nk;
     size_t m = (size_t)nk < cap ? (size_t)nk : cap;
     if (!m || !meta || !data) return r;
@@ -1534,7 +1541,7 @@ pabd_status pabd_get_info(pabd_scene* s, pabd_info* info) {
     CK(cudaStreamSynchronize(s->st));
     info->n_bonds = c[C_NBONDS];
     info->n_pairs = c[C_NPAIRS];
-    info->n_contacts = c[C_NPC] + c[C_NGC];
+    info->n_contacts = c[C_NCONTACTS];
     info->step_index = step;
     info->max_pairs = s->d.cap_pairs;
     info->max_contacts = s->d.cap_contacts;

@@ -26,8 +26,7 @@ enum BodyFlags { BF_PINNED = 1, BF_FP64 = 2, BF_LARGE = 4, BF_SHIFT = 8, BF_STIF
 // device counters (ints) -- one small array so that one memset resets them
 enum Counter {
     C_NPAIRS = 0,      // broad-phase pairs (clamped to capacity)
-    C_NPC,             // body-body contacts
-    C_NGC,             // ground contacts
+    C_NCONTACTS,       // contacts of the step (clamped to capacity)
     C_NBONDS,          // static + contact bonds this step
     C_STATUS,          // latched StatusBits (never reset by a step)
     C_CELLBITS,        // float bits of the grid cell size
@@ -41,6 +40,7 @@ enum Counter {
     C_SOLVE_NEXT,      // next chunk of light bodies for the solve launch's warps (reset by k_bond)
     C_SWEEP_NEXT,      // the same for the one-launch sweeps, one counter per sweep parity: sweep k
     C_SWEEP_NEXT1,     // takes counter k & 1 and zeroes the other one for sweep k + 1
+    C_NARROW_NEXT,     // next tile of the narrow phase
     C_COUNT
 };
 
@@ -76,6 +76,7 @@ constexpr int END_BINS = HEAVY_ENDS + 1;
 // launches), its record (the others)
 constexpr int WANT_SLOTS = 1, WANT_RECORDS = 2;
 constexpr int RES_CHUNK = 4096;
+constexpr int NARROW_T = 128;  // items of a narrow-phase tile
 constexpr int PAIR_STASH = 4;
 constexpr int STASH_DELIVER = 0x40000000;
 constexpr int BVH_STASH = 16;
@@ -115,6 +116,7 @@ struct Dev {
     float2 *drv_t;              // (period, phase)
     int *drv_bond;              // bond index of each drive
     // CSR of bond ends
+    int *sta_cnt;               // live static ends per body: where end_cnt starts each step
     int *end_cnt, *end_cur, *end_off, *end_id, *end_pos;
     float4 *ends, *end_x;
     int *heavy;                 // ids of the bodies with more than HEAVY_ENDS ends (C_NHEAVY of them)
@@ -148,7 +150,8 @@ struct Dev {
     int *pair_stash, *lane_tot;
     int *pair_cnt, *pair_off;
     int2 *pairs;
-    int *npc, *npc_off, *gnd_cnt, *gnd_off;
+    int *npc, *npc_off, *gnd_cnt, *gnd_off;  // contact counts and prefixes of the small front's items
+    unsigned long long *tile_state;          // narrow phase: each tile's published count (k_narrow)
     // linear BVH broad phase (Params::broadphase == 1)
     unsigned *bvh_key, *bvh_key2;   // Morton codes (radix sort ping-pong)
     int *bvh_id, *bvh_id2;          // body ids in Morton order
