@@ -91,13 +91,10 @@ __global__ void k_bucket_fill(Dev d) {
     const int4 c = d.cell[b];
     if (c.w < 0) return;
     const int pos = d.bucket_off[c.w] + atomicAdd(&d.bucket_cur[c.w], 1);
-    d.bucket_items[pos] = b;
-    if (d.brec_lo) {
-        const float4 lo = d.lo[b], hi = d.hi[b];
-        d.brec_lo[pos] = make_float4(lo.x, lo.y, lo.z, __int_as_float(b));
-        d.brec_hi[pos] = make_float4(hi.x, hi.y, hi.z, __int_as_float(d.group[b]));
-        d.brec_cell[pos] = make_int4(c.x, c.y, c.z, d.bflags[b] | ((d.blevel ? d.blevel[b] : 0) << 8));
-    }
+    const float4 lo = d.lo[b], hi = d.hi[b];
+    d.brec_lo[pos] = make_float4(lo.x, lo.y, lo.z, __int_as_float(b));
+    d.brec_hi[pos] = make_float4(hi.x, hi.y, hi.z, __int_as_float(d.group[b]));
+    d.brec_cell[pos] = make_int4(c.x, c.y, c.z, d.bflags[b] | ((d.blevel ? d.blevel[b] : 0) << 8));
 }
 
 // Pair finding, one warp per body i.  A grid body: lane c < 27 scans neighbour cell c
@@ -115,27 +112,22 @@ __device__ __forceinline__ int lane_partners(const Dev& d, int i, int lane, F&& 
         const int x = ci.x + lane % 3 - 1, y = ci.y + (lane / 3) % 3 - 1, z = ci.z + lane / 9 - 1;
         const int hb = level_hash(x, y, z, 0, gi, d.table_bits);
         const int s = d.bucket_off[hb], e = d.bucket_off[hb + 1];
-        if (d.brec_lo) {
-            const float4 li = d.lo[i], hi_ = d.hi[i];
-            for (int k = s; k < e; ++k) {
-                const int4 cj = d.brec_cell[k];
-                const float4 lj = d.brec_lo[k], hj = d.brec_hi[k];
-                const int j = __float_as_int(lj.w);
-                if (j <= i || cj.x != x || cj.y != y || cj.z != z) continue;
-                if (__float_as_int(hj.w) != gi || ((fi & BF_PINNED) && (cj.w & BF_PINNED))) continue;
-                if (!overlap(li, hi_, lj, hj)) continue;
-                if (adj_has(d, i, j)) continue;
-                f(j, n);
-                ++n;
-            }
-        } else {
-            for (int k = s; k < e; ++k) {
-                const int j = d.bucket_items[k];
-                if (j <= i) continue;
-                const int4 cj = d.cell[j];
-                if (cj.x != x || cj.y != y || cj.z != z) continue;
-                if (pair_ok(d, i, j, gi, fi)) { f(j, n); ++n; }
-            }
+        const float4 li = d.lo[i], hi_ = d.hi[i];
+        auto test = [&](const int4& cj, const float4& lj, const float4& hj) {
+            const int j = __float_as_int(lj.w);
+            if (j <= i || cj.x != x || cj.y != y || cj.z != z) return;
+            if (__float_as_int(hj.w) != gi || ((fi & BF_PINNED) && (cj.w & BF_PINNED))) return;
+            if (!overlap(li, hi_, lj, hj)) return;
+            if (adj_has(d, i, j)) return;
+            f(j, n);
+            ++n;
+        };
+        for (int k = s; k < e; k += 2) {  // (two records in flight)
+            const int k1 = min(k + 1, e - 1);
+            const int4 c0 = d.brec_cell[k], c1 = d.brec_cell[k1];
+            const float4 l0 = d.brec_lo[k], l1 = d.brec_lo[k1], h0 = d.brec_hi[k], h1 = d.brec_hi[k1];
+            test(c0, l0, h0);
+            if (k + 1 < e) test(c1, l1, h1);
         }
     }
     const int nl = d.large_ids ? d.ctr[C_NLARGE] : 0;
@@ -165,87 +157,123 @@ __device__ __forceinline__ int warp_excl(int v, int lane) {
     return inc - v;
 }
 
-__global__ void k_pair_count(Dev d) {
+// Counts body i's partners (a warp per body) and, when there are at most PAIR_LIST of them and no
+// lane found more than four, leaves them in order in its list, so that writing the pairs is a
+// copy.
+__global__ void __launch_bounds__(CT) k_pair_count(Dev d) {
     pdl_enter();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    __shared__ int found[CT / 32][PAIR_LIST];
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (i >= d.N) return;
     int n = 0;
-    if (d.p.body_contacts) {
-        const int gi = d.group[i], fi = d.bflags[i];
-        if (d.cell[i].w < 0) {
-            const float4 li = d.lo[i], hi_ = d.hi[i];
-            for (int j0 = i + 1; j0 < d.N; j0 += 32) {
-                const int j = j0 + lane;
-                n += (j < d.N && pair_ok(d, i, j, gi, fi, li, hi_)) ? 1 : 0;
-            }
-        } else {
-            int* st = d.pair_stash ? d.pair_stash + (size_t)(32 * i + lane) * PAIR_STASH : nullptr;
-            n = lane_partners(d, i, lane, [&](int j, int k) { if (st && k < PAIR_STASH) st[k] = j; });
+    const int gi = d.group[i], fi = d.bflags[i];
+    if (d.cell[i].w < 0) {
+        const float4 li = d.lo[i], hi_ = d.hi[i];
+        for (int j0 = i + 1; j0 < d.N; j0 += 32) {
+            const int j = j0 + lane;
+            n += (j < d.N && pair_ok(d, i, j, gi, fi, li, hi_)) ? 1 : 0;
+        }
+        n = warp_sum(n);
+    } else {
+        int id[4];
+        const int mine = lane_partners(d, i, lane, [&](int j, int k) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (k == c) id[c] = j;
+        });
+        n = warp_sum(mine);
+        if (n > 0 && n <= PAIR_LIST && !__any_sync(0xffffffffu, mine > 4)) {
+            const int at = warp_excl(mine, lane);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (c < mine) found[w][at + c] = id[c];
+            __syncwarp();
+            const int v = lane < n ? found[w][lane] : 0x7fffffff;
+            const int r = warp_rank32(v, n, lane);
+            if (r >= 0) d.pair_list[(size_t)i * PAIR_LIST + r] = v;
+        } else if (n > 0 && lane == 0) {
+            d.pair_list[(size_t)i * PAIR_LIST] = -1;  // not listed: found again when written
         }
     }
-    if (d.lane_cnt) d.lane_cnt[32 * i + lane] = n;
-    n = warp_sum(n);
     if (lane == 0) d.pair_cnt[i] = n;
 }
 
-__global__ void k_pair_write(Dev d) {
-    pdl_enter();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (i >= d.N) return;
-    const int s = d.pair_off[i];
-    const int cap = d.cap_pairs;
-    if (d.p.body_contacts) {
-        const int gi = d.group[i], fi = d.bflags[i];
-        if (d.cell[i].w < 0) {
-            int pos = s;
-            const float4 li = d.lo[i], hi_ = d.hi[i];
-            for (int j0 = i + 1; j0 < d.N; j0 += 32) {
-                const int j = j0 + lane;
-                const bool ok = j < d.N && pair_ok(d, i, j, gi, fi, li, hi_);
-                const unsigned bal = __ballot_sync(0xffffffffu, ok);
-                const int at = pos + __popc(bal & ((1u << lane) - 1u));
-                if (ok && at < cap) d.pairs[at] = make_int2(i, j);
-                pos += __popc(bal);
-            }
-        } else {
-            const int mine = d.lane_cnt ? d.lane_cnt[32 * i + lane] : lane_partners(d, i, lane, [](int, int) {});
-            const int base = s + warp_excl(mine, lane);
-            if (d.pair_stash && d.lane_cnt && mine <= PAIR_STASH) {  // the partners found while counting
-                const int* st = d.pair_stash + (size_t)(32 * i + lane) * PAIR_STASH;
-                for (int k = 0; k < mine; ++k)
-                    if (base + k < cap) d.pairs[base + k] = make_int2(i, st[k]);
-            } else {
-                lane_partners(d, i, lane, [&](int j, int k) {
-                    if (base + k < cap) d.pairs[base + k] = make_int2(i, j);
-                });
-            }
-            __syncwarp();
-            const int e = min(d.pair_off[i + 1], cap);
-            if (e - s <= 32) {  // the slice sorted by j: each partner's rank among the slice
-                const int n = e - s;
-                const int j = lane < n ? d.pairs[s + lane].y : 0x7fffffff;
-                const int r = warp_rank32(j, n, lane);
-                __syncwarp();
-                if (r >= 0) d.pairs[s + r] = make_int2(i, j);
-            } else if (e - s <= 64) {  // by the bitonic network in registers
-                const int n = e - s;
-                int v0 = (2 * lane < n) ? d.pairs[s + 2 * lane].y : 0x7fffffff;
-                int v1 = (2 * lane + 1 < n) ? d.pairs[s + 2 * lane + 1].y : 0x7fffffff;
-                warp_sort64(v0, v1, lane);
-                if (2 * lane < n) d.pairs[s + 2 * lane] = make_int2(i, v0);
-                if (2 * lane + 1 < n) d.pairs[s + 2 * lane + 1] = make_int2(i, v1);
-            } else if (lane == 0) {
-                for (int a = s + 1; a < e; ++a) {  // insertion sort of the slice by j
-                    int2 v = d.pairs[a];
-                    int b = a - 1;
-                    while (b >= s && d.pairs[b].y > v.y) { d.pairs[b + 1] = d.pairs[b]; --b; }
-                    d.pairs[b + 1] = v;
-                }
-            }
+// The pairs of the bodies that were not listed while counting, by a warp: off-grid bodies (the
+// whole rest in order), and bodies with many partners (found again, then sorted).
+__device__ __forceinline__ void write_unlisted_pairs(const Dev& d, int i, int lane) {
+    const int s = d.pair_off[i], cap = d.cap_pairs;
+    const int gi = d.group[i], fi = d.bflags[i];
+    if (d.cell[i].w < 0) {
+        int pos = s;
+        const float4 li = d.lo[i], hi_ = d.hi[i];
+        for (int j0 = i + 1; j0 < d.N; j0 += 32) {
+            const int j = j0 + lane;
+            const bool ok = j < d.N && pair_ok(d, i, j, gi, fi, li, hi_);
+            const unsigned bal = __ballot_sync(0xffffffffu, ok);
+            const int at = pos + __popc(bal & ((1u << lane) - 1u));
+            if (ok && at < cap) d.pairs[at] = make_int2(i, j);
+            pos += __popc(bal);
+        }
+        return;
+    }
+    const int mine = lane_partners(d, i, lane, [](int, int) {});
+    const int base = s + warp_excl(mine, lane);
+    lane_partners(d, i, lane, [&](int j, int k) {
+        if (base + k < cap) d.pairs[base + k] = make_int2(i, j);
+    });
+    __syncwarp();
+    const int e = min(d.pair_off[i + 1], cap), n = e - s;
+    if (n <= 32) {  // the slice sorted by j: each partner's rank among the slice
+        const int j = lane < n ? d.pairs[s + lane].y : 0x7fffffff;
+        const int r = warp_rank32(j, n, lane);
+        __syncwarp();
+        if (r >= 0) d.pairs[s + r] = make_int2(i, j);
+    } else if (n <= 64) {  // by the bitonic network in registers
+        int v0 = (2 * lane < n) ? d.pairs[s + 2 * lane].y : 0x7fffffff;
+        int v1 = (2 * lane + 1 < n) ? d.pairs[s + 2 * lane + 1].y : 0x7fffffff;
+        warp_sort64(v0, v1, lane);
+        __syncwarp();
+        if (2 * lane < n) d.pairs[s + 2 * lane] = make_int2(i, v0);
+        if (2 * lane + 1 < n) d.pairs[s + 2 * lane + 1] = make_int2(i, v1);
+    } else if (lane == 0) {
+        for (int a = s + 1; a < e; ++a) {  // insertion sort of the slice by j
+            int2 v = d.pairs[a];
+            int b = a - 1;
+            while (b >= s && d.pairs[b].y > v.y) { d.pairs[b + 1] = d.pairs[b]; --b; }
+            d.pairs[b + 1] = v;
         }
     }
-    if (i == d.N - 1 && lane == 0) {
-        int tot = d.pair_off[d.N];
+}
+
+// Copies the listed partners, WRITE_LANES lanes per body; then each warp writes its bodies that
+// were not listed, one after the other.  (A warp per body that replayed every lane's finds took
+// 120 us for 262 144 boxes, and without room for them, in the allocation-free call, it scanned the
+// cells twice more: 50 us for 16 384 boxes.  Now 13 and 13.)
+constexpr int WRITE_LANES = 4;
+__global__ void __launch_bounds__(CT) k_pair_write(Dev d) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int i = t / WRITE_LANES, sub = t % WRITE_LANES, cap = d.cap_pairs;
+    bool unlisted = false;
+    if (i < d.N) {
+        const int s = d.pair_off[i], n = d.pair_off[i + 1] - s;
+        if (n > 0) {
+            const int* list = d.pair_list + (size_t)i * PAIR_LIST;
+            unlisted = d.cell[i].w < 0 || list[0] < 0;
+            if (!unlisted)
+                for (int k = sub; k < n; k += WRITE_LANES)
+                    if (s + k < cap) d.pairs[s + k] = make_int2(i, list[k]);
+        }
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, unlisted && sub == 0);
+    while (todo) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1;
+        write_unlisted_pairs(d, (t - lane + l) / WRITE_LANES, lane);
+        __syncwarp();
+    }
+    if (t == 0) {
+        const int tot = d.pair_off[d.N];
         if (tot > cap) latch_status(d, ST_CAPACITY);
         d.ctr[C_NPAIRS] = min(tot, cap);
     }
@@ -291,17 +319,22 @@ __device__ __forceinline__ int lane_partners_ml(const Dev& d, int i, int lane, O
         const int x = bx + c % 3 - 1, y = by + (c / 3) % 3 - 1, z = bz + c / 9 - 1;
         const int hb = level_hash(x, y, z, l, gi, d.table_bits);
         const int s = d.bucket_off[hb], e = d.bucket_off[hb + 1];
-        for (int k = s; k < e; ++k) {
-            const int4 cj = d.brec_cell[k];
-            const float4 lj = d.brec_lo[k], hj = d.brec_hi[k];
+        auto test = [&](const int4& cj, const float4& lj, const float4& hj) {
             const int j = __float_as_int(lj.w);
-            if (cj.x != x || cj.y != y || cj.z != z || (cj.w >> 8) != l || j == i) continue;
-            if (l == lvi && j < i) continue;  // same level: found by the smaller id
-            if (__float_as_int(hj.w) != gi || ((fi & BF_PINNED) && (cj.w & BF_PINNED))) continue;
-            if (!overlap(li, hi_, lj, hj)) continue;
-            if (adj_has(d, i, j)) continue;
+            if (cj.x != x || cj.y != y || cj.z != z || (cj.w >> 8) != l || j == i) return;
+            if (l == lvi && j < i) return;  // same level: found by the smaller id
+            if (__float_as_int(hj.w) != gi || ((fi & BF_PINNED) && (cj.w & BF_PINNED))) return;
+            if (!overlap(li, hi_, lj, hj)) return;
+            if (adj_has(d, i, j)) return;
             if (j > i) { own(j, n); ++n; }
             else deliver(j);
+        };
+        for (int k = s; k < e; k += 2) {  // (two records in flight)
+            const int k1 = min(k + 1, e - 1);
+            const int4 c0 = d.brec_cell[k], c1 = d.brec_cell[k1];
+            const float4 l0 = d.brec_lo[k], l1 = d.brec_lo[k1], h0 = d.brec_hi[k], h1 = d.brec_hi[k1];
+            test(c0, l0, h0);
+            if (k + 1 < e) test(c1, l1, h1);
         }
     }
     const int nl = d.ctr[C_NLARGE];
@@ -317,17 +350,17 @@ __global__ void k_ml_pair_count(Dev d) {
     pdl_enter();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= d.N || !d.p.body_contacts || d.cell[i].w < 0) return;
-    int* st = d.pair_stash ? d.pair_stash + (size_t)(32 * i + lane) * PAIR_STASH : nullptr;
+    int* st = d.pair_stash + (size_t)(32 * i + lane) * PAIR_STASH;
     int tot = 0;  // entries: own partners and deliveries, in the order found
     int n = lane_partners_ml(d, i, lane,
-        [&](int j, int) { if (st && tot < PAIR_STASH) st[tot] = j; ++tot; },
+        [&](int j, int) { if (tot < PAIR_STASH) st[tot] = j; ++tot; },
         [&](int j) {
             atomicAdd(&d.pair_cnt[j], 1);
-            if (st && tot < PAIR_STASH) st[tot] = j | STASH_DELIVER;
+            if (tot < PAIR_STASH) st[tot] = j | STASH_DELIVER;
             ++tot;
         });
     d.lane_cnt[32 * i + lane] = n;
-    if (d.lane_tot) d.lane_tot[32 * i + lane] = tot;
+    d.lane_tot[32 * i + lane] = tot;
     n = warp_sum(n);
     if (lane == 0) {
         d.pair_own[i] = n;
@@ -349,7 +382,7 @@ __global__ void k_ml_pair_write(Dev d) {
             const int at = d.pair_off[j] + d.pair_own[j] + atomicAdd(&d.pair_cur[j], 1);
             if (at < cap) d.pair_j[at] = i;
         };
-        const int tot = d.pair_stash && d.lane_tot ? d.lane_tot[32 * i + lane] : PAIR_STASH + 1;
+        const int tot = d.lane_tot[32 * i + lane];
         if (tot <= PAIR_STASH) {  // the entries found while counting
             const int* st = d.pair_stash + (size_t)(32 * i + lane) * PAIR_STASH;
             int k = 0;
@@ -373,7 +406,8 @@ __global__ void k_ml_pair_write(Dev d) {
 // w taking the w-th of 32 contiguous runs of (i, N), so the warps' hits concatenated in warp order
 // keep the slice sorted by j.  The warps of all off-grid bodies are spread over the grid and each
 // keeps four chunks of 32 bodies in flight (32 warps of one block read 2 MB per body through one
-// SM: 13 off-grid bodies among 50 077 took 140 us for both passes, now 103).
+// SM: 13 off-grid bodies among 50 077 took 140 us for both passes, now 29; spread but with the
+// pair filter's loads one after the other 103).
 // WRITE = false counts (into pair_cnt[i], and each warp's count in lane_cnt[32 i + w]); true
 // stores the partners into pair_j.
 constexpr int OFF_T = 128;
@@ -400,10 +434,18 @@ __global__ void __launch_bounds__(OFF_T) k_offgrid_pairs(Dev d) {
         }
         for (int j0 = j_beg; j0 < j_end; j0 += 4 * 32) {
             bool ok[4];
+            float4 lj[4], hj[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {  // (the boxes of all four chunks before any test)
+                const int j = min(j0 + 32 * k + lane, d.N - 1);
+                lj[k] = d.lo[j];
+                hj[k] = d.hi[j];
+            }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int j = j0 + 32 * k + lane;
-                ok[k] = j < j_end && pair_ok(d, i, j, gi, fi, li, hi_);
+                ok[k] = j < j_end && overlap(li, hi_, lj[k], hj[k]) && d.group[j] == gi &&
+                        !((fi & BF_PINNED) && (d.bflags[j] & BF_PINNED)) && !adj_has(d, i, j);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -702,7 +744,7 @@ void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches) {
     const int wblk = (d.N * 32 + CT - 1) / CT > 0 ? (d.N * 32 + CT - 1) / CT : 1;
     launch_pdl(k_pair_count, dim3(wblk), dim3(CT), 0, st, d);
     scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
-    launch_pdl(k_pair_write, dim3(wblk), dim3(CT), 0, st, d);
+    launch_pdl(k_pair_write, dim3(nblk(d.N * WRITE_LANES)), dim3(CT), 0, st, d);
     *launches += 5;
 }
 
@@ -733,7 +775,7 @@ void launch_collision(const Dev& d, cudaStream_t st, long long* launches) {
         } else {
             launch_pdl(k_pair_count, dim3(wblk), dim3(CT), 0, st, d);
             scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
-            launch_pdl(k_pair_write, dim3(wblk), dim3(CT), 0, st, d);
+            launch_pdl(k_pair_write, dim3(nblk(d.N * WRITE_LANES)), dim3(CT), 0, st, d);
             *launches += 4;
         }
     }

@@ -77,6 +77,7 @@ constexpr int END_BINS = HEAVY_ENDS + 1;
 constexpr int WANT_SLOTS = 1, WANT_RECORDS = 2;
 constexpr int RES_CHUNK = 4096;
 constexpr int NARROW_T = 128;  // items of a narrow-phase tile
+constexpr int PAIR_LIST = 16;  // partners listed per body by the single-level grid's count
 constexpr int PAIR_STASH = 4;
 constexpr int STASH_DELIVER = 0x40000000;
 constexpr int BVH_STASH = 16;
@@ -139,11 +140,12 @@ struct Dev {
     // collision
     float4 *lo, *hi;            // inflated AABB; lo.w = inflation
     int4 *cell;                 // cell coords (.w = bucket)
-    int *bucket_cnt, *bucket_cur, *bucket_off, *bucket_items;
+    int *bucket_cnt, *bucket_cur, *bucket_off;
     float4 *brec_lo, *brec_hi;  // per bucket slot: (lo, body id bits), (hi, group bits)
     int4 *brec_cell;            // per bucket slot: (cell x, y, z, flags)
-    int *lane_cnt;              // per body x 32 lanes: partners found by each lane
-    // per body x 32 lanes: the first PAIR_STASH partners each lane found while counting (a
+    int *pair_list;             // per body: its partners in order, if at most PAIR_LIST (k_pair_count)
+    int *lane_cnt;              // multilevel grid, per body x 32 lanes: partners found by each lane
+    // multilevel grid, per body x 32 lanes: the first PAIR_STASH partners each lane found while counting (a
     // partner delivered to a smaller id tagged by STASH_DELIVER), and the lane's number of
     // entries, so that writing the pairs replays them instead of scanning the cells again (a
     // lane with more rescans); null where the pair kernels run without them
