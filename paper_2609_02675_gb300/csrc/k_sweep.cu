@@ -69,12 +69,15 @@ __device__ __forceinline__ void bond_one(const Dev& d, const float4* __restrict_
 // holds room for every possible contact, far more than a step has).  Each thread loads its
 // first bond's static part before it waits for the previous sweep (pdl_enter), so that the
 // loads overlap that sweep's last blocks; q^k and the augmented Lagrangian state are read after.
+// The first sweep follows the step's front itself, in a small scene the launch that writes the
+// bonds and their slots: there nothing is read before the wait.
 __global__ void __launch_bounds__(BOND_T, 5) k_bond(Dev d, const float4* __restrict__ q, int it) {
+    if (it == 0) pdl_enter();
     const int nb = d.ctr[C_NBONDS];  // (set by the step's front, before the sweeps)
     const int b0 = blockIdx.x * blockDim.x + threadIdx.x;
     BondStatic s0;
     if (b0 < nb) s0 = bond_static(d, b0);
-    pdl_enter();
+    if (it > 0) pdl_enter();
     // the solve launch that follows hands out its light bodies from this counter (the previous
     // solve launch has finished: pdl_enter waited for it)
     if (blockIdx.x == 0 && threadIdx.x == 0) d.ctr[C_SOLVE_NEXT] = 0;
