@@ -11,14 +11,6 @@ namespace pabd {
 constexpr int ST_T = 256;
 static inline int nblk(int n) { return n > 0 ? (n + ST_T - 1) / ST_T : 1; }
 
-// the predictor of every body (predict_body)
-__global__ void k_predict(Dev d) {
-    pdl_enter();
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= d.N) return;
-    predict_body(d, b);
-}
-
 // Rotation matrix -> unit quaternion (Shepperd's method: divide by the largest of
 // 4w^2, 4x^2, 4y^2, 4z^2).
 __device__ __forceinline__ float4 mat_to_quat(const float* R) {
@@ -43,8 +35,8 @@ __device__ __forceinline__ float4 mat_to_quat(const float* R) {
 
 // Velocity recovery (Alg. 1, Sec. 4.4): v = (c^{n+1} - c^n)/h;
 // [w]x = skew part of (A^{n+1} - A^n)(A^n)^T / h; Q^{n+1} = quat(A^{n+1}), sign-continuous.
-__device__ __forceinline__ void finalize_body(const Dev& d, int b, const float4* __restrict__ qf) {
-    if ((d.bflags[b] & BF_PINNED) || held(d, b)) return;  // (a held group keeps its state)
+__device__ __forceinline__ void finalize_body(const Dev& d, int b, const float4* __restrict__ qf, bool hold) {
+    if ((d.bflags[b] & BF_PINNED) || hold) return;  // (a held group keeps its state)
     float4 n0 = d.qn[3 * b], n1 = d.qn[3 * b + 1], n2 = d.qn[3 * b + 2];
     float4 f0 = qf[3 * b], f1 = qf[3 * b + 1], f2 = qf[3 * b + 2];
     const float c0[3] = {n0.x, n0.y, n0.z}, c1[3] = {f0.x, f0.y, f0.z};
@@ -77,22 +69,6 @@ __device__ __forceinline__ void finalize_body(const Dev& d, int b, const float4*
     d.qn[3 * b] = f0; d.qn[3 * b + 1] = f1; d.qn[3 * b + 2] = f2;
 }
 
-__global__ void k_finalize(Dev d, const float4* __restrict__ qf, int dyn) {
-    pdl_enter();
-    // under a residual threshold the last iterate sits in the buffer of the sweep count's parity
-    if (dyn) qf = (d.sweep_ctl[0] & 1) ? d.qb : d.qa;
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b == 0) atomicAdd((unsigned long long*)d.step_index, 1ull);
-    if (b >= d.N) return;
-    finalize_body(d, b, qf);
-}
-
-__global__ void k_drive_update(Dev d) {
-    pdl_enter();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < d.Ndrive) drive_update(d, k);
-}
-
 // ---- CSR of bond ends (csr.cuh) ----
 
 // (strides over this step's bonds, C_NBONDS of them)
@@ -110,13 +86,20 @@ __global__ void k_csr_sort(Dev d) {
     if (body < d.N) csr_place_body<WANT>(d, body, t % CSR_LANES);
 }
 
-// the heavy bodies' slices, one block per body
+// The last launch before the sweeps: the first HEAVY_BLOCKS blocks place the heavy bodies' ends, a
+// body each at a time (csr_sort_heavy; k_csr_sort has listed them), the others take the predictor.
+// Neither reads what the other writes, and as two launches the second waited for the first.
 template <int WANT>
-__global__ void __launch_bounds__(LONG_T) k_csr_sort_long(Dev d) {
+__global__ void __launch_bounds__(LONG_T) k_predict(Dev d) {
     pdl_enter();
     extern __shared__ int key[];
-    const int nheavy = d.ctr[C_NHEAVY];
-    for (int h = blockIdx.x; h < nheavy; h += gridDim.x) csr_sort_heavy<LONG_T, WANT>(d, d.heavy[h], key);
+    if ((int)blockIdx.x < HEAVY_BLOCKS) {
+        const int nheavy = d.ctr[C_NHEAVY];
+        for (int h = blockIdx.x; h < nheavy; h += HEAVY_BLOCKS) csr_sort_heavy<LONG_T, WANT>(d, d.heavy[h], key);
+        return;
+    }
+    const int b = (blockIdx.x - HEAVY_BLOCKS) * LONG_T + threadIdx.x;
+    if (b < d.N) predict_body(d, b);
 }
 
 // ---- light bodies ordered by (class, end count) ----
@@ -208,7 +191,15 @@ constexpr int RES_T = 128;
 // tree, the warps in order (thread 0 returns it)
 __device__ __forceinline__ double block_resid_sum(const Dev& d, int s, int e, double* part) {
     double acc = 0.0;
-    for (int b = s + threadIdx.x; b < e; b += RES_T) acc += d.resid_body[b];
+    int b = s + threadIdx.x;
+    for (; b + 7 * RES_T < e; b += 8 * RES_T) {  // (eight loads in flight, added in order)
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = d.resid_body[b + k * RES_T];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc += v[k];
+    }
+    for (; b < e; b += RES_T) acc += d.resid_body[b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
@@ -219,17 +210,30 @@ __device__ __forceinline__ double block_resid_sum(const Dev& d, int s, int e, do
     return t;
 }
 
-// Scenes with a group of more than RES_CHUNK bodies: a block per chunk of at most RES_CHUNK
-// bodies of one group (Dev::res_chunk, the chunks of each group in order) sums it as
-// k_group_resid sums a group, then each group adds its chunks' sums in order.  A group of one
-// chunk gets k_group_resid's value bit for bit; a larger group is summed by as many blocks as it
-// has chunks instead of by one.
-__global__ void __launch_bounds__(RES_T) k_resid_chunks(Dev d) {
+// The velocity recovery, and beside it the groups' residuals, which depend on the sweeps alone: the
+// first blocks sum a group each -- in a scene with a group of more than RES_CHUNK bodies, a chunk
+// of at most RES_CHUNK bodies of one group (Dev::res_chunk, the chunks of each group in order),
+// whose sums k_resid_groups adds per group in order; a group of one chunk gets the group sum's
+// value bit for bit -- and the other blocks recover their bodies' velocities.  Under a residual
+// threshold (dyn) the sweeps' checks hold the residuals, and the last iterate sits in the buffer
+// of the sweep count's parity.
+__global__ void __launch_bounds__(RES_T) k_finalize(Dev d, const float4* __restrict__ qf, int resid_blocks, int dyn) {
     pdl_enter();
     __shared__ double part[RES_T / 32];
-    const int2 c = d.res_chunk[blockIdx.x];
-    const double t = block_resid_sum(d, c.x, c.y, part);
-    if (threadIdx.x == 0) d.res_part[blockIdx.x] = t;
+    const int k = blockIdx.x;
+    if (k < resid_blocks) {
+        const int2 c = d.res_chunk ? d.res_chunk[k] : make_int2(d.group_off[k], d.group_off[k + 1]);
+        const double t = block_resid_sum(d, c.x, c.y, part);
+        if (threadIdx.x == 0) {
+            if (d.res_chunk) d.res_part[k] = t;
+            else d.resid_group[k] = sqrt(t);
+        }
+        return;
+    }
+    if (dyn) qf = (d.sweep_ctl[0] & 1) ? d.qb : d.qa;
+    const int b = (k - resid_blocks) * RES_T + threadIdx.x;
+    if (b == 0) atomicAdd((unsigned long long*)d.step_index, 1ull);
+    if (b < d.N) finalize_body(d, b, qf, held(d, b));
 }
 
 __global__ void k_resid_groups(Dev d) {
@@ -241,35 +245,24 @@ __global__ void k_resid_groups(Dev d) {
     d.resid_group[g] = sqrt(t);
 }
 
-__global__ void __launch_bounds__(RES_T) k_group_resid(Dev d) {
-    pdl_enter();
-    __shared__ double part[RES_T / 32];
-    const int g = blockIdx.x;
-    if (g >= d.G) return;
-    const double t = block_resid_sum(d, d.group_off[g], d.group_off[g + 1], part);
-    if (threadIdx.x == 0) d.resid_group[g] = sqrt(t);
-}
-
 void launch_predict(const Dev& d, cudaStream_t st, long long* launches) {
-    launch_pdl(k_predict, dim3(nblk(d.N)), dim3(ST_T), 0, st, d);
-    *launches += 1;
-}
-
-void launch_drive_update(const Dev& d, cudaStream_t st, long long* launches) {
-    if (d.Ndrive == 0) return;
-    launch_pdl(k_drive_update, dim3(nblk(d.Ndrive)), dim3(ST_T), 0, st, d);
+    with_want(d.csr_want, [&](auto w) {
+        launch_pdl(k_predict<decltype(w)::value>, dim3(HEAVY_BLOCKS + (d.N + LONG_T - 1) / LONG_T), dim3(LONG_T),
+                   2 * LONG_SMEM * sizeof(int), st, d);
+    });
     *launches += 1;
 }
 
 // The per-step counters and scratch that the collision and CSR stages accumulate into, zeroed
 // by one kernel at the head of the step: no memset nodes between the step's kernels, so each
-// of them may launch while its predecessor runs.
+// of them may launch while its predecessor runs.  The drives' anchors, which nothing before the
+// CSR reads, are set here too.
 __global__ void k_step_reset(Dev d) {
     pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) reset_counters(d);
     if (d.bvh_bounds && t < 6) d.bvh_bounds[t] = t < 3 ? 0x7fffffff : (int)0x80000000;
-    if (d.p.broadphase == 0 && t < (1 << d.table_bits)) {
+    if (d.p.body_contacts && d.p.broadphase == 0 && t < (1 << d.table_bits)) {
         d.bucket_cnt[t] = 0;
         d.bucket_cur[t] = 0;
     }
@@ -286,10 +279,11 @@ __global__ void k_step_reset(Dev d) {
             d.pair_cur[t] = 0;
         }
     }
+    if (t < d.Ndrive) drive_update(d, t);
 }
 
 void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches) {
-    const long long n = std::max<long long>({1ll << d.table_bits, d.N, ((long long)d.cap_pairs + d.N) / NARROW_T + 1});
+    const long long n = std::max<long long>({d.p.body_contacts ? 1ll << d.table_bits : 0, d.N, d.Ndrive, 2 * END_BINS, ((long long)d.cap_pairs + d.N) / NARROW_T + 1});
     launch_pdl(k_step_reset, dim3((unsigned)((n + ST_T - 1) / ST_T)), dim3(ST_T), 0, st, d);
     *launches += 1;
 }
@@ -300,8 +294,7 @@ void launch_csr(const Dev& d, cudaStream_t st, long long* launches) {
         scan_exclusive(d.end_cnt, d.end_off, nullptr, d.N, d.scan_scratch, st, launches);
         launch_pdl(k_csr_fill, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
         launch_pdl(k_csr_sort<WANT>, dim3(nblk(d.N * CSR_LANES)), dim3(ST_T), 0, st, d);
-        launch_pdl(k_csr_sort_long<WANT>, dim3(152), dim3(LONG_T), 2 * LONG_SMEM * sizeof(int), st, d);
-        *launches += 3;
+        *launches += 2;
     });
 }
 
@@ -309,7 +302,7 @@ void launch_csr(const Dev& d, cudaStream_t st, long long* launches) {
 // idle and take one block slot per group; a larger group is better spread over the per-body
 // kernel): one warp per group recovers its bodies' velocities (finalize_body) and sums
 // their residuals.  Lane l plays the residual block's threads l, l + 32, ... (its RES_T / 32
-// accumulators), each accumulator is combined by the same xor tree and the results added in the
+// accumulators, one body each), each accumulator is combined by the same xor tree and the results added in the
 // same order -- the block's value bit for bit.
 __global__ void k_finalize_groups(Dev d, const float4* __restrict__ qf) {
     pdl_enter();
@@ -317,15 +310,19 @@ __global__ void k_finalize_groups(Dev d, const float4* __restrict__ qf) {
     if (g == 0 && lane == 0) atomicAdd((unsigned long long*)d.step_index, 1ull);
     if (g >= d.G) return;
     const int s = d.group_off[g], e = d.group_off[g + 1];
-    for (int b = s + lane; b < e; b += 32) finalize_body(d, b, qf);
+    const bool hold = d.group_hold[g] != 0;
+    // (the residuals' loads are in flight while the bodies are recovered)
     double acc[RES_T / 32];
 #pragma unroll
     for (int w = 0; w < RES_T / 32; ++w) {
-        acc[w] = 0.0;
-        for (int b = s + 32 * w + lane; b < e; b += RES_T) acc[w] += d.resid_body[b];
+        const int b = s + 32 * w + lane;
+        acc[w] = b < e ? d.resid_body[b] : 0.0;
+    }
+    for (int b = s + lane; b < e; b += 32) finalize_body(d, b, qf, hold);
+#pragma unroll
+    for (int w = 0; w < RES_T / 32; ++w)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc[w] += __shfl_xor_sync(0xffffffffu, acc[w], o);
-    }
     if (lane == 0) {
         double t = 0.0;
 #pragma unroll
@@ -340,15 +337,13 @@ void launch_finalize(const Dev& d, const float4* q_fin, cudaStream_t st, long lo
         *launches += 1;
         return;
     }
-    launch_pdl(k_finalize, dim3(nblk(d.N)), dim3(ST_T), 0, st, d, q_fin, 0);
+    const int resid = d.res_chunk ? d.n_res_chunks : d.G;
+    launch_pdl(k_finalize, dim3(resid + std::max(1, (d.N + RES_T - 1) / RES_T)), dim3(RES_T), 0, st, d, q_fin, resid, 0);
+    *launches += 1;
     if (d.res_chunk) {
-        launch_pdl(k_resid_chunks, dim3(d.n_res_chunks), dim3(RES_T), 0, st, d);
         launch_pdl(k_resid_groups, dim3(nblk(d.G)), dim3(ST_T), 0, st, d);
-        *launches += 3;
-        return;
+        *launches += 1;
     }
-    launch_pdl(k_group_resid, dim3(d.G > 0 ? d.G : 1), dim3(RES_T), 0, st, d);
-    *launches += 2;
 }
 
 // ---- sweeps under a residual threshold (Sec. 4.2 stopping rule, per scene) ----
@@ -361,7 +356,7 @@ __global__ void k_sweep_ctl_init(Dev d) {
 }
 
 // After a sweep: one block per scene still running computes that sweep's residual (the same
-// fixed reduction as k_group_resid); at most resid_tol stops the scene, else it counts as
+// fixed reduction as k_finalize's); at most resid_tol stops the scene, else it counts as
 // active.  The last block to finish (a ticket counter) runs the loop control: one more sweep
 // done, go on while a scene is active and fewer than n_iter sweeps ran; in a graph it also
 // sets the conditional node's value.  The decision depends only on integer counts.
@@ -418,7 +413,7 @@ void launch_sweep_check(const Dev& d, unsigned long long handle, cudaStream_t st
 }
 
 void launch_finalize_dynamic(const Dev& d, cudaStream_t st, long long* launches) {
-    launch_pdl(k_finalize, dim3(nblk(d.N)), dim3(ST_T), 0, st, d, nullptr, 1);
+    launch_pdl(k_finalize, dim3(std::max(1, (d.N + RES_T - 1) / RES_T)), dim3(RES_T), 0, st, d, nullptr, 0, 1);
     *launches += 1;
 }
 

@@ -192,6 +192,7 @@ __global__ void k_al_warm(Dev d) {
 
 // the dual update from the step's final iterate (after the last sweep), into parity n_iter
 __global__ void k_al_final(Dev d, const float4* __restrict__ q) {
+    pdl_enter();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= d.Nc) return;
     const int4 m = d.bmeta[b];
@@ -226,7 +227,7 @@ void launch_al_warm(const Dev& d, cudaStream_t st, long long* launches) {
 
 void launch_al_final(const Dev& d, const float4* q, cudaStream_t st, long long* launches) {
     if (d.Nal == 0) return;
-    k_al_final<<<(d.Nc + 255) / 256, 256, 0, st>>>(d, q);
+    launch_pdl(k_al_final, dim3((d.Nc + 255) / 256), dim3(256), 0, st, d, q);
     *launches += 1;
 }
 

@@ -271,7 +271,6 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
         mark();
     } else {
         launch_step_reset(d, s->st, launches);
-        launch_drive_update(d, s->st, launches);
         if (d.sta_off) {
             // ground-only scene: collision, CSR and predictor in one fused front (the predictor's
             // stage is then empty in the profiling graph's split)
@@ -381,7 +380,6 @@ pabd_status autotune_sweep(pabd_scene* s) {
     d.csr_want = WANT_RECORDS;
     long long lc = 0;
     launch_step_reset(d, s->st, &lc);
-    launch_drive_update(d, s->st, &lc);
     launch_collision(d, s->st, &lc);
     if (!d.sta_off) {  // (a ground-only scene's collision launches do all of it)
         launch_csr(d, s->st, &lc);
@@ -448,7 +446,6 @@ pabd_status autotune_default(pabd_scene* s) {
     Dev dd = d;
     dd.csr_want = WANT_SLOTS | WANT_RECORDS;
     launch_step_reset(dd, s->st, &lc);
-    launch_drive_update(dd, s->st, &lc);
     if (dd.sta_off) {
         launch_ground_front(dd, s->st, &lc);
     } else {
@@ -1338,7 +1335,6 @@ pabd_status pabd_detect(pabd_scene* s) {
     pabd_status r = finalize_scene(s);
     if (r != PABD_OK) return r;
     launch_step_reset(s->d, s->st, &s->launches);
-    launch_drive_update(s->d, s->st, &s->launches);
     launch_collision(s->d, s->st, &s->launches);
     CK(cudaGetLastError());
     return PABD_OK;

@@ -96,7 +96,7 @@ struct Dev {
     float4 *xs;                 // expansion point of the per-body system (x, y, z, 0), see sys_init
     int *bflags, *group, *group_off;
     int small_groups;           // every group has at most 128 bodies: one warp per group finalizes it
-    // a group of more than RES_CHUNK bodies: its residual summed by chunks (k_resid_chunks),
+    // a group of more than RES_CHUNK bodies: its residual summed by chunks (k_finalize),
     // (start, end) of each chunk, each group's first chunk, the chunks' sums; null otherwise
     int2 *res_chunk;
     int *res_coff;
@@ -257,7 +257,8 @@ void scan_exclusive(const int* in, int* out, const int* n_dev, int n_cap, int* s
                     long long* launches);
 int scan_scratch_ints(int n_cap);
 
-// zeroes the step's counters and accumulation scratch; precedes launch_collision / launch_csr
+// zeroes the step's counters and accumulation scratch and sets the drives' anchors; precedes
+// launch_collision / launch_csr
 void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches);
 void launch_collision(const Dev& d, cudaStream_t st, long long* launches);
 // the front of a step in a ground-only scene: collision, CSR and predictor (k_collision.cu)
@@ -274,6 +275,7 @@ void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches);
 void launch_csr(const Dev& d, cudaStream_t st, long long* launches);
 // the light bodies ordered by (class, end count) into Dev::order (after launch_csr)
 void launch_light_order(const Dev& d, cudaStream_t st, long long* launches);
+// the predictor, and the heavy bodies' ends placed (after launch_csr)
 void launch_predict(const Dev& d, cudaStream_t st, long long* launches);
 void launch_bond(const Dev& d, const float4* q, int it, cudaStream_t st, long long* launches);
 // augmented Lagrangian: warm start (before the sweeps) and the update after the last sweep
@@ -289,7 +291,6 @@ void launch_finalize(const Dev& d, const float4* q_fin, cudaStream_t st, long lo
 void launch_sweep_ctl_init(const Dev& d, cudaStream_t st, long long* launches);
 void launch_sweep_check(const Dev& d, unsigned long long handle, cudaStream_t st, long long* launches);
 void launch_finalize_dynamic(const Dev& d, cudaStream_t st, long long* launches);
-void launch_drive_update(const Dev& d, cudaStream_t st, long long* launches);
 // fused persistent sweep (all n_iter iterations, cooperative launch); L lanes per body
 cudaError_t launch_fused_sweep(const Dev& d, int L, int block, int grid, cudaStream_t st, long long* launches);
 int fused_max_blocks(int L, int block, bool fp64);
