@@ -472,7 +472,7 @@ pabd_status autotune_default(pabd_scene* s) {
         for (int threads : {s->lanes, half}) {
             if (threads == 0 || (in_bins && threads != s->lanes)) continue;
             float tot = 1e30f;
-            for (int r = 0; r < 5; ++r) {
+            for (int r = 0; r < 4; ++r) {
                 // the one-launch sweeps' chunk counters, as the step's reset leaves them (each
                 // sweep zeroes the next sweep's counter, so a pass must start from clean ones)
                 CK(cudaMemsetAsync(dd.ctr + C_SWEEP_NEXT, 0, 2 * sizeof(int), s->st));
@@ -495,7 +495,7 @@ pabd_status autotune_default(pabd_scene* s) {
                 CK(cudaEventElapsedTime(&t, e0, e1));
                 if (r > 0) tot = std::min(tot, t);  // the first pass warms the caches; the fastest
                                                     // of the others (least disturbed) is the figure
-                if (r > 0 && (tot > 1.1f * best || tot > 1.f)) break;  // out of the running; long enough to trust
+                if (r > 0 && (tot > 1.05f * best || tot > 1.f)) break;  // out of the running; long enough to trust
             }
             CK(cudaGetLastError());
             fastest = std::min(fastest, tot);
