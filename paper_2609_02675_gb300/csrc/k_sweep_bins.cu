@@ -207,7 +207,15 @@ cudaError_t setup_sweep_bins(const BinsShape& b, int lanes, bool f64, int* fit) 
         auto kernel = k_sweep_bins<decltype(l)::value, typename decltype(x)::type>;
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = bins_config(b, attr);
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+        // (the attribute is the kernel's, not the scene's: all that a block may have, whatever
+        // other scenes need; bins that need more fit nowhere)
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return;
+        const int most = 227 * 1024 - (int)fa.sharedSizeBytes;
+        *fit = 0;
+        if ((long long)cfg.dynamicSmemBytes > most) return;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess && b.cluster > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cfg.numAttrs = 1;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(fit, kernel, &cfg);

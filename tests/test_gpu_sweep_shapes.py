@@ -115,3 +115,32 @@ def test_heavy_slices_rank_alike_among_many_bonds(P, extra):
     g.close()
     for o in outs:
         assert np.array_equal(o, ref)
+
+
+def test_bins_larger_than_shared_memory_are_left_out(P):
+    """A group whose iterates do not fit a block's shared memory sweeps as launches."""
+    outs = []
+    for mode in (2, 1):
+        g = P.Scene(_pile(3000), sweep_mode=mode, sweep_lanes=1)
+        g.step(2)
+        outs.append(g.state())
+        g.close()
+    assert np.isfinite(outs[0]).all() and np.array_equal(outs[0], outs[1])
+
+
+def test_step_recaptured_after_a_smaller_scene(P):
+    """A scene's step is captured again (for profiling) after a smaller scene with the same sweep
+    kernel was set up: its shared memory is still granted."""
+    outs = []
+    for other in (False, True):
+        g = P.Scene(_pile(1024), sweep_mode=2, sweep_lanes=4)
+        g.step(1)
+        if other:
+            h = P.Scene(_groups([5, 9]), sweep_mode=2, sweep_lanes=4)
+            h.step(1)
+            h.close()
+            g.set_profiling(True)
+        g.step(2)
+        outs.append(g.state())
+        g.close()
+    assert np.isfinite(outs[0]).all() and np.array_equal(outs[0], outs[1])
