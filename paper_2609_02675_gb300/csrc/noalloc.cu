@@ -25,10 +25,8 @@ constexpr size_t OFF_PCNT = OFF_BOFF + al(sizeof(int) * (NA_TABLE + 1));
 constexpr size_t OFF_POFF = OFF_PCNT + al(sizeof(int) * NA_MAX);
 constexpr size_t OFF_LARGE = OFF_POFF + al(sizeof(int) * (NA_MAX + 1));
 constexpr size_t OFF_CTR = OFF_LARGE + al(sizeof(int) * NA_MAX);
-constexpr size_t OFF_RLO = OFF_CTR + al(sizeof(int) * C_COUNT);
-constexpr size_t OFF_RHI = OFF_RLO + al(sizeof(float4) * NA_MAX);
-constexpr size_t OFF_RCELL = OFF_RHI + al(sizeof(float4) * NA_MAX);
-constexpr size_t OFF_LIST = OFF_RCELL + al(sizeof(int4) * NA_MAX);
+constexpr size_t OFF_REC = OFF_CTR + al(sizeof(int) * C_COUNT);
+constexpr size_t OFF_LIST = OFF_REC + al(2 * sizeof(float4) * NA_MAX);
 constexpr size_t OFF_SCAN = OFF_LIST + al(sizeof(int) * PAIR_LIST * NA_MAX);
 constexpr size_t SCAN_INTS = NA_TABLE / 4096 + 2;  // block totals of the largest scan
 constexpr size_t NA_BYTES = OFF_SCAN + al(sizeof(int) * SCAN_INTS);
@@ -74,7 +72,7 @@ bool current_context_id(unsigned long long* id) {
 
 }  // namespace
 
-// the scratch (about 3.4 MB); device code could name it directly, host code needs its address
+// the scratch (about 3.1 MB); device code could name it directly, host code needs its address
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 
 extern "C" pabd_status pabd_broadphase_noalloc(const float* q, const float* vel, const float* he,
@@ -128,9 +126,7 @@ extern "C" pabd_status pabd_broadphase_noalloc(const float* q, const float* vel,
     d.pair_off = (int*)(base + OFF_POFF);
     d.ctr = (int*)(base + OFF_CTR);
     d.large_ids = (int*)(base + OFF_LARGE);
-    d.brec_lo = (float4*)(base + OFF_RLO);
-    d.brec_hi = (float4*)(base + OFF_RHI);
-    d.brec_cell = (int4*)(base + OFF_RCELL);
+    d.brec = (float4*)(base + OFF_REC);
     d.pair_list = (int*)(base + OFF_LIST);
     d.scan_scratch = (int*)(base + OFF_SCAN);
     d.pairs = (int2*)pairs_out;

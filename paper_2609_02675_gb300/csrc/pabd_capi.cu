@@ -813,7 +813,7 @@ pabd_status finalize_scene(pabd_scene* s) {
     ok &= alloc_arr(s, d.lo, N) && alloc_arr(s, d.hi, N) && alloc_arr(s, d.cell, N);
     ok &= alloc_arr(s, d.bucket_cnt, T) && alloc_arr(s, d.bucket_cur, T) && alloc_arr(s, d.bucket_off, T + 1);
     ok &= alloc_arr(s, d.pair_cnt, N) && alloc_arr(s, d.pair_off, N + 1) && alloc_arr(s, d.pairs, d.cap_pairs);
-    ok &= alloc_arr(s, d.brec_lo, N) && alloc_arr(s, d.brec_hi, N) && alloc_arr(s, d.brec_cell, N);
+    ok &= alloc_arr(s, d.brec, 2 * (size_t)N);
     if (ds.body_contacts && p.broadphase == 0) {
         if (d.multilevel)
             ok &= alloc_arr(s, d.lane_cnt, (size_t)32 * N) && alloc_arr(s, d.pair_stash, (size_t)32 * PAIR_STASH * N) &&

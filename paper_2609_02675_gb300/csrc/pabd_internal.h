@@ -141,8 +141,7 @@ struct Dev {
     float4 *lo, *hi;            // inflated AABB; lo.w = inflation
     int4 *cell;                 // cell coords (.w = bucket)
     int *bucket_cnt, *bucket_cur, *bucket_off;
-    float4 *brec_lo, *brec_hi;  // per bucket slot: (lo, body id bits), (hi, group bits)
-    int4 *brec_cell;            // per bucket slot: (cell x, y, z, flags)
+    float4 *brec;               // per bucket slot: (lo, id, level and pinned bits), (hi, group bits)
     int *pair_list;             // per body: its partners in order, if at most PAIR_LIST (k_pair_count)
     int *lane_cnt;              // multilevel grid, per body x 32 lanes: partners found by each lane
     // multilevel grid, per body x 32 lanes: the first PAIR_STASH partners each lane found while counting (a

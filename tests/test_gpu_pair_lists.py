@@ -72,3 +72,26 @@ def test_pair_lists_equal_brute_force(P, sizes, spread, fast):
         else:
             key = got[:cap, 0].astype(np.int64) * n + got[:cap, 1]
             assert (np.diff(key) > 0).all() and np.isin(key, want[:, 0].astype(np.int64) * n + want[:, 1]).all()
+
+
+@pytest.mark.parametrize("crowd,spread", [(3, 0.3), (30, 0.6), (60, 1.5)])
+def test_pairs_across_levels(P, crowd, spread):
+    """Boxes of the grid's three levels and wider, a few or many to a cell (more to a lane than the
+    count keeps), some pinned: the oracle's pairs, from the grid and from the LBVH."""
+    import oracle as O
+    sc = _clusters([crowd] * 10, spread)
+    b = sc.bodies
+    rng = np.random.default_rng(crowd)
+    for k, he in enumerate([2.5] * 12 + [9.0] * 5 + [60.0] * 2):
+        b["he"][k] = he
+        b["c"][k] = (rng.uniform(0, 90), 5.0 + rng.uniform(-he, he), rng.uniform(-he, he))
+    b["pinned"][rng.integers(0, sc.n_bodies, 40)] = 1
+    ref = O.OracleScene(sc)
+    ref.detect()
+    want = ref.pairs()
+    assert len(want) > 10 * crowd
+    for bp in (0, 1):
+        g = P.Scene(sc, broadphase=bp, max_pairs=400 * sc.n_bodies, max_contacts=4000 * sc.n_bodies)
+        g.detect()
+        assert np.array_equal(g.pairs(), want), bp
+        g.close()
