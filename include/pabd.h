@@ -333,7 +333,7 @@ pabd_status pabd_destroy_scene(pabd_scene* s);
  * another runtime or memory pool, and plug-ins embedded in a host program that holds the
  * GPU's memory budget.  This call allocates nothing: its scratch (hash buckets, per-body
  * counts and offsets, the scan's block sums) is a static device array inside the library,
- * sized for PABD_NOALLOC_MAX_BODIES bodies (about 3.1 MB) and held by every GPU that loads
+ * sized for PABD_NOALLOC_MAX_BODIES bodies (about 3 MB) and held by every GPU that loads
  * the library until the process exits.  The paper has no counterpart of this entry point; it
  * returns the same sorted pair list as pabd_detect / pabd_read_pairs for a scene with these
  * bodies and no user bonds.

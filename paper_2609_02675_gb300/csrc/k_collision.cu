@@ -9,9 +9,9 @@
 // grid and is tested against all bodies instead of widening every cell.  Scenes with such
 // bodies by design use a multilevel grid instead (below), where a fast body moves up a level
 // rather than off the grid.  Bodies are counting-sorted into hash buckets; each body scans
-// the 27 cells around its own and keeps the neighbours j > i whose boxes overlap, whose cell
-// really is the visited one (so hash collisions never duplicate a pair), that share its group
-// and are not joined to it by a user bond.  Each body's partner list is sorted, so the final
+// the 27 cells around its own, each bucket once (cells that share one never duplicate a pair),
+// and keeps the neighbours j > i whose boxes overlap, that share its group and are not joined to
+// it by a user bond.  Each body's partner list is sorted, so the final
 // list is the sorted set of overlapping pairs -- independent of bucket order.
 //
 // Narrow phase: box-box contact manifold (reference face by separating axis over the six

@@ -72,7 +72,7 @@ bool current_context_id(unsigned long long* id) {
 
 }  // namespace
 
-// the scratch (about 3.1 MB); device code could name it directly, host code needs its address
+// the scratch (about 3 MB); device code could name it directly, host code needs its address
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 
 extern "C" pabd_status pabd_broadphase_noalloc(const float* q, const float* vel, const float* he,

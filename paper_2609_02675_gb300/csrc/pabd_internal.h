@@ -123,7 +123,7 @@ struct Dev {
     int *heavy;                 // ids of the bodies with more than HEAVY_ENDS ends (C_NHEAVY of them)
     // scenes whose only contacts are with the ground: each body's live static bond ends, sorted
     // by end id (2 bond + side), fixed at creation -- the CSR is these plus the step's ground
-    // contacts (k_csr_ground); null otherwise
+    // contacts (k_ground_bonds_csr); null otherwise
     int *sta_off, *sta_id;
     int *sta_body;              // the body of each entry of sta_id
     // ground contacts of the bodies before b in the fused front of a ground-only scene: the
@@ -147,7 +147,7 @@ struct Dev {
     // multilevel grid, per body x 32 lanes: the first PAIR_STASH partners each lane found while counting (a
     // partner delivered to a smaller id tagged by STASH_DELIVER), and the lane's number of
     // entries, so that writing the pairs replays them instead of scanning the cells again (a
-    // lane with more rescans); null where the pair kernels run without them
+    // warp with a lane that found more rescans); null where the pair kernels run without them
     int *pair_stash, *lane_tot;
     int *pair_cnt, *pair_off;
     int2 *pairs;
