@@ -259,7 +259,9 @@ pabd_status pabd_set_group_hold(pabd_scene* s, const uint8_t* hold, size_t n_gro
  * fused persistent sweep, sweep_mode 3): a wait gives up after `polls` polls (default 2^24,
  * about a second), latches PABD_ERR_TIMEOUT and ends its kernel, which the next
  * synchronising call returns; the scene's later steps are not trustworthy.  Tests shorten the
- * bound to check that a wait that runs out is reported.  polls == 0 is PABD_ERR_ARG. */
+ * bound to check that a wait that runs out is reported.  Collision detection, too, waits at most
+ * so many polls for a count, and then makes that count itself: the same results, later, and no
+ * error.  polls == 0 is PABD_ERR_ARG. */
 pabd_status pabd_set_wait_limit(pabd_scene* s, uint32_t polls);
 
 /* Stage timing.  With profiling on, pabd_step launches a second captured graph that also

@@ -354,9 +354,9 @@ __device__ __forceinline__ Contact write_contact(const Dev& d, int slot, int typ
     return c;
 }
 
-// One item of the small front's two narrow passes.  Items [0, np) are this step's pairs, items np + b
-// the ground corners of body b (apart, so that no item runs both manifolds in series).
-__device__ __forceinline__ void narrow_count_item(const Dev& d, int tt, int np) {
+// Contacts of one narrow-phase item, counted alone.  Items [0, np) are this step's pairs, items
+// np + b the ground corners of body b (apart, so that no item runs both manifolds in series).
+__device__ __forceinline__ int narrow_item_contacts(const Dev& d, int tt, int np) {
     if (tt < np) {
         int2 pr = d.pairs[tt];
         FBox fa, fb;
@@ -365,17 +365,20 @@ __device__ __forceinline__ void narrow_count_item(const Dev& d, int tt, int np) 
         LocalPoly poly;
         Manifold mf;
         int out;
-        d.npc[tt] = box_box(fa, fb, pr.x, pr.y, poly, mf, out, [](const Corner&, int) {});
-    } else {
-        const int t = tt - np;
-        int n = 0;
-        if (d.p.has_ground && !(d.bflags[t] & BF_PINNED)) {
-            FBox fa;
-            load_box(d, t, fa);
-            n = ground_corners(d, fa, t, [](int, int, const float*, const float*, int) {});
-        }
-        d.gnd_cnt[t] = n;
+        return box_box(fa, fb, pr.x, pr.y, poly, mf, out, [](const Corner&, int) {});
     }
+    const int t = tt - np;
+    if (!d.p.has_ground || (d.bflags[t] & BF_PINNED)) return 0;
+    FBox fa;
+    load_box(d, t, fa);
+    return ground_corners(d, fa, t, [](int, int, const float*, const float*, int) {});
+}
+
+// an item of the first of the small front's two narrow passes
+__device__ __forceinline__ void narrow_count_item(const Dev& d, int tt, int np) {
+    const int n = narrow_item_contacts(d, tt, np);
+    if (tt < np) d.npc[tt] = n;
+    else d.gnd_cnt[tt - np] = n;
 }
 
 // writes the item's contacts from npc_off and, after the npc pair contacts, gnd_off on;

@@ -37,16 +37,11 @@ __device__ __forceinline__ void place_end(const Dev& d, int id, int p) {
     }
 }
 
-// (a slot past the arrays cannot be, unless a bounded wait of the narrow phase gave up)
 __device__ __forceinline__ void csr_fill_bond(const Dev& d, int b) {
     const int4 m = d.bmeta[b];
     auto put = [&](int body, int id) {
-        if (end_live(d, body)) {
-            const int p = d.end_off[body] + atomicAdd(&d.end_cur[body], 1);
-            if (p < d.cap_ends) d.end_id[p] = id;
-        } else {
-            d.end_pos[id] = -1;
-        }
+        if (end_live(d, body)) d.end_id[d.end_off[body] + atomicAdd(&d.end_cur[body], 1)] = id;
+        else d.end_pos[id] = -1;
     };
     put(m.x, 2 * b);
     put(m.y, 2 * b + 1);

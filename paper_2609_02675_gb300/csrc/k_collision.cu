@@ -460,6 +460,16 @@ __global__ void __launch_bounds__(OFF_T) k_offgrid_pairs(Dev d) {
 
 // ---- narrow phase ----
 
+// contacts of a tile of k_narrow's items, counted again by a warp (out of line: hardly ever wanted)
+__device__ __noinline__ int tile_contacts(const Dev& d, int tile, int np) {
+    int n = 0;
+    for (int t = threadIdx.x & 31; t < NARROW_T; t += 32) {
+        const int item = tile * NARROW_T + t;
+        if (item < np + d.N) n += narrow_item_contacts(d, item, np);
+    }
+    return __reduce_add_sync(0xffffffffu, n);
+}
+
 // The whole narrow phase in one pass.  Items [0, np) are this step's pairs, items np + b the ground
 // corners of body b; a tile of NARROW_T items is a block's, a thread each.  The block keeps its
 // items' contacts in shared memory while it learns how many contacts precede its tile -- the
@@ -467,15 +477,16 @@ __global__ void __launch_bounds__(OFF_T) k_offgrid_pairs(Dev d) {
 // nearest one whose whole prefix is known (decoupled look-back, Merrill and Garland 2016) -- and
 // then writes them, a thread per contact.  Contacts come out in item order whatever the order of
 // the blocks.  Tiles are taken from a counter, so a tile's predecessors are running or done; the
-// wait for them is bounded all the same (PABD_ERR_TIMEOUT).  The bodies' bond ends are counted on
-// the way, on top of their static ones.
+// wait for them is bounded all the same, and where it runs out the waiting warp counts the missing
+// tile's contacts itself (tile_contacts): a late tile costs time, and every contact keeps its one
+// slot.  The bodies' bond ends are counted on the way, on top of their static ones.
 //
 // It replaced a counting pass, two prefix sums, a pass that derived every manifold again to write
 // it, and the count of bond ends.  Bound by the clipping's dependent steps and their trips to
 // shared memory (16 warps per SM, its 46 KB a block): 532 325 pairs of a settled bed 115 us
 // (counting 156 and writing 187 us; in one pass with the polygons in local memory 274), 258 048
 // pairs of a pile, all touching, 78 us (57 and 90).
-__global__ void __launch_bounds__(NARROW_T) k_narrow(Dev d) {
+__global__ void __launch_bounds__(NARROW_T) k_narrow(const __grid_constant__ Dev d) {
     constexpr int T = NARROW_T, MAXC = 8;
     __shared__ float corners[2 * MAXC * 5 * T];  // the items' polygons, then their contacts (SharedPoly)
     __shared__ float nrm[3][T], wgt[T], dht[T], face_x[T];
@@ -550,19 +561,19 @@ __global__ void __launch_bounds__(NARROW_T) k_narrow(Dev d) {
                 for (int first = tile - 1;; first -= 32) {  // tiles first, first - 1, ...: one per lane
                     const int k = first - lane;
                     unsigned long long v = WHOLE;  // (before tile 0: nothing)
-                    unsigned polls = 0;
-                    if (k >= 0) {
-                        while (((v = state[k]) >> 32) == 0) {
-                            if (++polls > limit) {
-                                latch_status(d, ST_TIMEOUT);
-                                v = WHOLE;
-                                break;
-                            }
-                        }
+                    unsigned whole, late;  // lanes with a whole prefix; unpublished ones before the nearest
+                    int last;              // the nearest lane with a whole prefix
+                    for (unsigned polls = 0;; ++polls) {
+                        if (k >= 0) v = state[k];
+                        whole = __ballot_sync(0xffffffffu, (v >> 32) == 2);
+                        last = whole ? __ffs(whole) - 1 : 31;
+                        late = __ballot_sync(0xffffffffu, v == 0 && lane <= last);
+                        if (late == 0 || polls >= limit) break;
                     }
-                    __syncwarp();
-                    const unsigned whole = __ballot_sync(0xffffffffu, (v >> 32) == 2);
-                    const int last = whole ? __ffs(whole) - 1 : 31;  // nearest with a whole prefix
+                    for (; late; late &= late - 1) {
+                        const int l = __ffs(late) - 1, n = tile_contacts(d, first - l, np);
+                        if (lane == l) v = PART | (unsigned)n;
+                    }
                     int c = lane <= last ? (int)(unsigned)v : 0;
                     c = __reduce_add_sync(0xffffffffu, c);
                     before += c;

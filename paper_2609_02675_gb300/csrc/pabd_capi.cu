@@ -175,7 +175,7 @@ struct pabd_scene {
     std::vector<float2> al_init;
     // stream on which the body of the residual-threshold loop is captured into its graph node
     cudaStream_t body_st = nullptr;
-    // polls before a device-side wait gives up (PABD_ERR_TIMEOUT); about a second by default
+    // polls before a device-side wait gives up; about a second by default
     unsigned wait_polls = 1u << 24;
     // pinned staging of the group hold masks: HOLD_SLOTS slots of G bytes used in turn, each
     // reused only after its previous copy to the device has completed
@@ -898,9 +898,6 @@ pabd_status finalize_scene(pabd_scene* s) {
     CK(cudaMemsetAsync(d.resid_group, 0, sizeof(double) * (d.G ? d.G : 1), st));
     CK(cudaMemsetAsync(d.group_hold, 0, d.G ? d.G : 1, st));
     CK(cudaMemsetAsync(d.end_pos, 0xff, sizeof(int) * d.cap_ends, st));
-    // (valid ids and bodies wherever a step cut short by a timed-out wait might read past its own)
-    CK(cudaMemsetAsync(d.end_id, 0, sizeof(int) * d.cap_ends, st));
-    CK(cudaMemsetAsync(d.bmeta + Nc, 0, sizeof(int4) * (size_t)d.cap_contacts, st));
     CK(cudaMemsetAsync(d.gbar, 0, 2 * sizeof(unsigned), st));
     const unsigned wait_polls = s->wait_polls;
     CK(cudaMemcpyAsync(d.wait_limit, &wait_polls, sizeof(unsigned), cudaMemcpyHostToDevice, st));

@@ -135,7 +135,7 @@ struct Dev {
     float4 *rec;                // bond-end records in CSR order, 3 float4 per end (pack_end)
     int csr_want;               // what the CSR is built with (WANT_SLOTS, WANT_RECORDS)
     unsigned *gbar;             // grid barrier: arrival counter, generation
-    unsigned *wait_limit;       // polls before a device-side wait gives up (PABD_ERR_TIMEOUT)
+    unsigned *wait_limit;       // polls before a device-side wait gives up
     int2 *bin_range;            // body range of each bin of k_sweep_bins, or null
     // collision
     float4 *lo, *hi;            // inflated AABB; lo.w = inflation
