@@ -1,6 +1,7 @@
 // All n_iter sweeps of a step in one launch, for scenes whose groups are small (sweep mode 2).
 //
-// Bodies interact only inside their group, so whole groups are dealt to bins of consecutive
+// Bodies interact only inside their group (a scene whose user bonds join groups is swept by
+// launches), so whole groups are dealt to bins of consecutive
 // bodies and each bin is swept by one thread-block cluster on its own: nothing is exchanged
 // between clusters.  The bin's iterates live in shared memory, twice (Jacobi), a copy in every
 // block of the cluster: a body's new iterate is stored into all the copies through distributed

@@ -227,7 +227,8 @@ int sweep_threads(int lanes, int N, int ext_bodies, int policy) {
 // 121-body net 3.7 against 4.9 us, 8 chained bodies 3.0 against 5.4, a 250-box pile 3.8 against
 // 4.5; larger groups would take turns on the cluster's 16 SMs while a launch spreads them over
 // all.  The same happens to more clusters than the device holds at once (setup_sweep_bins):
-// 30 piles of 1500 boxes take 6.3 us against 4.8.
+// 30 piles of 1500 boxes take 6.3 us against 4.8.  Nor where a user bond joins two groups: a bin's
+// iterates are its own groups' alone.
 std::vector<int2> choose_bins(const std::vector<int>& group_off, int G, int N, int lanes, BinsShape* out) {
     int gmax = 0;
     for (int g = 0; g < G; ++g) gmax = std::max(gmax, group_off[g + 1] - group_off[g]);
@@ -922,7 +923,10 @@ pabd_status finalize_scene(pabd_scene* s) {
     if (L != 1 && L != 2 && L != 4 && L != 8 && L != 16) return PABD_ERR_ARG;
     s->lanes = L;
     s->threads = sweep_threads(L, N, s->fp64_bodies, p.precision_policy);
-    if (p.resid_tol <= 0) {
+    bool groups_apart = true;
+    for (const HostBond& hb : s->bonds) groups_apart &= hb.i < 0 || hb.j < 0 || group[hb.i] == group[hb.j];
+    s->bins = BinsShape{};
+    if (p.resid_tol <= 0 && groups_apart) {
         const std::vector<int2> bins = choose_bins(group_off, d.G, N, L, &s->bins);
         if (s->bins.n) {
             int fit = 0;
