@@ -169,13 +169,14 @@ __device__ __forceinline__ int warp_excl(int v, int lane) {
 
 // Counts body i's partners (a warp per body) and, when there are at most PAIR_LIST of them and no
 // lane found more than four, leaves them in order in its list, so that writing the pairs is a
-// copy.
+// copy; a body with partners and no list is noted for the writing pass (Dev::pair_rest).
 __global__ void __launch_bounds__(CT) k_pair_count(Dev d) {
     pdl_enter();
     __shared__ int found[CT / 32][PAIR_LIST];
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (i >= d.N) return;
     int n = 0;
+    bool listed = false;
     const int gi = d.group[i], fi = d.bflags[i];
     if (d.cell[i].w < 0) {
         const float4 li = d.lo[i], hi_ = d.hi[i];
@@ -192,7 +193,8 @@ __global__ void __launch_bounds__(CT) k_pair_count(Dev d) {
                 if (k == c) id[c] = j;
         });
         n = warp_sum(mine);
-        if (n > 0 && n <= PAIR_LIST && !__any_sync(0xffffffffu, mine > 4)) {
+        listed = n > 0 && n <= PAIR_LIST && !__any_sync(0xffffffffu, mine > 4);
+        if (listed) {
             const int at = warp_excl(mine, lane);
 #pragma unroll
             for (int c = 0; c < 4; ++c)
@@ -201,16 +203,21 @@ __global__ void __launch_bounds__(CT) k_pair_count(Dev d) {
             const int v = lane < n ? found[w][lane] : 0x7fffffff;
             const int r = warp_rank32(v, n, lane);
             if (r >= 0) d.pair_list[(size_t)i * PAIR_LIST + r] = v;
-        } else if (n > 0 && lane == 0) {
-            d.pair_list[(size_t)i * PAIR_LIST] = -1;  // not listed: found again when written
         }
     }
-    if (lane == 0) d.pair_cnt[i] = n;
+    if (lane == 0) {
+        d.pair_cnt[i] = n;
+        if (n > 0 && !listed) {  // found again when written
+            d.pair_list[(size_t)i * PAIR_LIST] = -1;
+            d.pair_rest[atomicAdd(&d.ctr[C_NREST], 1)] = i;
+        }
+    }
 }
 
-// The pairs of the bodies that were not listed while counting, by a warp: off-grid bodies (the
-// whole rest in order), and bodies with many partners (found again, then sorted).
-__device__ __forceinline__ void write_unlisted_pairs(const Dev& d, int i, int lane) {
+// The pairs of a body that was not listed while counting, by a warp: an off-grid body's (the
+// whole rest in order), or those of a body with many partners (found again, in any order, then
+// sorted; a slice that the capacity cuts keeps any of them).  cur: a word of shared memory.
+__device__ __forceinline__ void write_unlisted_pairs(const Dev& d, int i, int lane, int* cur) {
     const int s = d.pair_off[i], cap = d.cap_pairs;
     const int gi = d.group[i], fi = d.bflags[i];
     if (d.cell[i].w < 0) {
@@ -226,10 +233,11 @@ __device__ __forceinline__ void write_unlisted_pairs(const Dev& d, int i, int la
         }
         return;
     }
-    const int mine = lane_partners(d, i, lane, [](int, int) {});
-    const int base = s + warp_excl(mine, lane);
-    lane_partners(d, i, lane, [&](int j, int k) {
-        if (base + k < cap) d.pairs[base + k] = make_int2(i, j);
+    if (lane == 0) *cur = s;
+    __syncwarp();
+    lane_partners(d, i, lane, [&](int j, int) {
+        const int at = atomicAdd(cur, 1);
+        if (at < cap) d.pairs[at] = make_int2(i, j);
     });
     __syncwarp();
     const int e = min(d.pair_off[i + 1], cap), n = e - s;
@@ -255,32 +263,33 @@ __device__ __forceinline__ void write_unlisted_pairs(const Dev& d, int i, int la
     }
 }
 
-// Copies the listed partners, WRITE_LANES lanes per body; then each warp writes its bodies that
-// were not listed, one after the other.  (A warp per body that replayed every lane's finds took
-// 120 us for 262 144 boxes, and without room for them, in the allocation-free call, it scanned the
-// cells twice more: 50 us for 16 384 boxes.  Now 13 and 13.)
+// Copies the listed partners, WRITE_LANES lanes per body; then the warps share out the bodies that
+// were not listed, each its first by its index and the next ones from a counter (an off-grid body's
+// sweep takes the longer the smaller its id).  (A warp per body that replayed every lane's finds
+// took 120 us for 262 144 boxes, and without room for them, in the allocation-free call, it scanned
+// the cells twice more: 50 us for 16 384 boxes.  Now 13 and 13.  Left to the warps that copy around
+// them, eight to a warp, the unlisted ones were the launch's length: detection of 60 000 cubes of
+// which 568 are off the grid 3077 us, now 1850, of 1000 crowded ones, 42 partners each, 1294, now
+// 350.)
 constexpr int WRITE_LANES = 4;
 __global__ void __launch_bounds__(CT) k_pair_write(Dev d) {
     pdl_enter();
+    __shared__ int cur[CT / 32];
     const int t = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     const int i = t / WRITE_LANES, sub = t % WRITE_LANES, cap = d.cap_pairs;
-    bool unlisted = false;
     if (i < d.N) {
         const int s = d.pair_off[i], n = d.pair_off[i + 1] - s;
-        if (n > 0) {
-            const int* list = d.pair_list + (size_t)i * PAIR_LIST;
-            unlisted = d.cell[i].w < 0 || list[0] < 0;
-            if (!unlisted)
-                for (int k = sub; k < n; k += WRITE_LANES)
-                    if (s + k < cap) d.pairs[s + k] = make_int2(i, list[k]);
-        }
+        const int* list = d.pair_list + (size_t)i * PAIR_LIST;
+        if (n > 0 && list[0] >= 0)
+            for (int k = sub; k < n; k += WRITE_LANES)
+                if (s + k < cap) d.pairs[s + k] = make_int2(i, list[k]);
     }
-    unsigned todo = __ballot_sync(0xffffffffu, unlisted && sub == 0);
-    while (todo) {
-        const int l = __ffs(todo) - 1;
-        todo &= todo - 1;
-        write_unlisted_pairs(d, (t - lane + l) / WRITE_LANES, lane);
-        __syncwarp();
+    const int rest = d.ctr[C_NREST], warps = gridDim.x * (CT / 32);
+    for (int r = t >> 5; r < rest;) {
+        write_unlisted_pairs(d, d.pair_rest[r], lane, &cur[threadIdx.x >> 5]);
+        if (rest <= warps) break;
+        if (lane == 0) r = warps + atomicAdd(&d.ctr[C_REST_NEXT], 1);
+        r = __shfl_sync(0xffffffffu, r, 0);
     }
     if (t == 0) {
         const int tot = d.pair_off[d.N];
@@ -735,6 +744,10 @@ void launch_ground_front(const Dev& d, cudaStream_t st, long long* launches) {
     *launches += 2;
 }
 
+// k_pair_write's grid: WRITE_LANES threads per body, and at least a warp per body while all are
+// resident at once
+static inline int pair_write_blocks(int n) { return std::max(nblk(n * WRITE_LANES), stride_grid(32ll * n, CT)); }
+
 // The broad phase alone (bucket / counter resets, AABBs, grid, sorted pair list), on whatever
 // buffers `d` points at; used by the allocation-free entry point.
 void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches) {
@@ -749,7 +762,7 @@ void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches) {
     const int wblk = (d.N * 32 + CT - 1) / CT > 0 ? (d.N * 32 + CT - 1) / CT : 1;
     launch_pdl(k_pair_count, dim3(wblk), dim3(CT), 0, st, d);
     scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
-    launch_pdl(k_pair_write, dim3(nblk(d.N * WRITE_LANES)), dim3(CT), 0, st, d);
+    launch_pdl(k_pair_write, dim3(pair_write_blocks(d.N)), dim3(CT), 0, st, d);
     *launches += 5;
 }
 
@@ -780,7 +793,7 @@ void launch_collision(const Dev& d, cudaStream_t st, long long* launches) {
         } else {
             launch_pdl(k_pair_count, dim3(wblk), dim3(CT), 0, st, d);
             scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
-            launch_pdl(k_pair_write, dim3(nblk(d.N * WRITE_LANES)), dim3(CT), 0, st, d);
+            launch_pdl(k_pair_write, dim3(pair_write_blocks(d.N)), dim3(CT), 0, st, d);
             *launches += 4;
         }
     }

@@ -820,7 +820,7 @@ pabd_status finalize_scene(pabd_scene* s) {
             ok &= alloc_arr(s, d.lane_cnt, (size_t)32 * N) && alloc_arr(s, d.pair_stash, (size_t)32 * PAIR_STASH * N) &&
                   alloc_arr(s, d.lane_tot, (size_t)32 * N);
         else
-            ok &= alloc_arr(s, d.pair_list, (size_t)PAIR_LIST * N);
+            ok &= alloc_arr(s, d.pair_list, (size_t)PAIR_LIST * N) && alloc_arr(s, d.pair_rest, N);
     }
     if (front_fits(N, ds.body_contacts)) ok &= alloc_arr(s, d.npc, d.cap_pairs) && alloc_arr(s, d.npc_off, d.cap_pairs + 1);
     if (ds.body_contacts) ok &= alloc_arr(s, d.tile_state, ((size_t)d.cap_pairs + N) / NARROW_T + 1);

@@ -41,6 +41,8 @@ enum Counter {
     C_SWEEP_NEXT,      // the same for the one-launch sweeps, one counter per sweep parity: sweep k
     C_SWEEP_NEXT1,     // takes counter k & 1 and zeroes the other one for sweep k + 1
     C_NARROW_NEXT,     // next tile of the narrow phase
+    C_NREST,           // bodies whose partners the single-level grid's count did not list (Dev::pair_rest)
+    C_REST_NEXT,       // and the next of them past the first one of each warp that writes them
     C_COUNT
 };
 
@@ -143,6 +145,7 @@ struct Dev {
     int *bucket_cnt, *bucket_cur, *bucket_off;
     float4 *brec;               // per bucket slot: (lo, id, level and pinned bits), (hi, group bits)
     int *pair_list;             // per body: its partners in order, if at most PAIR_LIST (k_pair_count)
+    int *pair_rest;             // the bodies that have partners and no such list
     int *lane_cnt;              // multilevel grid, per body x 32 lanes: partners found by each lane
     // multilevel grid, per body x 32 lanes: the first PAIR_STASH partners each lane found while counting (a
     // partner delivered to a smaller id tagged by STASH_DELIVER), and the lane's number of
