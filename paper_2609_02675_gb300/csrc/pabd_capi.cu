@@ -372,6 +372,11 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
     mark();
 }
 
+// Where a tuner's trial sweeps leave the bodies' squared updates: the scene's own (Dev::resid_body)
+// are part of its state, a held group's residual being that of its last step.  (Dev::qstar is
+// written anew by every step's predictor, and no sweep reads it.)
+double* trial_resid(const Dev& d) { return reinterpret_cast<double*>(d.qstar); }
+
 // Launch-shape autotuner for the fused sweep: with the scene's step-0 collision, CSR and
 // predictor in place (none of them changes q^n), time the sweep for each candidate grid of
 // HEAVY_T-thread blocks; keep the fastest.  The shape never changes the results (each body's
@@ -379,6 +384,7 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
 pabd_status autotune_sweep(pabd_scene* s) {
     Dev d = s->d;
     d.csr_want = WANT_RECORDS;
+    d.resid_body = trial_resid(d);
     long long lc = 0;
     launch_step_reset(d, s->st, &lc);
     launch_collision(d, s->st, &lc);
@@ -446,6 +452,7 @@ pabd_status autotune_default(pabd_scene* s) {
     long long lc = 0;
     Dev dd = d;
     dd.csr_want = WANT_SLOTS | WANT_RECORDS;
+    dd.resid_body = trial_resid(d);
     launch_step_reset(dd, s->st, &lc);
     if (dd.sta_off) {
         launch_ground_front(dd, s->st, &lc);
