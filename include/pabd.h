@@ -197,7 +197,7 @@ typedef struct {
     int64_t tuned;            /* 1 if sweep_mode and light_order were chosen by timing (sweep_mode
                                  0 in the descriptor, no resid_tol, no AL_DISTANCE bonds) */
     int64_t tune_sweep_ns[4]; /* the autotuner's time per sweep for each candidate (the fastest of
-                                 up to four timed passes over n_iter sweeps and of its
+                                 up to three timed passes over n_iter sweeps and of its
                                  thread counts per body), nanoseconds: one launch per sweep
                                  ordered (or one for all sweeps over clusters) / in body order, a bond and a solve
                                  launch per sweep ordered / in body order (0: not tuned) */

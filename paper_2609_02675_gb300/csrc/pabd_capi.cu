@@ -488,7 +488,7 @@ pabd_status autotune_default(pabd_scene* s) {
                 float4* cur = dd.qa;
                 float4* nxt = dd.qb;
                 if (in_bins) launch_sweep_bins(dd, s->bins, s->lanes, s->st, &lc);
-                else for (int it = 0; it < n_it; ++it) {
+                else for (int it = 0; it < (r == 0 ? 1 : n_it); ++it) {
                     if (mode == 2) {
                         launch_sweep_one(dd, cur, nxt, it, s->lanes, threads, s->st, &lc, true);
                     } else {
@@ -501,9 +501,10 @@ pabd_status autotune_default(pabd_scene* s) {
                 CK(cudaEventSynchronize(e1));
                 float t = 0.f;
                 CK(cudaEventElapsedTime(&t, e0, e1));
-                if (r > 0) tot = std::min(tot, t);  // the first pass warms the caches; the fastest
-                                                    // of the others (least disturbed) is the figure
-                if (r > 0 && (tot > 1.05f * best || tot > 1.f)) break;  // out of the running; long enough to trust
+                if (r > 0) tot = std::min(tot, t);  // the first pass, of one sweep, loads the kernels and warms
+                                                    // the caches; the fastest of the others is the figure
+                // (out of the running; or long enough to trust, alone or as one of two)
+                if (r > 0 && (tot > 1.05f * best || tot > 1.f || (r > 1 && tot > 0.15f))) break;
             }
             CK(cudaGetLastError());
             fastest = std::min(fastest, tot);
