@@ -42,8 +42,8 @@ __device__ __forceinline__ int cell_coord(float x, float inv_cs) {
     return (int)t;
 }
 
-__device__ __forceinline__ int cell_hash(int x, int y, int z, int bits) {
-    unsigned h = (unsigned)x * 73856093u ^ (unsigned)y * 19349663u ^ (unsigned)z * 83492791u;
+__device__ __forceinline__ int cell_hash(unsigned x, unsigned y, unsigned z, int bits) {
+    unsigned h = x * 73856093u ^ y * 19349663u ^ z * 83492791u;
     h ^= h >> 16;
     h *= 0x7feb352du;
     h ^= h >> 15;
@@ -64,7 +64,7 @@ __device__ __forceinline__ float level_cell(const Dev& d, int lv) {
 // within +-2^20; groups apart, so that scenes in the same place do not fill each other's buckets:
 // 24 piles of 8000 boxes counted their pairs in 27 us, now 11)
 __device__ __forceinline__ int level_hash(int x, int y, int z, int lv, int group, int bits) {
-    return cell_hash(x + (lv << 22) + group * 0x2545f491, y, z, bits);
+    return cell_hash((unsigned)x + ((unsigned)lv << 22) + (unsigned)group * 0x2545f491u, (unsigned)y, (unsigned)z, bits);
 }
 
 __global__ void k_cells(Dev d) {
