@@ -414,7 +414,6 @@ __global__ void k_ml_pair_write(Dev d) {
 // WRITE = false counts (into pair_cnt[i], and each warp's count in lane_cnt[32 i + w]); true
 // stores the partners into pair_j.
 constexpr int OFF_T = 128;
-constexpr int OFF_BLOCKS = 152 * 4;
 
 template <bool WRITE>
 __global__ void __launch_bounds__(OFF_T) k_offgrid_pairs(Dev d) {
@@ -784,10 +783,10 @@ void launch_collision(const Dev& d, cudaStream_t st, long long* launches) {
         const int wblk = (d.N * 32 + CT - 1) / CT > 0 ? (d.N * 32 + CT - 1) / CT : 1;  // one warp per body
         if (d.multilevel) {
             launch_pdl(k_ml_pair_count, dim3(wblk), dim3(CT), 0, st, d);
-            launch_pdl(k_offgrid_pairs<false>, dim3(OFF_BLOCKS), dim3(OFF_T), 0, st, d);
+            launch_pdl(k_offgrid_pairs<false>, dim3(resident_slots(4)), dim3(OFF_T), 0, st, d);
             scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
             launch_pdl(k_ml_pair_write, dim3(wblk), dim3(CT), 0, st, d);
-            launch_pdl(k_offgrid_pairs<true>, dim3(OFF_BLOCKS), dim3(OFF_T), 0, st, d);
+            launch_pdl(k_offgrid_pairs<true>, dim3(resident_slots(4)), dim3(OFF_T), 0, st, d);
             *launches += 6;
             launch_pair_sort(d, st, launches);
         } else {

@@ -211,14 +211,14 @@ bool alloc_arr(pabd_scene* s, T*& p, size_t n) {
 }
 
 // Threads per body of the sweep launches where the autotuner does not time both: as many as
-// lanes while they all fit on the device at once (152 SMs x 4 blocks x 128 threads), else half
+// lanes while they all fit on the device at once (4 blocks of 128 threads per SM), else half
 // as many -- every thread repeats its body's solve, and a pile of 8000 boxes (16 lanes) sweeps in
 // 7.0 us on 8 threads per body against 9.8 us on 16, one of 30 000 (4 lanes) in 8.9 us against
 // 11.6, but one of 4800 in 6.1 against 5.8.  Not where most bodies take the extended path, whose
 // second sum then follows the first (256 trees: 15.0 against 12.6 us).
 int sweep_threads(int lanes, int N, int ext_bodies, int policy) {
     if (policy == 2 || lanes == 1) return lanes;
-    return (long long)lanes * N > 152 * 4 * 128 && 2LL * ext_bodies < N ? lanes / 2 : lanes;
+    return (long long)lanes * N > resident_slots(4) * 128 && 2LL * ext_bodies < N ? lanes / 2 : lanes;
 }
 
 // The bins of k_sweep_bins (consecutive whole groups), or none where the sweeps run as launches.
@@ -468,7 +468,7 @@ pabd_status autotune_default(pabd_scene* s) {
     CK(cudaEventCreate(&e1));
     const int n_it = d.p.n_iter;
     // (half the threads never won while the lanes' threads fill less than the device)
-    const bool many = (long long)s->lanes * d.N > 152 * 4 * 96;
+    const bool many = (long long)s->lanes * d.N > resident_slots(4) * 96;
     const int half = many && s->lanes > 1 && d.p.precision_policy != 2 ? s->lanes / 2 : 0;
     float best = 1e30f;
     for (int c = 0; c < 4; ++c) {
