@@ -736,7 +736,7 @@ __global__ void k_ground_bonds_csr(Dev d) {
 
 void launch_ground_front(const Dev& d, cudaStream_t st, long long* launches) {
     launch_pdl(k_ground_prelude, dim3(nblk(d.N)), dim3(CT), 0, st, d);
-    scan_exclusive(d.gnd_blk, d.gnd_bof, nullptr, nblk(d.N), d.scan_scratch, st, launches);
+    scan_exclusive(d.gnd_blk, d.gnd_bof, nblk(d.N), d.scan_scratch, st, launches);
     with_want(d.csr_want, [&](auto w) {
         launch_pdl(k_ground_bonds_csr<decltype(w)::value>, dim3(stride_grid((long long)d.cap_ends + d.N + 1, CT)), dim3(CT), 0, st, d);
     });
@@ -756,11 +756,11 @@ void launch_broadphase(const Dev& d, cudaStream_t st, long long* launches) {
     cudaMemsetAsync(d.ctr, 0, sizeof(int) * C_COUNT, st);
     launch_pdl(k_aabb, dim3(nblk(d.N)), dim3(CT), 0, st, d);
     launch_pdl(k_cells, dim3(nblk(d.N)), dim3(CT), 0, st, d);
-    scan_exclusive(d.bucket_cnt, d.bucket_off, nullptr, T, d.scan_scratch, st, launches);
+    scan_exclusive(d.bucket_cnt, d.bucket_off, T, d.scan_scratch, st, launches);
     launch_pdl(k_bucket_fill, dim3(nblk(d.N)), dim3(CT), 0, st, d);
     const int wblk = (d.N * 32 + CT - 1) / CT > 0 ? (d.N * 32 + CT - 1) / CT : 1;
     launch_pdl(k_pair_count, dim3(wblk), dim3(CT), 0, st, d);
-    scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
+    scan_exclusive(d.pair_cnt, d.pair_off, d.N, d.scan_scratch, st, launches);
     launch_pdl(k_pair_write, dim3(pair_write_blocks(d.N)), dim3(CT), 0, st, d);
     *launches += 5;
 }
@@ -778,20 +778,20 @@ void launch_collision(const Dev& d, cudaStream_t st, long long* launches) {
     } else {
         const int T = 1 << d.table_bits;
         launch_pdl(k_cells, dim3(nblk(d.N)), dim3(CT), 0, st, d);
-        scan_exclusive(d.bucket_cnt, d.bucket_off, nullptr, T, d.scan_scratch, st, launches);
+        scan_exclusive(d.bucket_cnt, d.bucket_off, T, d.scan_scratch, st, launches);
         launch_pdl(k_bucket_fill, dim3(nblk(d.N)), dim3(CT), 0, st, d);
         const int wblk = (d.N * 32 + CT - 1) / CT > 0 ? (d.N * 32 + CT - 1) / CT : 1;  // one warp per body
         if (d.multilevel) {
             launch_pdl(k_ml_pair_count, dim3(wblk), dim3(CT), 0, st, d);
             launch_pdl(k_offgrid_pairs<false>, dim3(resident_slots(4)), dim3(OFF_T), 0, st, d);
-            scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
+            scan_exclusive(d.pair_cnt, d.pair_off, d.N, d.scan_scratch, st, launches);
             launch_pdl(k_ml_pair_write, dim3(wblk), dim3(CT), 0, st, d);
             launch_pdl(k_offgrid_pairs<true>, dim3(resident_slots(4)), dim3(OFF_T), 0, st, d);
             *launches += 6;
             launch_pair_sort(d, st, launches);
         } else {
             launch_pdl(k_pair_count, dim3(wblk), dim3(CT), 0, st, d);
-            scan_exclusive(d.pair_cnt, d.pair_off, nullptr, d.N, d.scan_scratch, st, launches);
+            scan_exclusive(d.pair_cnt, d.pair_off, d.N, d.scan_scratch, st, launches);
             launch_pdl(k_pair_write, dim3(pair_write_blocks(d.N)), dim3(CT), 0, st, d);
             *launches += 4;
         }

@@ -340,7 +340,7 @@ void launch_lbvh_pairs(const Dev& d, cudaStream_t st, long long* launches) {
     int* ca_ = d.rx_cnt;
     int* cb = d.rx_cnt2;
     for (int shift = 0; shift < 32; shift += 8) {
-        scan_exclusive(ca_, d.rx_off, nullptr, 256 * ntile, d.scan_scratch, st, launches);
+        scan_exclusive(ca_, d.rx_off, 256 * ntile, d.scan_scratch, st, launches);
         launch_pdl(k_rx_scatter, dim3(ntile), dim3(RX_TILE), 0, st, ka, ia, kb, ib, n, shift, ntile, d.rx_off, ca_,
                    shift < 24 ? cb : (int*)nullptr);
         unsigned* tk = ka; ka = kb; kb = tk;
@@ -351,7 +351,7 @@ void launch_lbvh_pairs(const Dev& d, cudaStream_t st, long long* launches) {
     launch_pdl(k_bvh_build, dim3(bblk(n - 1)), dim3(BT), 0, st, d);
     launch_pdl(k_bvh_refit, dim3(bblk(n)), dim3(BT), 0, st, d);
     launch_pdl(k_bvh_pair_count, dim3((n + 63) / 64 > 0 ? (n + 63) / 64 : 1), dim3(64), 0, st, d);
-    scan_exclusive(d.pair_cnt, d.pair_off, nullptr, n, d.scan_scratch, st, launches);
+    scan_exclusive(d.pair_cnt, d.pair_off, n, d.scan_scratch, st, launches);
     launch_pdl(k_bvh_pair_write, dim3(bblk(n)), dim3(BT), 0, st, d);
     *launches += 9;
     launch_pair_sort(d, st, launches);

@@ -1,8 +1,7 @@
-// Exclusive prefix sums of int arrays whose length lives in device memory, so that the
-// launches can be captured once in a CUDA graph and replayed while the lengths change.
+// Exclusive prefix sums of int arrays.
 // Chunks of 4096 values (1024 threads x 4) are scanned per block; block totals go to a
 // scratch array that one block scans; a third pass adds the block offsets.  Arrays of one
-// chunk take one block, arrays of up to a few hundred thousand values one cluster of blocks.
+// chunk take one block, arrays of up to 131 072 values one cluster of blocks.
 #include "pabd_internal.h"
 
 namespace pabd {
@@ -39,11 +38,9 @@ __device__ __forceinline__ int block_incl_scan(int v, int* smem, int* total) {
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_chunks(const int* __restrict__ in, int* __restrict__ out,
-                                                              const int* n_dev, int n_cap, int* block_sums,
-                                                              int single) {
+                                                              int n, int* block_sums, int single) {
     pdl_enter();
     __shared__ int smem[32];
-    const int n = n_dev ? min(*n_dev, n_cap) : n_cap;
     const int base = blockIdx.x * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
     int v[SCAN_ITEMS];
     int s = 0;
@@ -66,11 +63,9 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_chunks(const int* __restr
     }
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_totals(int* block_sums, int nb, int* out, const int* n_dev,
-                                                              int n_cap) {
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_totals(int* block_sums, int nb, int* out, int n) {
     pdl_enter();
     __shared__ int smem[32];
-    const int n = n_dev ? min(*n_dev, n_cap) : n_cap;
     const int base = threadIdx.x * SCAN_ITEMS;
     int v[SCAN_ITEMS];
     int s = 0;
@@ -90,10 +85,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_totals(int* block_sums, i
     if (threadIdx.x == 0) out[n] = total;
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_add(int* out, const int* n_dev, int n_cap,
-                                                           const int* block_sums) {
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_add(int* out, int n, const int* block_sums) {
     pdl_enter();
-    const int n = n_dev ? min(*n_dev, n_cap) : n_cap;
     if (blockIdx.x == 0) return;
     const int add = block_sums[blockIdx.x];
     const int base = blockIdx.x * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
@@ -112,13 +105,10 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_add(int* out, const int* 
 constexpr int SCAN_BLOCKS = 8;
 constexpr int CL_ITEMS = 8;
 constexpr int CL_CHUNK = SCAN_THREADS * CL_ITEMS;
-// Two passes cost what the three launches do (262 144 values take four: 2 us more); an array
-// whose length is on the device is sized for far more values than it holds.
+// Two passes cost what the three launches do (262 144 values take four: 2 us more).
 constexpr int SCAN_CLUSTER_MAX = 2 * SCAN_BLOCKS * CL_CHUNK;
-constexpr int SCAN_CLUSTER_MAX_CAP = 4 * SCAN_BLOCKS * CL_CHUNK;
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_cluster(const int* __restrict__ in, int* __restrict__ out,
-                                                               const int* n_dev, int n_cap) {
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_cluster(const int* __restrict__ in, int* __restrict__ out, int n) {
     __shared__ int smem[32];
     __shared__ int totals[2][SCAN_BLOCKS];
     unsigned rank;
@@ -127,7 +117,6 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_cluster(const int* __rest
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     pdl_enter();
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    const int n = n_dev ? min(*n_dev, n_cap) : n_cap;
     int carry = 0;
     // (every block takes every pass, whether its run holds values or not: the barriers match)
     for (int c0 = 0, pass = 0; c0 < n; c0 += SCAN_BLOCKS * CL_CHUNK, ++pass) {
@@ -187,7 +176,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_cluster(const int* __rest
     if (rank == 0 && threadIdx.x == 0) out[n] = carry;
 }
 
-static void launch_scan_cluster(const int* in, int* out, const int* n_dev, int n_cap, cudaStream_t st) {
+static void launch_scan_cluster(const int* in, int* out, int n, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(SCAN_BLOCKS);
     cfg.blockDim = dim3(SCAN_THREADS);
@@ -201,28 +190,27 @@ static void launch_scan_cluster(const int* in, int* out, const int* n_dev, int n
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaLaunchKernelEx(&cfg, k_scan_cluster, in, out, n_dev, n_cap);
+    cudaLaunchKernelEx(&cfg, k_scan_cluster, in, out, n);
 }
 
-int scan_scratch_ints(int n_cap) { return (n_cap + SCAN_CHUNK - 1) / SCAN_CHUNK + 1; }
+int scan_scratch_ints(int n) { return (n + SCAN_CHUNK - 1) / SCAN_CHUNK + 1; }
 
-void scan_exclusive(const int* in, int* out, const int* n_dev, int n_cap, int* scratch, cudaStream_t st,
-                    long long* launches) {
-    const int nb = n_cap > 0 ? (n_cap + SCAN_CHUNK - 1) / SCAN_CHUNK : 1;
+void scan_exclusive(const int* in, int* out, int n, int* scratch, cudaStream_t st, long long* launches) {
+    const int nb = n > 0 ? (n + SCAN_CHUNK - 1) / SCAN_CHUNK : 1;
     if (nb == 1) {
-        launch_pdl(k_scan_chunks, dim3(1), dim3(SCAN_THREADS), 0, st, in, out, n_dev, n_cap, scratch, 1);
+        launch_pdl(k_scan_chunks, dim3(1), dim3(SCAN_THREADS), 0, st, in, out, n, scratch, 1);
         *launches += 1;
         return;
     }
-    if (n_cap <= (n_dev ? SCAN_CLUSTER_MAX_CAP : SCAN_CLUSTER_MAX)) {
-        launch_scan_cluster(in, out, n_dev, n_cap, st);
+    if (n <= SCAN_CLUSTER_MAX) {
+        launch_scan_cluster(in, out, n, st);
         *launches += 1;
         return;
     }
-    // the level-2 scan handles up to SCAN_CHUNK block totals (n_cap <= 16.7 M)
-    launch_pdl(k_scan_chunks, dim3(nb), dim3(SCAN_THREADS), 0, st, in, out, n_dev, n_cap, scratch, 0);
-    launch_pdl(k_scan_totals, dim3(1), dim3(SCAN_THREADS), 0, st, scratch, nb, out, n_dev, n_cap);
-    launch_pdl(k_scan_add, dim3(nb), dim3(SCAN_THREADS), 0, st, out, n_dev, n_cap, scratch);
+    // the level-2 scan handles up to SCAN_CHUNK block totals (n <= 16.7 M)
+    launch_pdl(k_scan_chunks, dim3(nb), dim3(SCAN_THREADS), 0, st, in, out, n, scratch, 0);
+    launch_pdl(k_scan_totals, dim3(1), dim3(SCAN_THREADS), 0, st, scratch, nb, out, n);
+    launch_pdl(k_scan_add, dim3(nb), dim3(SCAN_THREADS), 0, st, out, n, scratch);
     *launches += 3;
 }
 

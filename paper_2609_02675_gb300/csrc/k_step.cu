@@ -291,7 +291,7 @@ void launch_step_reset(const Dev& d, cudaStream_t st, long long* launches) {
 void launch_csr(const Dev& d, cudaStream_t st, long long* launches) {
     with_want(d.csr_want, [&](auto w) {
         constexpr int WANT = decltype(w)::value;
-        scan_exclusive(d.end_cnt, d.end_off, nullptr, d.N, d.scan_scratch, st, launches);
+        scan_exclusive(d.end_cnt, d.end_off, d.N, d.scan_scratch, st, launches);
         launch_pdl(k_csr_fill, dim3(stride_grid(d.cap_bonds, ST_T)), dim3(ST_T), 0, st, d);
         launch_pdl(k_csr_sort<WANT>, dim3(nblk(d.N * CSR_LANES)), dim3(ST_T), 0, st, d);
         *launches += 2;

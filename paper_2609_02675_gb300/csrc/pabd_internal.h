@@ -59,7 +59,7 @@ struct Params {
 };
 
 // A body with more than HEAVY_ENDS bond ends (a large body under a pile or a bed of grains)
-// is gathered and solved by a whole block of HEAVY_T threads instead of L lanes (the last
+// is gathered and solved by a whole block of HEAVY_T threads instead of L lanes (the first
 // HEAVY_BLOCKS blocks of every sweep launch take the heavy bodies), and its CSR slice is
 // sorted by a block.
 constexpr int HEAVY_ENDS = 64;
@@ -253,11 +253,9 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 // ---- launchers (all asynchronous on `st`) ----
-// scan: out[0..n] exclusive prefix sums of in[0..n-1], n read from *n_dev (or n_cap if
-// n_dev is null), out[n] = total; grid sized for n_cap.
-void scan_exclusive(const int* in, int* out, const int* n_dev, int n_cap, int* scratch, cudaStream_t st,
-                    long long* launches);
-int scan_scratch_ints(int n_cap);
+// scan: out[0..n] exclusive prefix sums of in[0..n-1], out[n] = total
+void scan_exclusive(const int* in, int* out, int n, int* scratch, cudaStream_t st, long long* launches);
+int scan_scratch_ints(int n);
 
 // zeroes the step's counters and accumulation scratch and sets the drives' anchors; precedes
 // launch_collision / launch_csr

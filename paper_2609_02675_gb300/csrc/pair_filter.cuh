@@ -1,6 +1,8 @@
-// The pair filter shared by the broad phases (grid hash in k_collision.cu, LBVH in
-// k_lbvh.cu): partner j of body i is accepted when it shares i's group, the two are not both
-// pinned, their inflated boxes overlap and no user bond joins them (reading R21).
+// The pair filter of the broad phases (grid hash in k_collision.cu, LBVH in k_lbvh.cu, small
+// front in k_front.cu): partner j of body i is accepted when it shares i's group, the two are not
+// both pinned, their inflated boxes overlap and no user bond joins them (reading R21).  pair_ok
+// reads all of j's part; where a broad phase has some of it in hand -- a bucket's record, a tree
+// node's box, boxes in shared memory -- it makes the same tests from that.
 #pragma once
 #include "pabd_internal.h"
 
@@ -34,10 +36,6 @@ __device__ __forceinline__ bool pair_ok(const Dev& d, int i, int j, int gi, int 
     if (!overlap(li, hi, lj, hj)) return false;
     if (adj_has(d, i, j)) return false;
     return true;
-}
-
-__device__ __forceinline__ bool pair_ok(const Dev& d, int i, int j, int gi, int fi) {
-    return pair_ok(d, i, j, gi, fi, d.lo[i], d.hi[i]);
 }
 
 }  // namespace pabd

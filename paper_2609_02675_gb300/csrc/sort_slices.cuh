@@ -10,7 +10,7 @@
 namespace pabd {
 
 constexpr int LONG_T = 1024;
-constexpr int LONG_SMEM = 4096;  // ints of dynamic shared memory (16 KB: several blocks per SM, no carve-out change)
+constexpr int LONG_SMEM = 4096;  // keys of a sorted run, words of a bitmap (launches that may rank take two arrays of them, 32 KB)
 
 // 64 keys held two per lane (key k in lane k / 2, slot k % 2) sorted ascending by the 32
 // lanes of a warp: a bitonic network of shuffles
