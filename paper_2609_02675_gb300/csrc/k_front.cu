@@ -14,7 +14,8 @@
 // chained bodies 18.5 us (42.4), 40 of them 23.9 (42.3), a pile of 30 boxes 33.6 (52.5), of 128
 // 44.8 (54.7), a slab under 121 boxes 45.1 (73.1); without body contacts, 19 bodies 18.3 (22.5)
 // but 121 bodies 20.2 (18.5).  Spread over a cluster, with global memory between the stages, it
-// took longer than the kernels from 250 bodies on.
+// took longer than the kernels from 250 bodies on.  (Not for a state with many contacts, see
+// choose_front in pabd_capi.cu.)
 #include "contacts.cuh"
 #include "csr.cuh"
 #include "predict.cuh"

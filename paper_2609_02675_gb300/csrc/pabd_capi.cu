@@ -165,6 +165,7 @@ struct pabd_scene {
     int threads = 8;  // threads per body of the sweep launches (sweep_threads)
     BinsShape bins;   // mode 2: all sweeps in one launch where in_bins (choose_bins)
     bool in_bins = false;
+    bool front = false;  // the step starts with the one-launch front (choose_front)
     // the default path's autotuner: whether it chose the mode and light order, and the mean
     // sweep time it measured for each candidate (mode 2 ordered, mode 2 in body order, mode 1
     // ordered, mode 1 in body order), nanoseconds
@@ -263,7 +264,7 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
         if (ev) cudaEventRecordWithFlags(ev[e++], s->st, cudaEventRecordExternal);
     };
     mark();
-    if (front_fits(d.N, d.p.body_contacts)) {
+    if (s->front) {
         // small scene: everything up to the sweeps in one launch (its stages are then all in the
         // profiling graph's first)
         launch_front(d, s->st, launches);
@@ -372,6 +373,26 @@ void enqueue_step(pabd_scene* s, long long* launches, const cudaEvent_t* ev = nu
     mark();
 }
 
+// Whether a small scene's step starts with the one-launch front (k_front.cu), by the contacts of its
+// current state, whose manifolds are one SM's work there.  Steps with the front and with the kernels
+// it replaces, us: 252 contacts (27 packed boxes) 96 and 105, 636 (a wall of 60) 106 and 111, 1120
+// (a layer of 100) 117 and 114, 1512 (a wall of 120) 142 and 122; 100 boxes that all overlap many
+// others, 8672 contacts, 320 and 94.
+constexpr int FRONT_CONTACTS = 1024;
+pabd_status choose_front(pabd_scene* s) {
+    const Dev& d = s->d;
+    s->front = front_fits(d.N, d.p.body_contacts);
+    if (!s->front || !d.p.body_contacts) return PABD_OK;
+    long long lc = 0;
+    launch_step_reset(d, s->st, &lc);
+    launch_collision(d, s->st, &lc);
+    int n = 0;
+    CK(cudaMemcpyAsync(&n, d.ctr + C_NCONTACTS, sizeof(int), cudaMemcpyDeviceToHost, s->st));
+    CK(cudaStreamSynchronize(s->st));
+    s->front = n <= FRONT_CONTACTS;
+    return PABD_OK;
+}
+
 // Where a tuner's trial sweeps leave the bodies' squared updates: the scene's own (Dev::resid_body)
 // are part of its state, a held group's residual being that of its last step.  (Dev::qstar is
 // written anew by every step's predictor, and no sweep reads it.)
@@ -426,11 +447,6 @@ pabd_status autotune_sweep(pabd_scene* s) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (best >= 1e30f) { s->fused = 0; s->mode = 1; }
-    // leave the counters as a fresh scene has them
-    CK(cudaMemsetAsync(d.ctr, 0, sizeof(int) * C_COUNT, s->st));
-    int nb0 = d.Nc;
-    CK(cudaMemcpyAsync(d.ctr + C_NBONDS, &nb0, sizeof(int), cudaMemcpyHostToDevice, s->st));
-    CK(cudaStreamSynchronize(s->st));
     return PABD_OK;
 }
 
@@ -960,6 +976,8 @@ pabd_status finalize_scene(pabd_scene* s) {
         s->mode = 2;
         CK(cudaStreamCreateWithFlags(&s->body_st, cudaStreamNonBlocking));
     }
+    const pabd_status fr = choose_front(s);
+    if (fr != PABD_OK) return fr;
     s->fused = (s->mode == 3) && N > 0;
     if (s->fused) {
         int coop = 0, dev = 0;
@@ -974,11 +992,11 @@ pabd_status finalize_scene(pabd_scene* s) {
     } else if ((ds.sweep_mode == 0 || ds.light_order == 0) && p.resid_tol <= 0) {
         pabd_status tr = autotune_default(s);
         if (tr != PABD_OK) return tr;
-        // leave the counters as a fresh scene has them
-        CK(cudaMemsetAsync(d.ctr, 0, sizeof(int) * C_COUNT, st));
-        CK(cudaMemcpyAsync(d.ctr + C_NBONDS, &nb0, sizeof(int), cudaMemcpyHostToDevice, st));
-        CK(cudaStreamSynchronize(st));
     }
+    // leave the counters as a fresh scene has them
+    CK(cudaMemsetAsync(d.ctr, 0, sizeof(int) * C_COUNT, st));
+    CK(cudaMemcpyAsync(d.ctr + C_NBONDS, &nb0, sizeof(int), cudaMemcpyHostToDevice, st));
+    CK(cudaStreamSynchronize(st));
     // the state the first step's warm start reads (the trial sweeps above may have written it)
     if (d.Nal) {
         CK(up((d.p.n_iter & 1) ? d.al_st1 : d.al_st0, s->al_init.data(), sizeof(float2) * Nc));
@@ -1253,11 +1271,13 @@ pabd_status pabd_tune(pabd_scene* s) {
     r = poll_status(s);
     if (r != PABD_OK) return r;
     const int mode0 = s->mode, sorted0 = s->d.light_sorted, threads0 = s->threads;
-    const bool bins0 = s->in_bins;
+    const bool bins0 = s->in_bins, front0 = s->front;
     r = autotune_default(s);
+    if (r == PABD_OK) r = choose_front(s);
     if (r != PABD_OK) return r;
     CK(cudaStreamSynchronize(s->st));
-    if (s->mode == mode0 && s->d.light_sorted == sorted0 && s->threads == threads0 && s->in_bins == bins0) return PABD_OK;
+    if (s->mode == mode0 && s->d.light_sorted == sorted0 && s->threads == threads0 && s->in_bins == bins0 && s->front == front0)
+        return PABD_OK;
     // the step graphs were captured with the old shape: capture them again
     cudaGraphExecDestroy(s->exec);
     cudaGraphDestroy(s->graph);
