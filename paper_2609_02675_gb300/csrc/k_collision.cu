@@ -83,10 +83,11 @@ __global__ void k_cells(Dev d) {
 }
 
 // Bodies into their buckets, with a copy of what the pair test reads -- the box, the group, the id,
-// level and pinned flag -- in one 32-byte record (Dev::brec): the candidates lie anywhere, and a
-// sector of the L2 each is what the pair search costs.  (The cell, too, made it three sectors; that
-// no partner is met twice is the scan's business, which takes each bucket once.  262 144 boxes:
-// pairs counted in 164 us, now 132; a quadruped on 50 000 grains 77, now 62.)
+// level and pinned flag -- in one 32-byte record (Dev::brec): the candidates lie anywhere, and
+// waiting for them is most of what the pair search costs (262 144 boxes: 9 of 20 cycles per issued
+// instruction at 42 warps per SM, L1 68 % busy).  (The cell, too, made it three sectors; that no
+// partner is met twice is the scan's business, which takes each bucket once.  262 144 boxes: pairs
+// counted in 164 us, now 132; a quadruped on 50 000 grains 77, now 62.)
 constexpr int REC_ID_BITS = 28;  // (a body takes kilobytes of device memory: more do not fit)
 __device__ __forceinline__ int rec_id(float w) { return __float_as_int(w) & ((1 << REC_ID_BITS) - 1); }
 __device__ __forceinline__ int rec_level(float w) { return (__float_as_int(w) >> REC_ID_BITS) & 7; }
@@ -490,8 +491,10 @@ __device__ __noinline__ int tile_contacts(const Dev& d, int tile, int np) {
 // slot.  The bodies' bond ends are counted on the way, on top of their static ones.
 //
 // It replaced a counting pass, two prefix sums, a pass that derived every manifold again to write
-// it, and the count of bond ends.  Bound by the clipping's dependent steps and their trips to
-// shared memory (16 warps per SM, its 46 KB a block): 532 325 pairs of a settled bed 115 us
+// it, and the count of bond ends.  Bound by latency at 16 warps per SM (its 46 KB a block): the
+// block's barriers, where a tile waits for its longest item and for the look-back (5.0 of 13 cycles
+// per issued instruction on a pile), then the boxes' loads (3.7), the clipping's dependent steps
+// and divergence (half the lanes idle on a settled bed).  532 325 pairs of a settled bed 115 us
 // (counting 156 and writing 187 us; in one pass with the polygons in local memory 274), 258 048
 // pairs of a pile, all touching, 78 us (57 and 90).
 __global__ void __launch_bounds__(NARROW_T) k_narrow(const __grid_constant__ Dev d) {

@@ -13,8 +13,9 @@
 // k_sweep_one, so the results are the same bit for bit.
 //
 // What bounds it: instruction issue of one warp per scheduler along the dependent chain of a
-// body's sum, factorisation and rotation (8 chained bodies: 2200 instructions a sweep, 3.3 cycles
-// each, of which 1.35 wait for instruction fetch and 1.1 for the previous result).  Per sweep,
+// body's sum, factorisation and rotation (8 chained bodies: 2160 instructions a sweep, 2.7 cycles
+// each, of which 0.65 wait for the previous result and 0.57 for instruction fetch; a 121-body net
+// 4.7, with the cluster's barrier and its stores 1.1).  Per sweep,
 // against one launch per sweep: 8 chained bodies 3.0 us (5.4), 121-body spring net 3.7 (4.9),
 // 250-box pile 3.8 (4.5).
 #include "sweep_shape.h"
