@@ -227,8 +227,9 @@ pabd_status pabd_step(pabd_scene* s, int nsteps);
 pabd_status pabd_step_eager(pabd_scene* s, int nsteps);
 
 /* Re-run the sweep autotuner of a scene created with sweep_mode 0 on its current state (for
- * instance once a pile has landed, when its contacts are in place) and re-capture its step
- * graph if the choice changed.  Synchronises the scene's stream.  The trial sweeps change no
+ * instance once a pile has landed, when its contacts are in place), choose anew whether a small
+ * scene's step starts with one launch (not where it has many contacts) and re-capture its step
+ * graph if a choice changed.  Synchronises the scene's stream.  The trial sweeps change no
  * state; the pair and contact lists afterwards are those of the current state.  Returns
  * PABD_OK without tuning for scenes whose shape is fixed (sweep_mode 1-3, resid_tol > 0,
  * AL_DISTANCE bonds); a latched device error is returned first. */
