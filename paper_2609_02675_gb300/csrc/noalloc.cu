@@ -27,8 +27,7 @@ constexpr size_t OFF_LARGE = OFF_POFF + al(sizeof(int) * (NA_MAX + 1));
 constexpr size_t OFF_CTR = OFF_LARGE + al(sizeof(int) * NA_MAX);
 constexpr size_t OFF_REC = OFF_CTR + al(sizeof(int) * C_COUNT);
 constexpr size_t OFF_LIST = OFF_REC + al(2 * sizeof(float4) * NA_MAX);
-constexpr size_t OFF_REST = OFF_LIST + al(sizeof(int) * PAIR_LIST * NA_MAX);
-constexpr size_t OFF_SCAN = OFF_REST + al(sizeof(int) * NA_MAX);
+constexpr size_t OFF_SCAN = OFF_LIST + al(sizeof(int) * PAIR_LIST * NA_MAX);
 constexpr size_t SCAN_INTS = NA_TABLE / 4096 + 2;  // block totals of the largest scan
 constexpr size_t NA_BYTES = OFF_SCAN + al(sizeof(int) * SCAN_INTS);
 
@@ -129,7 +128,7 @@ extern "C" pabd_status pabd_broadphase_noalloc(const float* q, const float* vel,
     d.large_ids = (int*)(base + OFF_LARGE);
     d.brec = (float4*)(base + OFF_REC);
     d.pair_list = (int*)(base + OFF_LIST);
-    d.pair_rest = (int*)(base + OFF_REST);
+    d.pair_rest = d.bucket_cur;
     d.scan_scratch = (int*)(base + OFF_SCAN);
     d.pairs = (int2*)pairs_out;
     long long launches = 0;

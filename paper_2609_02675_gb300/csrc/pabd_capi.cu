@@ -837,6 +837,7 @@ pabd_status finalize_scene(pabd_scene* s) {
     ok &= alloc_arr(s, d.gbar, 2) && alloc_arr(s, d.wait_limit, 1);
     ok &= alloc_arr(s, d.lo, N) && alloc_arr(s, d.hi, N) && alloc_arr(s, d.cell, N);
     ok &= alloc_arr(s, d.bucket_cnt, T) && alloc_arr(s, d.bucket_cur, T) && alloc_arr(s, d.bucket_off, T + 1);
+    d.pair_rest = d.bucket_cur;
     ok &= alloc_arr(s, d.pair_cnt, N) && alloc_arr(s, d.pair_off, N + 1) && alloc_arr(s, d.pairs, d.cap_pairs);
     ok &= alloc_arr(s, d.brec, 2 * (size_t)N);
     if (ds.body_contacts && p.broadphase == 0) {
@@ -844,7 +845,7 @@ pabd_status finalize_scene(pabd_scene* s) {
             ok &= alloc_arr(s, d.lane_cnt, (size_t)32 * N) && alloc_arr(s, d.pair_stash, (size_t)32 * PAIR_STASH * N) &&
                   alloc_arr(s, d.lane_tot, (size_t)32 * N);
         else
-            ok &= alloc_arr(s, d.pair_list, (size_t)PAIR_LIST * N) && alloc_arr(s, d.pair_rest, N);
+            ok &= alloc_arr(s, d.pair_list, (size_t)PAIR_LIST * N);
     }
     if (front_fits(N, ds.body_contacts)) ok &= alloc_arr(s, d.npc, d.cap_pairs) && alloc_arr(s, d.npc_off, d.cap_pairs + 1);
     if (ds.body_contacts) ok &= alloc_arr(s, d.tile_state, ((size_t)d.cap_pairs + N) / NARROW_T + 1);

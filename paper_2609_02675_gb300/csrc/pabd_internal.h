@@ -145,7 +145,8 @@ struct Dev {
     int *bucket_cnt, *bucket_cur, *bucket_off;
     float4 *brec;               // per bucket slot: (lo, id, level and pinned bits), (hi, group bits)
     int *pair_list;             // per body: its partners in order, if at most PAIR_LIST (k_pair_count)
-    int *pair_rest;             // the bodies that have partners and no such list
+    int *pair_rest;             // the bodies that have partners and no such list (in bucket_cur, whose
+                                // work is done when the buckets are filled)
     int *lane_cnt;              // multilevel grid, per body x 32 lanes: partners found by each lane
     // multilevel grid, per body x 32 lanes: the first PAIR_STASH partners each lane found while counting (a
     // partner delivered to a smaller id tagged by STASH_DELIVER), and the lane's number of
